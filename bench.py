@@ -38,10 +38,7 @@ sys.path.insert(0, ROOT)
 # ncu measured for a kernel on this workload at full size, with the SHA-256
 # of the source file that kernel was built from: reported only while that
 # file is unchanged (the capture and its command are summarised in profiles/)
-NCU_TRAFFIC = {
-    "allpairs": ("paper_2502_14446_gb300/csrc/k_verify.cu",
-                 "a39b245a329753dd18d0acb758ba6c2e98e01237865e13a464ea6655e31809dd", 6614610),
-}
+NCU_TRAFFIC = {}
 
 
 def measured_traffic(kernel):
@@ -222,8 +219,8 @@ def roofline(kernel, k_ms, k_n, info, st, wl, steps, pk, sms=152):
                       the sliding cross product of the diagonal recurrence
                       (two FMA, 4 flop) and the Pearson threshold test on
                       per-window factors (one FMA, one multiply, one
-                      compare: 4); the kernels execute more (centring,
-                      column sums, three thresholds)
+                      compare: 4); the kernel tests with one FMA (3 in
+                      all), and runs groups with a passing dimension twice
       sort_*          20 bytes per index entry (window, dim, repetition):
                       its 8-byte key read, the sorted 12-byte (key, window)
                       written; every kernel of the index sort together

@@ -275,13 +275,8 @@ int momenti_search_finish(momenti_handle* h, momenti_motif* out, int32_t* n_out,
  * of Definition top-k), on the GPU, float64 re-verified.  Same outputs and
  * errors as momenti_topk.
  *
- * For a float32 series the all-pairs sweep has several forms that record
- * the same pairs; the first sweep of an index times them on a part of the
- * grid and keeps the fastest per (device, padded D, log2 w, log2 M) for the
- * process.  Environment: MOMENTI_AUTOTUNE=0 takes the default form,
- * MOMENTI_SWEEP_VARIANT=v (a digit) forces form v, MOMENTI_TRACE=1 prints
- * the choice, one line per traversal chunk and one per exact-path sweep to
- * stderr. */
+ * Environment: MOMENTI_TRACE=1 prints one line per traversal chunk and one
+ * per exact-path sweep to stderr. */
 int momenti_topk_exact(momenti_handle* h, momenti_motif* out, int32_t* n_out);
 
 /* Eq. zned per dimension and Definition distdims for m given pairs
@@ -458,11 +453,12 @@ uint64_t momenti_launch_count(void);
  * A name ending in '*' selects every kernel whose name starts with the part
  * before it (for example "sort_*": all kernels of the index sort).
  * Kernel names: split_f32, split_f64, point_major, window_stats,
- * stats_pm, col_prep, mean16, r_sample, draw, layout_hash, layout_boff,
+ * stats_pm, mean16, r_sample, draw, layout_hash, layout_boff,
  * proj_hash_fp32, proj_hash_tc, rehash, sort_init, sort_hist, sort_scan,
  * sort_scatter, sort_local, tensor_keys, chunk_agg, chunk_scan, scan_local, scan_top,
  * scan_add, collide, bucket_jobs, subbucket, subwarp, hs_clear,
- * verify_events, verify_pairs, allpairs, allpairs_batch, select_pairs. */
+ * verify_events, verify_pairs, sweep_table, allpairs, allpairs_sample,
+ * allpairs_batch, select_pairs. */
 int momenti_time_kernel(const char* name);
 
 /* Device time in milliseconds accumulated by the timed kernel since the

@@ -30,13 +30,8 @@ struct Index {
   float* xT = nullptr;        // [n][Dp] point-major copy of xs_hi (D <= 8), dims padded with 0
   float* xlT = nullptr;       // [n][Dp] point-major copy of xs_lo
   int Dp = 0;                 // 4, 8 or 16 when xT is present
-  float* xW = nullptr;        // [n][DW] point-major copy of xs_hi for 16 < D <= 64, float32 input
-  int DW = 0;                 // 32 or 64 when xW is present
   float* smT = nullptr;       // [n-15][Dp] means of 16 consecutive points (D <= 8, w >= 32)
   float* stT = nullptr;       // [M][3][Dp] point-major mu_hi, mu_lo, inv_sig (D <= 8)
-  float* isT = nullptr;       // [M][Dp] 1/sigma (padding dims 1), float32 input, D <= 16
-  float* isW = nullptr;       // [M][DW] 1/sigma (padding dims 1), with xW
-  uint8_t* cflag = nullptr;   // [M] column window not testable in float32 by the sweep
   double* mu = nullptr;       // [D][M]
   double* sig = nullptr;      // [D][M]
   float* mu_hi = nullptr;     // [D][M]  float(mu)
@@ -272,8 +267,6 @@ cudaError_t launch_verify_events(const Index& ix, int d, const HashSet& hs,
 cudaError_t launch_verify_pairs(const Index& ix, int d, const uint64_t* pairs, int64_t m,
                                 int fp64, double* per_dim, double* dist_d, uint64_t* dims,
                                 cudaStream_t s);
-// Exact all-pairs: every non-trivial pair with approximate dist_d <= tau
-// appended to out (a << 32 | b) with count in *count (may exceed cap).
 // Output of an all-pairs sweep: pairs whose approximate dist_d (float32
 // Pearson form, within 1% + 0.01 of the exact value) lies in (lo, thr]
 // go to out / out_d while count < cap; count counts them all and hist
@@ -288,46 +281,50 @@ struct ApRec {
   float lo = -1.f;
   float hscale = 0.f;          // kApBins / (thr - lo)
 };
-cudaError_t launch_allpairs(const Index& ix, int d, float thr, const ApRec& rc, cudaStream_t s);
-// Whether the row-staged sweep of wide series (16 < D <= 64) takes this index
-// (a point-major copy, and its staged rows fit a CTA's shared memory).
-bool rows2_usable(const Index& ix);
-// ---- k_wide64_*.cu: the 64-dimension sweeps, each instantiated in a
-// translation unit of its own (they dominate the build; units compile in
-// parallel).  gy_max cuts the grid to its first diagonal blocks.
-cudaError_t launch_rows4_64(const Index& ix, int d, float thr, const ApRec& rc, cudaStream_t s,
-                            int64_t gy_max);
-cudaError_t launch_rows2_64(const Index& ix, int d, float thr, const ApRec& rc, cudaStream_t s,
-                            int64_t gy_max);
-cudaError_t launch_rows2_64_rowmin(const Index& ix, int d, float* rowmin, cudaStream_t s);
-cudaError_t launch_wide64(const Index& ix, int d, float thr, const ApRec& rc, float* rowmin,
-                          bool rowmin_mode, cudaStream_t s);
 
-// One series' recording sweep inside a batched launch.
+// ---- k_sweep.cu ---------------------------------------------------------
+// The sweep's view of an index: its table (k_sweep.cu: df, dg and sigma per
+// window, in planes of transposed 64-window blocks), the series' points in the same
+// order, and the window means.
+struct SweepView {
+  const void* tab = nullptr;     // [Mpad / 64][3][64][G] vectors of 2 P dims
+  const void* xp = nullptr;      // [npad][G]
+  const void* xl = nullptr;      // [npad][G] low parts, float64 input only
+  const double* mu = nullptr;    // [D][M]
+  int64_t M = 0, Mpad = 0, npad = 0;
+  int D = 0, P = 0, G = 0;       // dims, pairs of dims per lane, lanes per diagonal
+  int w = 0, excl = 0;
+};
+// One series' recording sweep.
 struct SweepJob {
-  Index ix;
+  SweepView v;
   ApRec rc;
   float thr = 0.f;
   int d = 0;
+  int seg = 0;                   // rows per block (set by the launch)
+  // optional: += 8-row groups run by the warps, and those run twice
+  unsigned long long* groups = nullptr;
 };
 struct SweepItem {
-  uint32_t job, bx, by;     // series, row block (kSeg windows), diagonal block
+  uint32_t job, bx, by;          // series, row block, diagonal block
 };
-// Whether the sweep of this index can join a batched launch (float32
-// input, D <= 16, the statistics form).
-bool sweep_batchable(const Index& ix);
-// The recording sweeps of several series (each batchable) in one
-// persistent launch per padded dimension count, on stream s; every job's
-// record buffers must be ready on s.
-cudaError_t launch_allpairs_batch(const std::vector<SweepJob>& jobs, cudaStream_t s);
-// The column table of the statistics sweep (isT, cflag), after the window
-// statistics; nothing when the index has no isT.
-cudaError_t launch_col_prep(const Index& ix, cudaStream_t s);
+// Bytes of the table of an index, and the table built into buf (16-byte
+// aligned, that many bytes) on stream s; *out views it.
+size_t sweep_table_bytes(const Index& ix);
+cudaError_t launch_sweep_table(const Index& ix, void* buf, SweepView* out, cudaStream_t s);
+// The recording sweep over all pairs of one series.
+cudaError_t launch_allpairs(const SweepView& v, int d, float thr, const ApRec& rc, cudaStream_t s);
+// The same over a spread sample of about `fraction` of the grid's blocks
+// (of seg rows each); *pairs = the pairs it holds, groups[2] (zeroed by the
+// caller) the groups of rows run, and those that took the slow branch.
+cudaError_t launch_allpairs_sample(const SweepView& v, int d, float thr, const ApRec& rc, double fraction,
+                                   int seg, double* pairs, unsigned long long* groups, cudaStream_t s);
+// The recording sweeps of several series in one persistent launch on
+// stream s; every job's table and record buffers must be ready on s.
+cudaError_t launch_allpairs_batch(std::vector<SweepJob> jobs, cudaStream_t s);
+
+// ---- k_verify.cu, continued ---------------------------------------------
 // Recorded pairs whose approximate distance lies in (lo, hi], compacted.
 cudaError_t launch_select_pairs(const uint64_t* pairs, const float* dd, uint64_t m, float lo,
                                 float hi, uint64_t* out, unsigned long long* count, cudaStream_t s);
-// Row minima of dist_d over non-trivial partners (approximate), for the
-// first threshold of the all-pairs path; rowmin [M].
-cudaError_t launch_allpairs_rowmin(const Index& ix, int d, float* rowmin, cudaStream_t s);
-
 }  // namespace momenti

@@ -1,0 +1,966 @@
+// The recording sweep of the exact all-pairs path (the final fallback of
+// Algorithm 1): every non-trivial pair of windows whose approximate dist_d
+// lies in (lo, thr] is appended to a list, with a histogram of the
+// distances.  One form for every series (float32 and float64 input, 1 to
+// 64 dimensions).
+//
+// Recurrence.  Along a diagonal b = a + delta of the distance matrix the
+// centred cross product of two windows,
+//   C(a, b) = sum_t (x_{a+t} - mu_a) (x_{b+t} - mu_b),
+// satisfies exactly
+//   C(a, b) = C(a - 1, b - 1) + df_a dg_b + dg_a df_b,
+//   df_a = (x_{a+w-1} - x_{a-1}) / 2,
+//   dg_a = (x_{a+w-1} - mu_a) + (x_{a-1} - mu_{a-1})
+// (the mean-centred streaming update of the matrix-profile literature:
+// Zimmerman et al., "Matrix Profile XIV", SoCC 2019).  df, dg and sigma
+// are per-window values: they are computed once per search in float64 and
+// rounded (k_sweep_table), so a pair and dimension costs two FMA for the
+// recurrence and one for the threshold test, and nothing of the state
+// depends on the series' level: it is C itself, in float32, restarted
+// directly every `seg` rows.  Its error per step is one rounding of C and
+// of the two products; a form that slides products centred on a constant
+// carries those and the centring offset's on top.
+//
+// Test.  dist_f <= t  <=>  corr >= c(t) = 1 - t^2 / 2w  <=>
+// C >= c(t) w sigma_a sigma_b.  dist_d <= thr needs one dimension with
+// dist <= thr / d (the smallest of d values is at most their mean): one FMA
+// per dimension against a row factor, whose sign bits are combined over the
+// 8 rows x 8 diagonals a lane runs between two branches.  A group in which
+// one passed runs again with a test of all dimensions together (sw_redo).
+//
+// Layout.  A lane holds 2 P dimensions (P = 2, or 1: sw_pairs) of 8
+// neighbouring diagonals; G = ceil(D / 2P) lanes share a diagonal (32 / G
+// diagonal groups in a warp).  Per row a lane reads the row's record from
+// shared memory (one address per g: a broadcast) and one new column record,
+// which the 8 diagonals use in the next 8 rows: the 8 columns in flight
+// live in registers, indexed statically by unrolling 8 rows.  Both sides
+// then read 96 bytes per 32 pair-dimensions, a quarter of what one diagonal
+// per lane reads.  Neighbouring lanes' columns are 8 windows apart, which
+// in window order would put them on the same banks: the table stores blocks
+// of 64 windows transposed (8 x 8), so that they are consecutive.
+//
+// What bounds it (D = 8, w = 300, 5e9 pairs, edge below the background):
+// 7.3 ms, 5.5 pair-dimensions per cycle and scheduler of the 10.7 that three
+// FMA on the FP32 lanes allow; 8 warps per SM, fixed-latency dependencies
+// first.  The form before, one diagonal per lane sliding centred products,
+// took 35.6 ms; at D = 32, w = 500, n = 2e5, 145 against 848 ms.
+//
+// Windows that the float32 test cannot resolve (flat, or with a level
+// change of more than about 100 sigma within the last 256 windows) have
+// sigma = NaN in the table: their tests give NaN, whose sign bit is clear,
+// so they always reach the slow branch, which takes them as candidates.
+#include "internal.h"
+
+#include <algorithm>
+#include <cstdint>
+
+namespace momenti {
+
+namespace {
+
+constexpr int kSwThreads = 128;
+constexpr int kSwWarps = kSwThreads / 32;
+constexpr int kSwR = 8;                 // diagonals per lane
+constexpr int kSwPad = 2048;            // records after the last window / point
+constexpr int kSwFlagBack = 256;        // windows looked back at for the level-change mark
+
+// P pairs of dims: 2 P floats of one kind, loaded with one instruction.
+template <int P>
+struct __align__(8 * P) SwVec {
+  float2 v[P];
+};
+
+// CTAs per SM: what the registers of 8 diagonals x 2 P dims leave without
+// spilling in the loop (255 and 168 registers a thread).
+template <int P>
+constexpr int kSwBlocks = P == 2 ? 2 : 3;
+
+// Position of point b in its array: 8 x 8 transposed blocks.
+__host__ __device__ __forceinline__ int64_t sw_pos(int64_t b) {
+  return (b & ~int64_t(63)) + ((b & 7) << 3) + ((b >> 3) & 7);
+}
+// Offset of window b in the table, in units of G vectors: blocks of 64
+// windows with their df, dg and sigma planes (64 units each) one after
+// another, so that a warp's load of one kind touches whole cache lines (12
+// lines a load when the three lay together: L1 was the limit).
+__host__ __device__ __forceinline__ int64_t sw_off(int64_t b) {
+  return (b >> 6) * 192 + ((b & 7) << 3) + ((b >> 3) & 7);
+}
+
+// Pairs of dims per lane for a series of D dims.  Two pairs read half the
+// instructions per pair-dimension; one pair wastes at most one dimension
+// instead of three, which pays at D = 1, 2, 5, 6 (a sweep of n = 1e5, w =
+// 300 at D = 5: 5.8 ms against 6.6 with two).
+int sw_pairs(int D) { return D <= 2 || D == 5 || D == 6 ? 1 : 2; }
+int64_t sw_round(int64_t m) { return ((m + 63) & ~int64_t(63)) + 64 + kSwPad; }
+
+// Rows staged in shared memory at a time.
+template <int P>
+__host__ __device__ __forceinline__ int sw_rows(int G) { return G * P <= 8 ? 64 : (G * P <= 16 ? 32 : 16); }
+// A warp's queue of hits: 32 plus what one row can add (8 per group of
+// lanes); an entry holds C per dim, row and column in an odd number of
+// 16-byte units, so that lanes reading their own entries spread over the
+// banks.
+__host__ __device__ __forceinline__ int sw_queue(int G) { return 32 + kSwR * (32 / G); }
+template <int P>
+__host__ __device__ __forceinline__ int sw_entry(int G) { return 4 * (((G * 2 * P + 2 + 3) / 4) | 1); }
+template <int P>
+size_t sw_smem(int G) {
+  return size_t(2) * sw_rows<P>(G) * G * 3 * sizeof(SwVec<P>) +
+         size_t(kSwWarps) * (size_t(2) * kSwR * 32 * sizeof(SwVec<P>) + size_t(sw_queue(G)) * sw_entry<P>(G) * 4);
+}
+size_t sw_smem(const SweepView& v) { return v.P == 2 ? sw_smem<2>(v.G) : sw_smem<1>(v.G); }
+
+// Table of an index: per window and group of 4 dims {df x4, dg x4, sigma x4};
+// per point the 4 values (and their low parts for float64 input).  A block
+// builds 64 windows and points: first the marks (one warp per dim, the
+// level change bounded by the range of the means before the exact scan of
+// the 256 windows before it), then the records.
+template <int P>
+__global__ void __launch_bounds__(256) k_sweep_table(Index ix, SweepView v, SwVec<P>* __restrict__ tab,
+                                                     SwVec<P>* __restrict__ xp, SwVec<P>* __restrict__ xl) {
+  __shared__ int mark[64];
+  const int64_t B = int64_t(blockIdx.x) * 64;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int64_t M = ix.M, n = ix.n;
+  if (threadIdx.x < 64) mark[threadIdx.x] = 0;
+  __syncthreads();
+  if (B < M) {
+    const int64_t q0 = B > kSwFlagBack ? B - kSwFlagBack : 0, q1 = min(M, B + 64);
+    for (int f = warp; f < ix.D; f += 8) {
+      const float* mh = ix.mu_hi + int64_t(f) * M;
+      float lo = INFINITY, hi = -INFINITY;
+      for (int64_t q = q0 + lane; q < q1; q += 32) {
+        lo = fminf(lo, mh[q]);
+        hi = fmaxf(hi, mh[q]);
+      }
+      for (int o = 16; o > 0; o >>= 1) {
+        lo = fminf(lo, __shfl_xor_sync(0xffffffffu, lo, o));
+        hi = fmaxf(hi, __shfl_xor_sync(0xffffffffu, hi, o));
+      }
+      const double range = double(hi) - double(lo);
+      for (int64_t b = B + lane; b < q1; b += 32) {
+        const double sg = ix.sig[int64_t(f) * M + b], var = sg * sg;
+        bool bad = ix.inv_sig[int64_t(f) * M + b] == 0.f;
+        if (!bad && !(var > 1e-4 * (var + range * range))) {
+          const float mb = mh[b];
+          float dmax = 0.f;
+          for (int64_t q = b > kSwFlagBack ? b - kSwFlagBack : 0; q <= b; ++q)
+            dmax = fmaxf(dmax, fabsf(mh[q] - mb));
+          const double dm = double(dmax);
+          bad = !(var > 1e-4 * (var + dm * dm));
+        }
+        if (bad) atomicOr(&mark[int(b - B)], 1);
+      }
+    }
+  }
+  __syncthreads();
+  const int G = v.G;
+  for (int q = threadIdx.x; q < 64 * G; q += 256) {
+    const int c = q & 63, g = q >> 6;
+    const int64_t b = B + c;
+    const bool in = b < M;
+    SwVec<P> df, dg, sg, xh, xlo;
+#pragma unroll
+    for (int e = 0; e < 2 * P; ++e) {
+      const int f = 2 * P * g + e;
+      float vdf = 0.f, vdg = 0.f, vx = 0.f, vl = 0.f;
+      // past the last window: a sigma no correlation reaches; no such dim: 0
+      float vs = f < ix.D ? 1e30f : 0.f;
+      if (f < ix.D) {
+        const float* h = ix.xs_hi + int64_t(f) * n;
+        const float* l = ix.has_lo ? ix.xs_lo + int64_t(f) * n : nullptr;
+        auto X = [&](int64_t t) { return double(h[t]) + (l ? double(l[t]) : 0.0); };
+        if (in) {
+          if (b > 0) {
+            const double xi = X(b + ix.w - 1), xo = X(b - 1);
+            vdf = float(0.5 * (xi - xo));
+            vdg = float((xi - ix.mu[int64_t(f) * M + b]) + (xo - ix.mu[int64_t(f) * M + b - 1]));
+          }
+          vs = mark[c] ? __int_as_float(0x7fc00000) : float(ix.sig[int64_t(f) * M + b]);
+        }
+        if (b < n) {
+          vx = h[b];
+          if (l) vl = l[b];
+        }
+      }
+      float2* o[5] = {&df.v[e / 2], &dg.v[e / 2], &sg.v[e / 2], &xh.v[e / 2], &xlo.v[e / 2]};
+      const float val[5] = {vdf, vdg, vs, vx, vl};
+#pragma unroll
+      for (int k = 0; k < 5; ++k) {
+        if (e & 1) o[k]->y = val[k];
+        else o[k]->x = val[k];
+      }
+    }
+    const int64_t p = sw_pos(b) * G + g;
+    if (b < v.Mpad) {
+      SwVec<P>* t = tab + sw_off(b) * G + g;
+      t[0] = df;
+      t[64 * G] = dg;
+      t[128 * G] = sg;
+    }
+    if (b < v.npad) {
+      xp[p] = xh;
+      if (xl) xl[p] = xlo;
+    }
+  }
+}
+
+// A pair whose approximate dist_d lies in (rc.lo, thr]: appended (with its
+// approximate distance) while there is room, and counted in the histogram
+// of (rc.lo, thr] either way.
+__device__ __forceinline__ void sw_record(const ApRec& rc, uint32_t a, uint32_t b, float dd) {
+  // one counter atomic per group of converged lanes
+  const unsigned act = __activemask();
+  const int lane = threadIdx.x & 31, leader = __ffs(act) - 1;
+  unsigned long long base = 0;
+  if (lane == leader) base = atomicAdd(rc.count, (unsigned long long)__popc(act));
+  base = __shfl_sync(act, base, leader);
+  const unsigned long long pos = base + __popc(act & ((1u << lane) - 1u));
+  if (pos < rc.cap) {
+    rc.out[pos] = (uint64_t(a) << 32) | uint64_t(b);
+    rc.out_d[pos] = dd;
+  }
+  if (rc.hist) {
+    const float x = (dd - rc.lo) * rc.hscale;
+    const int bin = x < float(kApBins - 1) ? int(fmaxf(x, 0.f)) : kApBins - 1;
+    atomicAdd(&rc.hist[bin], 1u);
+  }
+}
+
+// Sorts N registers (a power of two) descending: bitonic network.
+template <int N>
+__device__ __forceinline__ void sort_desc(float (&c)[N]) {
+#pragma unroll
+  for (int k = 2; k <= N; k <<= 1)
+#pragma unroll
+    for (int j = k >> 1; j > 0; j >>= 1)
+#pragma unroll
+      for (int i = 0; i < N; ++i) {
+        const int l = i ^ j;
+        if (l > i) {
+          const float hi = fmaxf(c[i], c[l]), lo = fminf(c[i], c[l]);
+          c[i] = (i & k) ? lo : hi;
+          c[l] = (i & k) ? hi : lo;
+        }
+      }
+}
+
+// dist_d of one hit from its correlations (less yl): the sum of the
+// distances of the d largest.  N >= D values in registers.
+template <int N>
+__device__ __forceinline__ float sw_dist(const float* e, int D, int d, float yl, float wf) {
+  float c[N];
+#pragma unroll
+  for (int f = 0; f < N; ++f) c[f] = f < D ? e[f] + yl : -INFINITY;
+  sort_desc<N>(c);
+  float sm = 0.f;
+#pragma unroll
+  for (int f = 0; f < N; ++f)
+    if (f < d) sm += sqrtf(fmaxf(2.f * wf * (1.f - c[f]), 0.f));
+  return sm;
+}
+
+// The joint test.  With lambda = q thr / d, dist_d <= thr gives
+//   sum over the d best dims of (lambda - x_f) >= d lambda - thr,
+// and lambda - x_f, as a function of the correlation y_f = 1 - x_f^2 / 2w,
+// is convex above y_l = 1 - lambda^2 / 2w, where it is 0, so below its chord
+// to (1, lambda).  Hence
+//   sum over all dims of max(0, y_f - y_l) >= (d - d / q) (1 - y_l).
+// At q = 1.5 this passes a tenth of the pairs that have one dimension
+// within thr / d on the sensor workload (0.3 % against 3.3 %); for d = 1,
+// where the one-dimension test is the exact one, q is near 1.
+struct SwJoint {
+  float yl, need;
+};
+__device__ __forceinline__ SwJoint sw_joint(const SweepJob* jb) {
+  const float q = jb->d > 1 ? 1.5f : 1.02f;
+  const float lam = q * jb->thr / float(jb->d);
+  SwJoint j;
+  j.yl = 1.f - lam * lam / (2.f * float(jb->v.w));
+  j.need = (float(jb->d) * (1.f - 1.f / q) - 1e-3f) * (1.f - j.yl);
+  return j;
+}
+
+// The queued hits of a warp, the last 32 at a time (all of them when
+// `all`), one per lane: pairs that exist and are not trivial get their
+// distance; pairs with an unresolvable window (NaN) distance 0.  Returns
+// the number left.
+template <int P>
+__device__ __noinline__ int sw_drain(const SweepJob* jb, float* queue, int qn, bool all) {
+  const SweepView& v = jb->v;
+  const int lane = threadIdx.x & 31;
+  const int D = v.D, d = jb->d, QS = sw_entry<P>(v.G);
+  const float thr = jb->thr, wf = float(v.w), yl = sw_joint(jb).yl;
+  __syncwarp();
+  while (qn >= 32 || (all && qn > 0)) {
+    const int n = min(32, qn);
+    qn -= n;
+    if (lane < n) {
+      float* e = queue + (qn + lane) * QS;
+      const uint32_t a = __float_as_uint(e[QS - 2]), b = __float_as_uint(e[QS - 1]);
+      if (int64_t(b) < v.M && int64_t(b) - int64_t(a) > int64_t(v.excl)) {
+        float sm = 0.f;
+        if (!isnan(e[0])) {
+          if (D <= 8) sm = sw_dist<8>(e, D, d, yl, wf);
+          else if (D <= 16) sm = sw_dist<16>(e, D, d, yl, wf);
+          else {
+            for (int q = 0; q < d && sm <= thr; ++q) {
+              float best = -INFINITY;
+              int at = 0;
+              for (int f = 0; f < D; ++f) {
+                const float c = e[f];
+                if (c > best) {
+                  best = c;
+                  at = f;
+                }
+              }
+              e[at] = -INFINITY;
+              sm += sqrtf(fmaxf(2.f * wf * (1.f - (best + yl)), 0.f));
+            }
+          }
+        }
+        if (sm <= thr && sm > jb->rc.lo) sw_record(jb->rc, a, b, sm);
+      }
+    }
+    __syncwarp();
+  }
+  return qn;
+}
+
+template <int P>
+__device__ __forceinline__ void cp_async(uint32_t dst, const void* src) {
+  if constexpr (P == 2)
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src) : "memory");
+  else
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(dst), "l"(src) : "memory");
+}
+
+// Where a lane works: group g of dims of the warp's diagonal group ld.
+struct SwLane {
+  int g, base;
+  uint32_t below, group;   // lanes of the diagonal groups before this one's, and of its own
+  bool live, lead;
+  int ld;
+};
+__device__ __forceinline__ SwLane sw_lane(int G) {
+  const int lane = threadIdx.x & 31, LPW = 32 / G;
+  SwLane l;
+  l.g = lane % G;
+  l.ld = min(lane / G, LPW - 1);
+  l.base = l.ld * G;
+  l.below = (1u << l.base) - 1u;
+  l.group = G == 32 ? ~0u : (((1u << G) - 1u) << l.base);
+  l.live = lane / G < LPW;
+  l.lead = l.live && l.g == 0;
+  return l;
+}
+
+// One row of the recurrence and the test for the lane's 8 diagonals (row i
+// of an 8-row group, column a + i + r in slot (i + r) & 7); t[r] has the
+// sign bit clear when a dim of diagonal r passes.  After diagonal 0, the
+// slot of its column takes the column 8 further.
+template <int P>
+__device__ __forceinline__ void sw_row(float2 (&C)[kSwR][P], SwVec<P> (&df)[kSwR], SwVec<P> (&dg)[kSwR],
+                                       SwVec<P> (&sg)[kSwR], const SwVec<P>& rf, const SwVec<P>& rg,
+                                       const float2 (&nt)[P], int i, const SwVec<P>* pc, int G, uint32_t (&t)[kSwR]) {
+#pragma unroll
+  for (int r = 0; r < kSwR; ++r) {
+    const int k = (i + r) & 7;
+    uint32_t sb = ~0u;
+#pragma unroll
+    for (int p = 0; p < P; ++p) {
+      C[r][p] = __ffma2_rn(rf.v[p], dg[k].v[p], C[r][p]);
+      C[r][p] = __ffma2_rn(rg.v[p], df[k].v[p], C[r][p]);
+      const float2 e = __ffma2_rn(nt[p], sg[k].v[p], C[r][p]);
+      sb &= __float_as_uint(e.x) & __float_as_uint(e.y);
+    }
+    t[r] = sb;
+    if (r == 0) {
+      df[i] = pc[0];
+      dg[i] = pc[64 * G];
+      sg[i] = pc[128 * G];
+    }
+  }
+}
+
+// Loads the 8 columns from b0 (a multiple of 8) into the slots.
+template <int P>
+__device__ __forceinline__ void sw_cols(const SwVec<P>* tab, int64_t b0, int G, int g, SwVec<P> (&df)[kSwR],
+                                        SwVec<P> (&dg)[kSwR], SwVec<P> (&sg)[kSwR]) {
+  const SwVec<P>* p = tab + sw_off(b0) * G + g;
+#pragma unroll
+  for (int r = 0; r < kSwR; ++r, p += 8 * G) {
+    df[r] = p[0];
+    dg[r] = p[64 * G];
+    sg[r] = p[128 * G];
+  }
+}
+
+// An 8-row group in which some dim of some pair passed the first test,
+// again from its start (the cross products in ck), up to its last hot row
+// (bits of hot), with the joint test in the hot rows: the correlations of
+// the lane's dims, their part of the sum, the sum over the
+// diagonal's lanes.  Passing pairs go to the queue, one entry per pair.
+// Returns the queue's length.  Two rows per turn, with the columns moved
+// along in registers: unrolled over all 8 rows, the code fell out of the
+// instruction cache (a sweep of n = 2e4 at a
+// loose threshold took 7.3 ms against 3.4).
+template <int P, int GT>
+__device__ __noinline__ int sw_redo(const SweepJob* jb, const SwVec<P>* rows, SwVec<P>* ck, float* queue,
+                                    int64_t a, int64_t b, uint32_t hot, int qn) {
+  const int G = GT ? GT : jb->v.G, QS = sw_entry<P>(G), lane = threadIdx.x & 31;
+  const SwLane L = sw_lane(G);
+  const SwVec<P>* tab = static_cast<const SwVec<P>*>(jb->v.tab);
+  const float wf = float(jb->v.w);
+  const SwJoint J = sw_joint(jb);
+  const float2 nyl = make_float2(-J.yl, -J.yl);
+  int top = 0;                                                   // the largest power of two below G
+  for (int o = 1; o < G; o <<= 1) top = o;
+  float2 C[kSwR][P];
+  SwVec<P> df[kSwR + 1], dg[kSwR + 1], ib[kSwR + 1];             // columns b + i .. b + i + 8; ib: 1 / sigma
+  auto inv = [](const SwVec<P>& s) {
+    SwVec<P> o;
+#pragma unroll
+    for (int p = 0; p < P; ++p) o.v[p] = make_float2(__fdividef(1.f, s.v[p].x), __fdividef(1.f, s.v[p].y));
+    return o;
+  };
+  auto load = [&](int c, int slot) {
+    const SwVec<P>* p0 = tab + sw_off(b + c) * G + L.g;
+    df[slot] = p0[0];
+    dg[slot] = p0[64 * G];
+    ib[slot] = inv(p0[128 * G]);
+  };
+#pragma unroll
+  for (int r = 0; r < kSwR; ++r) {
+    const SwVec<P> c = ck[r * 32 + lane];
+#pragma unroll
+    for (int p = 0; p < P; ++p) C[r][p] = c.v[p];
+    load(r, r);
+  }
+#pragma unroll 1
+  for (int i2 = 0; hot >> i2; i2 += 2) {
+    load(i2 + 8, 8);
+#pragma unroll
+    for (int h = 0; h < 2; ++h, rows += 3 * G) {
+      const int i = i2 + h;
+      const SwVec<P> rf = rows[0], rg = rows[G];
+#pragma unroll
+      for (int r = 0; r < kSwR; ++r)
+#pragma unroll
+        for (int p = 0; p < P; ++p) {
+          C[r][p] = __ffma2_rn(rf.v[p], dg[h + r].v[p], C[r][p]);
+          C[r][p] = __ffma2_rn(rg.v[p], df[h + r].v[p], C[r][p]);
+        }
+      if (!((hot >> i) & 1u)) continue;
+      SwVec<P> ws = rows[2 * G];
+#pragma unroll
+      for (int p = 0; p < P; ++p) ws.v[p] = make_float2(wf * ws.v[p].x, wf * ws.v[p].y);
+      const SwVec<P> ia = inv(ws);                               // 1 / (w sigma_a)
+      float2 y[kSwR][P];
+      float sum[kSwR];
+      uint32_t hit = 0;
+#pragma unroll
+      for (int r = 0; r < kSwR; ++r) {
+        float2 part = make_float2(0.f, 0.f);
+#pragma unroll
+        for (int p = 0; p < P; ++p) {
+          y[r][p] = __ffma2_rn(__fmul2_rn(C[r][p], ib[h + r].v[p]), ia.v[p], nyl);
+          part = __fadd2_rn(part, make_float2(fmaxf(y[r][p].x, 0.f), fmaxf(y[r][p].y, 0.f)));
+        }
+        sum[r] = fmaf(0.f, y[r][0].x, part.x + part.y);          // NaN (an unresolvable window) stays NaN
+      }
+      if (G == 2) {                                              // over the diagonal's lanes
+#pragma unroll
+        for (int r = 0; r < kSwR; ++r) sum[r] += __shfl_xor_sync(0xffffffffu, sum[r], 1);
+      } else
+      // (to its first one, in a tree that takes any G)
+#pragma unroll 1
+      for (int o = top, len = G; o > 0; len = o, o >>= 1) {
+        const bool add = L.g < o && L.g + o < len;
+#pragma unroll
+        for (int r = 0; r < kSwR; ++r) {
+          const float u = __shfl_down_sync(0xffffffffu, sum[r], o);
+          if (add) sum[r] += u;
+        }
+      }
+#pragma unroll
+      for (int r = 0; r < kSwR; ++r)
+        if (!(sum[r] < J.need)) hit |= 1u << r;
+      if (!L.lead) hit = 0;
+      uint32_t rmask = __reduce_or_sync(0xffffffffu, hit);
+      if (!rmask) continue;
+      __syncwarp();
+#pragma unroll
+      for (int r = 0; r < kSwR; ++r) {                           // the checkpoint has been read: room for y
+        SwVec<P> c;
+#pragma unroll
+        for (int p = 0; p < P; ++p) c.v[p] = y[r][p];
+        ck[r * 32 + lane] = c;
+      }
+#pragma unroll 1
+      while (rmask) {
+        const int r = __ffs(rmask) - 1;
+        rmask &= rmask - 1u;
+        const uint32_t gm = __ballot_sync(0xffffffffu, (hit >> r) & 1u);
+        if (L.live && ((gm >> L.base) & 1u)) {
+          float* e = queue + (qn + __popc(gm & L.below)) * QS;
+          reinterpret_cast<SwVec<P>*>(e)[L.g] = ck[r * 32 + lane];
+          if (L.lead) {
+            e[QS - 2] = __uint_as_float(uint32_t(a + i));
+            e[QS - 1] = __uint_as_float(uint32_t(b + i + r));
+          }
+        }
+        qn += __popc(gm);
+      }
+      if (qn >= 32) qn = sw_drain<P>(jb, queue, qn, false);
+    }
+#pragma unroll
+    for (int r = 0; r + 2 <= kSwR; ++r) {
+      df[r] = df[r + 2];
+      dg[r] = dg[r + 2];
+      ib[r] = ib[r + 2];
+    }
+    load(i2 + 9, 7);
+  }
+  return qn;
+}
+
+// One block of the sweep: row windows [bx seg, bx seg + seg), the
+// diagonals of row `by` of the grid (kSwWarps * (32 / G) * 8 of them, from
+// a multiple of 8 at or below eps + 1).
+template <int P, int GT>
+__device__ __forceinline__ void sw_block(const SweepJob* jb, int64_t bx, int64_t by) {
+  extern __shared__ __align__(16) unsigned char sw_mem[];
+  const SweepView& v = jb->v;
+  const int G = GT ? GT : v.G, D = v.D, w = v.w;
+  const int64_t M = v.M;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int LPW = 32 / G;
+  const SwLane L = sw_lane(G);
+  const int g = L.g;
+  const int64_t a0 = bx * jb->seg;
+  const int64_t dlo = ((int64_t(v.excl) + 1) & ~int64_t(7)) + by * (kSwWarps * LPW * kSwR);
+  const int64_t dfirst = max(dlo, int64_t(v.excl) + 1);          // the block's first diagonal
+  if (dfirst >= M || a0 >= M - dfirst) return;                   // block-uniform
+  const int nrow = int(min(int64_t(jb->seg), M - dfirst - a0));
+  const int64_t b0 = a0 + dlo + int64_t(warp * LPW + L.ld) * kSwR; // this lane's first column, a multiple of 8
+  const int RS = sw_rows<P>(G);
+  SwVec<P>* rows = reinterpret_cast<SwVec<P>*>(sw_mem);                // [2][RS][3][G]
+  SwVec<P>* ck = rows + 2 * RS * G * 3 + warp * (2 * kSwR * 32); // [warps][2][8][32]: C at an 8-row group's start
+  float* queue = reinterpret_cast<float*>(rows + 2 * RS * G * 3 + kSwWarps * 2 * kSwR * 32) +
+                 warp * sw_queue(G) * sw_entry<P>(G);
+  const SwVec<P>* __restrict__ tab = static_cast<const SwVec<P>*>(v.tab);
+  auto stage = [&](int s) {                                      // rows [s RS, s RS + RS) of the block
+    const int rn = min(RS, ((nrow + 7) & ~7) - s * RS);
+    const uint32_t dst = uint32_t(__cvta_generic_to_shared(rows + (s & 1) * RS * G * 3));
+    for (int q = threadIdx.x; q < rn * G * 3; q += kSwThreads) {
+      const int r = q / (3 * G), c = q - r * 3 * G;
+      const int k = c / G;                                       // plane, then group
+      cp_async<P>(dst + uint32_t(q) * uint32_t(sizeof(SwVec<P>)),
+                  tab + (sw_off(a0 + s * RS + r) + 64 * k) * G + (c - k * G));
+    }
+    asm volatile("cp.async.commit_group;" ::: "memory");
+  };
+  __syncthreads();                  // a previous block of this CTA is done with the row buffers
+  stage(0);
+
+  // ---- direct start: C(a0, b) of the lane's 8 columns.  The columns are
+  // centred on the first one's mean c and corrected by
+  // (c - mu_b) sum_t u_t, u_t = x_{a0+t} - mu_a0 (a sum that is zero but
+  // for rounding)
+  float2 C[kSwR][P];
+  {
+    SwVec<P> mah, mal, cc;
+#pragma unroll
+    for (int e = 0; e < (2 * P); ++e) {
+      const int f = (2 * P) * g + e;
+      const bool in = f < D;
+      const double ma = in ? v.mu[int64_t(f) * M + a0] : 0.0;
+      const float hi = float(ma), lo = float(ma - double(hi));
+      const float c = in ? float(v.mu[int64_t(f) * M + min(b0, M - 1)]) : 0.f;
+      if (e & 1) { mah.v[e / 2].y = hi; mal.v[e / 2].y = lo; cc.v[e / 2].y = c; }
+      else { mah.v[e / 2].x = hi; mal.v[e / 2].x = lo; cc.v[e / 2].x = c; }
+    }
+    const SwVec<P>* px = static_cast<const SwVec<P>*>(v.xp) + g;
+    const SwVec<P>* pl = v.xl ? static_cast<const SwVec<P>*>(v.xl) + g : nullptr;
+    auto value = [&](int64_t pos, const SwVec<P>& m) {
+      SwVec<P> x = px[pos * G];
+#pragma unroll
+      for (int p = 0; p < P; ++p) x.v[p] = __fadd2_rn(x.v[p], make_float2(-m.v[p].x, -m.v[p].y));
+      if (pl) {
+        const SwVec<P> l = pl[pos * G];
+#pragma unroll
+        for (int p = 0; p < P; ++p) x.v[p] = __fadd2_rn(x.v[p], l.v[p]);
+      }
+      return x;
+    };
+    SwVec<P> col[kSwR];
+    float2 su[P];
+#pragma unroll
+    for (int p = 0; p < P; ++p) su[p] = make_float2(0.f, 0.f);
+#pragma unroll
+    for (int r = 0; r < kSwR; ++r) {
+#pragma unroll
+      for (int p = 0; p < P; ++p) C[r][p] = make_float2(0.f, 0.f);
+      col[r] = value(sw_pos(b0 + r), cc);
+    }
+    for (int t = 0; t < w; t += 8) {
+      const int64_t pr = sw_pos(a0 + t), pc = sw_pos(b0 + t + 8);
+#pragma unroll
+      for (int i = 0; i < 8; ++i) {
+        SwVec<P> u = value(pr + 8 * i, mah);
+#pragma unroll
+        for (int p = 0; p < P; ++p) {
+          u.v[p] = __fadd2_rn(u.v[p], make_float2(-mal.v[p].x, -mal.v[p].y));
+          if (t + i >= w) u.v[p] = make_float2(0.f, 0.f);
+          su[p] = __fadd2_rn(su[p], u.v[p]);
+        }
+#pragma unroll
+        for (int r = 0; r < kSwR; ++r)
+#pragma unroll
+          for (int p = 0; p < P; ++p) C[r][p] = __ffma2_rn(u.v[p], col[(i + r) & 7].v[p], C[r][p]);
+        col[i] = value(pc + 8 * i, cc);
+      }
+    }
+#pragma unroll
+    for (int r = 0; r < kSwR; ++r) {
+#pragma unroll
+      for (int p = 0; p < P; ++p) {
+        float dm[2];
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+          const int f = (2 * P) * g + 2 * p + h;
+          const float c = h ? cc.v[p].y : cc.v[p].x;
+          dm[h] = f < D ? float(double(c) - v.mu[int64_t(f) * M + min(b0 + r, M - 1)]) : 0.f;
+        }
+        C[r][p] = __ffma2_rn(make_float2(dm[0], dm[1]), su[p], C[r][p]);
+        // a dim that does not exist: negative, against sigma 0
+        if ((2 * P) * g + 2 * p >= D) C[r][p].x = -1.f;
+        if ((2 * P) * g + 2 * p + 1 >= D) C[r][p].y = -1.f;
+      }
+    }
+  }
+
+  // ---- the columns in flight and the row factor of the test
+  const int cstep = 8 * G;                                       // vectors between the columns of an 8-row group
+  SwVec<P> df[kSwR], dg[kSwR], sg[kSwR];
+  sw_cols<P>(tab, b0, G, g, df, dg, sg);
+#pragma unroll
+  for (int r = 0; r < kSwR; ++r) {
+    SwVec<P> c;
+#pragma unroll
+    for (int p = 0; p < P; ++p) c.v[p] = C[r][p];
+    ck[r * 32 + lane] = c;
+  }
+  const float t1 = jb->thr / float(jb->d);
+  const float nk = -(1.f - t1 * t1 / (2.f * float(w))) * float(w);
+  const float2 nk2 = make_float2(nk, nk);
+  int qn = 0, cb = 0, redone = 0;   // queued hits, this group's checkpoint, groups run twice
+  const int nstage = (nrow + RS - 1) / RS;
+  for (int s = 0; s < nstage; ++s) {
+    asm volatile("cp.async.wait_group 0;" ::: "memory");
+    __syncthreads();                // this stage's rows are here, the other buffer is free
+    if (s == 0) {                   // the first row takes no update
+      for (int q = threadIdx.x; q < G * 2; q += kSwThreads) {
+#pragma unroll
+        for (int p = 0; p < P; ++p) rows[q].v[p] = make_float2(0.f, 0.f);
+      }
+      __syncthreads();
+    }
+    if (s + 1 < nstage) stage(s + 1);
+    const int rn = min(RS, ((nrow + 7) & ~7) - s * RS);
+    const SwVec<P>* rp = rows + (s & 1) * RS * G * 3 + g;
+    SwVec<P> nf = rp[0], ng = rp[G], ns = rp[2 * G];                    // the next row's record
+    // 8 rows at a time without a branch: the tests' sign bits of all their
+    // pairs are combined, and a group in which one passed runs once more
+    // from its start (a branch after every row, with what it kept from
+    // overlapping, took 185 ms on the wide workload against 145)
+    for (int r0 = 0; r0 < rn; r0 += 8) {
+      const int64_t ro = int64_t(s) * RS + r0;
+      const SwVec<P>* pc = tab + sw_off(b0 + ro + 8) * G + g;
+      const SwVec<P>* r8 = rp;
+      uint32_t quiet = ~0u;                                      // bit 7 - i: no dim of row i's pairs passed
+#pragma unroll
+      for (int i = 0; i < 8; ++i) {
+        const SwVec<P> rf = nf, rg = ng;
+        float2 nt[P];
+#pragma unroll
+        for (int p = 0; p < P; ++p) nt[p] = __fmul2_rn(ns.v[p], nk2);
+        if (i < 7 || r0 + 8 < rn) rp += G * 3;                   // (the last row of the stage is read again)
+        nf = rp[0];
+        ng = rp[G];
+        ns = rp[2 * G];
+        uint32_t t[kSwR];
+        sw_row<P>(C, df, dg, sg, rf, rg, nt, i, pc, G, t);
+        pc += cstep;
+        const uint32_t all = ((t[0] & t[1] & t[2]) & (t[3] & t[4])) & ((t[5] & t[6]) & t[7]);
+        quiet = __funnelshift_l(all, quiet, 1);
+      }
+      cb ^= kSwR * 32;
+#pragma unroll
+      for (int r = 0; r < kSwR; ++r) {                           // C at the next group's start
+        SwVec<P> c;
+#pragma unroll
+        for (int p = 0; p < P; ++p) c.v[p] = C[r][p];
+        ck[cb + r * 32 + lane] = c;
+      }
+      if (__any_sync(0xffffffffu, quiet != ~0u)) {
+        ++redone;
+        const uint32_t hot = __brev(__reduce_or_sync(0xffffffffu, ~quiet)) >> 24;   // bit i: row i
+        qn = sw_redo<P, GT>(jb, r8, ck + (cb ^ (kSwR * 32)), queue, a0 + ro, b0 + ro, hot, qn);
+        // the state again from memory, so that none of it lives across the call
+#pragma unroll
+        for (int r = 0; r < kSwR; ++r) {
+          const SwVec<P> c = ck[cb + r * 32 + lane];
+#pragma unroll
+          for (int p = 0; p < P; ++p) C[r][p] = c.v[p];
+        }
+        sw_cols<P>(tab, b0 + ro + 8, G, g, df, dg, sg);
+        nf = rp[0];
+        ng = rp[G];
+        ns = rp[2 * G];
+      }
+    }
+  }
+  sw_drain<P>(jb, queue, qn, true);
+  if (jb->groups && lane == 0) {
+    atomicAdd(&jb->groups[0], (unsigned long long)((nrow + 7) / 8));
+    atomicAdd(&jb->groups[1], (unsigned long long)redone);
+  }
+}
+
+template <int P, int GT>
+__global__ void __launch_bounds__(kSwThreads, kSwBlocks<P>)
+k_sweep(const __grid_constant__ SweepJob jb, int64_t ybase) {
+  sw_block<P, GT>(&jb, int64_t(blockIdx.x), ybase + int64_t(blockIdx.y));
+}
+
+// Every stride-th block of the sweep's grid, at a varying offset.
+__host__ __device__ __forceinline__ int64_t sw_sampled(int64_t q, int64_t stride) {
+  return q * stride + int64_t((uint64_t(q) * 2654435761ull) % uint64_t(stride));
+}
+template <int P>
+__global__ void __launch_bounds__(kSwThreads, kSwBlocks<P>)
+k_sweep_sample(const __grid_constant__ SweepJob jb, int64_t nbx, int64_t stride) {
+  const int64_t q = sw_sampled(int64_t(blockIdx.x), stride);
+  sw_block<P, 0>(&jb, q % nbx, q / nbx);
+}
+
+// The sweeps of several series in one persistent launch: each CTA takes
+// (series, row block, diagonal block) items from a device queue in order
+// (largest series first) until the queue is empty; an item is one block of
+// the sweep above on that series' index, threshold and record buffers.
+template <int P>
+__global__ void __launch_bounds__(kSwThreads, kSwBlocks<P>)
+k_sweep_batch(const SweepJob* __restrict__ jobs, const SweepItem* __restrict__ items, int nitems,
+              int* __restrict__ next) {
+  __shared__ int cur;
+  for (;;) {
+    __syncthreads();                // every thread has read the previous item
+    if (threadIdx.x == 0) cur = atomicAdd(next, 1);
+    __syncthreads();
+    const int it = cur;
+    if (it >= nitems) return;       // block-uniform
+    const SweepItem q = items[it];
+    sw_block<P, 0>(jobs + q.job, int64_t(q.bx), int64_t(q.by));
+  }
+}
+
+int64_t sw_diags(int G) { return int64_t(kSwWarps) * (32 / G) * kSwR; }   // per block
+
+// Diagonal blocks of the whole sweep (0: no non-trivial pair).
+int64_t sw_gy(const SweepView& v) {
+  const int64_t first = int64_t(v.excl) + 1;
+  if (first >= v.M) return 0;
+  const int64_t lo = first & ~int64_t(7), nd = sw_diags(v.G);
+  return (v.M - lo + nd - 1) / nd;
+}
+
+// Rows per block.  A block pays a direct start of w points (about 22
+// issue slots each) before its rows (about 78 each); a launch runs about
+// three blocks per SM at a time.  Long blocks where there are many of
+// them, shorter ones where a wave would not be filled.
+int sw_seg(const SweepView& v) {
+  const int64_t slots = int64_t(sm_count()) * (v.P == 2 ? kSwBlocks<2> : kSwBlocks<1>), nd = sw_diags(v.G), gy = sw_gy(v);
+  int best = 2048;
+  double best_cost = 1e300;
+  for (int seg = 2048; seg >= 32; seg >>= 1) {
+    int64_t blocks = 0;
+    for (int64_t by = 0; by < gy; ++by) {
+      const int64_t d0 = ((int64_t(v.excl) + 1) & ~int64_t(7)) + by * nd;
+      blocks += std::max<int64_t>(0, (v.M - d0 + seg - 1) / seg);
+    }
+    const double waves = std::max(1.0, double(blocks) / double(slots));
+    const double cost = (waves > 4.0 ? waves : std::ceil(waves)) * (22.0 * v.w + 78.0 * seg);
+    if (cost < best_cost) {
+      best_cost = cost;
+      best = seg;
+    }
+  }
+  return best;
+}
+
+}  // namespace
+
+size_t sweep_table_bytes(const Index& ix) {
+  const int P = sw_pairs(ix.D);
+  const size_t G = size_t((ix.D + 2 * P - 1) / (2 * P));
+  return (size_t(sw_round(ix.M)) * 3 + size_t(sw_round(ix.n)) * (ix.has_lo ? 2 : 1)) * G * (8 * size_t(P));
+}
+
+template <int P>
+static cudaError_t sweep_table(const Index& ix, SweepView& v, void* buf, cudaStream_t s) {
+  SwVec<P>* tab = static_cast<SwVec<P>*>(buf);
+  SwVec<P>* xp = tab + v.Mpad * v.G * 3;
+  SwVec<P>* xl = ix.has_lo ? xp + v.npad * v.G : nullptr;
+  v.tab = tab;
+  v.xp = xp;
+  v.xl = xl;
+  MOMENTI_LAUNCH("sweep_table", s, k_sweep_table<P><<<unsigned(v.npad / 64), 256, 0, s>>>(ix, v, tab, xp, xl));
+  return cudaGetLastError();
+}
+
+cudaError_t launch_sweep_table(const Index& ix, void* buf, SweepView* out, cudaStream_t s) {
+  SweepView v;
+  v.M = ix.M;
+  v.Mpad = sw_round(ix.M);
+  v.npad = sw_round(ix.n);
+  v.D = ix.D;
+  v.P = sw_pairs(ix.D);
+  v.G = (ix.D + 2 * v.P - 1) / (2 * v.P);
+  v.w = ix.w;
+  v.excl = ix.excl;
+  v.mu = ix.mu;
+  const cudaError_t e = v.P == 2 ? sweep_table<2>(ix, v, buf, s) : sweep_table<1>(ix, v, buf, s);
+  *out = v;
+  return e;
+}
+
+template <int P, int GT>
+static cudaError_t sweep(const SweepJob& jb, int64_t gy, cudaStream_t s) {
+  const size_t smem = sw_smem<P>(jb.v.G);
+  cudaError_t e = allow_smem(reinterpret_cast<const void*>(k_sweep<P, GT>), smem);
+  if (e != cudaSuccess) return e;
+  for (int64_t y0 = 0; y0 < gy; y0 += 65535) {
+    dim3 grid{unsigned((jb.v.M + jb.seg - 1) / jb.seg), unsigned(std::min<int64_t>(65535, gy - y0)), 1u};
+    MOMENTI_LAUNCH("allpairs", s, k_sweep<P, GT><<<grid, kSwThreads, smem, s>>>(jb, y0));
+  }
+  return cudaGetLastError();
+}
+
+cudaError_t launch_allpairs(const SweepView& v, int d, float thr, const ApRec& rc, cudaStream_t s) {
+  const int64_t gy = sw_gy(v);
+  if (gy <= 0) return cudaSuccess;
+  SweepJob jb;
+  jb.v = v;
+  jb.rc = rc;
+  jb.thr = thr;
+  jb.d = d;
+  jb.seg = sw_seg(v);
+  // offsets of the lanes' groups as constants where D is common: the
+  // runtime form spills (7.8 ms against 6.8 at D = 5, n = 1e5)
+  if (v.P == 1) return v.G == 1 ? sweep<1, 1>(jb, gy, s) : sweep<1, 3>(jb, gy, s);
+  switch (v.G) {
+    case 1: return sweep<2, 1>(jb, gy, s);
+    case 2: return sweep<2, 2>(jb, gy, s);
+    case 3: return sweep<2, 3>(jb, gy, s);
+    case 4: return sweep<2, 4>(jb, gy, s);
+    case 5: return sweep<2, 5>(jb, gy, s);
+    case 6: return sweep<2, 6>(jb, gy, s);
+    case 8: return sweep<2, 8>(jb, gy, s);
+    case 16: return sweep<2, 16>(jb, gy, s);
+    default: return sweep<2, 0>(jb, gy, s);
+  }
+}
+
+template <int P>
+static cudaError_t sweep_sample(const SweepJob& jb, int64_t nbx, int64_t blocks, int64_t stride, cudaStream_t s) {
+  const size_t smem = sw_smem<P>(jb.v.G);
+  cudaError_t e = allow_smem(reinterpret_cast<const void*>(k_sweep_sample<P>), smem);
+  if (e != cudaSuccess) return e;
+  MOMENTI_LAUNCH("allpairs_sample", s, k_sweep_sample<P><<<unsigned(blocks), kSwThreads, smem, s>>>(jb, nbx, stride));
+  return cudaGetLastError();
+}
+
+cudaError_t launch_allpairs_sample(const SweepView& v, int d, float thr, const ApRec& rc, double fraction,
+                                   int seg, double* pairs, unsigned long long* groups, cudaStream_t s) {
+  *pairs = 0.0;
+  const int64_t gy = sw_gy(v), nd = sw_diags(v.G);
+  if (gy <= 0) return cudaSuccess;
+  SweepJob jb;
+  jb.v = v;
+  jb.rc = rc;
+  jb.thr = thr;
+  jb.d = d;
+  jb.seg = seg;
+  jb.groups = groups;
+  const int64_t nbx = (v.M + seg - 1) / seg, total = nbx * gy;
+  const int64_t stride = std::max<int64_t>(1, std::min<int64_t>(int64_t(1.0 / fraction), total));
+  const int64_t blocks = std::min<int64_t>((total + stride - 1) / stride, int64_t(1) << 30);
+  // pairs the sampled blocks hold
+  for (int64_t q = 0; q < blocks; ++q) {
+    const int64_t lin = sw_sampled(q, stride);
+    if (lin >= total) continue;
+    const int64_t a0 = (lin % nbx) * seg, dlo = ((int64_t(v.excl) + 1) & ~int64_t(7)) + (lin / nbx) * nd;
+    const int64_t d0 = std::max(dlo, int64_t(v.excl) + 1), d1 = std::min(dlo + nd, v.M);
+    // rows a0 .. a0 + seg - 1 against diagonals d0 .. d1 - 1 with a + delta < M
+    for (int64_t dl = d0; dl < d1; dl += 64) {
+      const int64_t c = std::min<int64_t>(64, d1 - dl);
+      *pairs += double(c) * double(std::max<int64_t>(0, std::min<int64_t>(seg, v.M - (dl + c / 2) - a0)));
+    }
+  }
+  return v.P == 2 ? sweep_sample<2>(jb, nbx, blocks, stride, s) : sweep_sample<1>(jb, nbx, blocks, stride, s);
+}
+
+template <int P>
+static cudaError_t sweep_batch(const SweepJob* jobs, const std::vector<SweepItem>& items, size_t smem,
+                               cudaStream_t s) {
+  if (items.empty()) return cudaSuccess;
+  SweepItem* ditems = nullptr;
+  int* dnext = nullptr;
+  cudaError_t e = cudaMallocAsync(&ditems, items.size() * sizeof(SweepItem), s);
+  if (e == cudaSuccess) e = cudaMallocAsync(&dnext, sizeof(int), s);
+  if (e == cudaSuccess) e = cudaMemcpyAsync(ditems, items.data(), items.size() * sizeof(SweepItem), cudaMemcpyHostToDevice, s);
+  if (e == cudaSuccess) e = cudaMemsetAsync(dnext, 0, sizeof(int), s);
+  if (e == cudaSuccess) e = allow_smem(reinterpret_cast<const void*>(k_sweep_batch<P>), smem);
+  if (e == cudaSuccess) {
+    const int64_t grid = std::min<int64_t>(int64_t(sm_count()) * kSwBlocks<P>, int64_t(items.size()));
+    MOMENTI_LAUNCH("allpairs_batch", s, k_sweep_batch<P><<<unsigned(grid), kSwThreads, smem, s>>>(jobs, ditems, int(items.size()), dnext));
+    e = cudaGetLastError();
+  }
+  if (ditems) cudaFreeAsync(ditems, s);
+  if (dnext) cudaFreeAsync(dnext, s);
+  return e;
+}
+
+cudaError_t launch_allpairs_batch(std::vector<SweepJob> jobs, cudaStream_t s) {
+  if (jobs.empty()) return cudaSuccess;
+  // items of every job, largest series first; one launch per form
+  std::stable_sort(jobs.begin(), jobs.end(), [](const SweepJob& x, const SweepJob& y) { return x.v.M > y.v.M; });
+  std::vector<SweepItem> items[2];
+  size_t smem[2] = {0, 0};
+  for (size_t q = 0; q < jobs.size(); ++q) {
+    SweepJob& j = jobs[q];
+    const int64_t gy = sw_gy(j.v);
+    if (gy <= 0) continue;
+    const int f = j.v.P - 1;
+    j.seg = sw_seg(j.v);
+    smem[f] = std::max(smem[f], sw_smem(j.v));
+    for (int64_t by = 0; by < gy; ++by) {
+      const int64_t dfirst = std::max(((int64_t(j.v.excl) + 1) & ~int64_t(7)) + by * sw_diags(j.v.G),
+                                      int64_t(j.v.excl) + 1);
+      for (int64_t bx = 0; bx * j.seg < j.v.M - dfirst; ++bx)
+        items[f].push_back(SweepItem{uint32_t(q), uint32_t(bx), uint32_t(by)});
+    }
+  }
+  SweepJob* djobs = nullptr;
+  cudaError_t e = cudaMallocAsync(&djobs, jobs.size() * sizeof(SweepJob), s);
+  if (e == cudaSuccess) e = cudaMemcpyAsync(djobs, jobs.data(), jobs.size() * sizeof(SweepJob), cudaMemcpyHostToDevice, s);
+  if (e == cudaSuccess) e = sweep_batch<1>(djobs, items[0], smem[0], s);
+  if (e == cudaSuccess) e = sweep_batch<2>(djobs, items[1], smem[1], s);
+  if (djobs) cudaFreeAsync(djobs, s);
+  return e;
+}
+
+}  // namespace momenti

@@ -1,5 +1,4 @@
-// Candidate verification (the distance check of Algorithm 1's inner loop)
-// and the exact all-pairs path (the final fallback of Algorithm 1).
+// Candidate verification (the distance check of Algorithm 1's inner loop).
 //
 // Per pair: the z-normalised Euclidean distance of Eq. (zned) in every
 // dimension, computed directly from the centred windows,
@@ -8,330 +7,360 @@
 // lower dimension), dims_d as a mask and dist_d^max (Eq. distdmax).  One
 // warp per pair, lanes over t, in float32 (the traversal) or float64 (the
 // final re-verification).
-//
-// The all-pairs path walks the diagonals b - a = delta of the distance
-// matrix: along a diagonal the dot product of the two centred windows
-// slides by one product in and one out, restarted from a direct sum every
-// kSeg steps; the per-dimension distance follows from the Pearson form
-// dist^2 = n_a + n_b - 2 w corr (Section 2), n = w for non-flat windows and
-// 0 for flat ones.  Pairs whose dist_d may be <= tau are collected and then
-// verified exactly by the direct form above.
 #include "internal.h"
 
 #include <algorithm>
-#include <cstdio>
-#include <cstdlib>
-#include <map>
-#include <mutex>
-#include <string>
-#include <tuple>
-#include <vector>
-
-#include "k_verify_kernels.cuh"
+#include <cstdint>
 
 namespace momenti {
 
 namespace {
 
-bool aligned32(const void* q) { return (reinterpret_cast<uintptr_t>(q) & 31u) == 0; }
-
-// Candidates for this index (0 when the recording sweep has no variants:
-// float64 input, no point-major copy).  The statistics forms read column
-// rows with 256-bit loads, so their rows must start on 32-byte boundaries
-// (the pool aligns far beyond that; checked, not assumed).
-int sweep_variants(const Index& ix) {
-  if (ix.xW && ix.isW && rows2_usable(ix) && aligned32(ix.xW) && aligned32(ix.isW)) return 2;
-  if (ix.isT && ix.xT && !ix.has_lo && aligned32(ix.xT) && aligned32(ix.isT))
-    return rows_fit(ix.w, ix.Dp) ? 3 : 2;
-  return 0;
+__device__ __forceinline__ float warp_sum(float v) {
+  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+  return v;
+}
+__device__ __forceinline__ double warp_sum(double v) {
+  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+  return v;
+}
+template <typename T>
+__device__ __forceinline__ T warp_max(T v) {
+  for (int o = 16; o > 0; o >>= 1) v = max(v, __shfl_xor_sync(0xffffffffu, v, o));
+  return v;
 }
 
-// Variant v: wide: 0 statistics, 1 slid; D <= 16: 0 statistics with the
-// taller stage, 1 statistics with half of it, 2 slid.
-cudaError_t sweep_launch(const Index& ix, int v, int d, float thr, const ApRec& rc, cudaStream_t s,
-                         int64_t gy_max) {
-  if (ix.xW) {
-    if (ix.DW == 32) return v == 0 ? rows4_launch<32>(ix, d, thr, rc, s, gy_max) : rows2_launch<32>(ix, d, thr, rc, s, gy_max);
-    return v == 0 ? launch_rows4_64(ix, d, thr, rc, s, gy_max) : launch_rows2_64(ix, d, thr, rc, s, gy_max);
-  }
-  switch (ix.Dp) {
-    case 4:
-      if (v == 0) return rows3_launch<4, kRowSub3, 3>(ix, d, thr, rc, s, gy_max);
-      if (v == 1) return rows3_launch<4, kRowSub3 / 2, 3>(ix, d, thr, rc, s, gy_max);
-      return rows_slid_launch<4>(ix, d, thr, rc, s, gy_max);
-    case 8:
-      if (v == 0) return rows3_launch<8, kRowSub3, 3>(ix, d, thr, rc, s, gy_max);
-      if (v == 1) return rows3_launch<8, kRowSub3 / 2, 3>(ix, d, thr, rc, s, gy_max);
-      return rows_slid_launch<8>(ix, d, thr, rc, s, gy_max);
-    default:
-      if (v == 0) return rows3_launch<16, kRowSub3 / 2, 2>(ix, d, thr, rc, s, gy_max);
-      if (v == 1) return rows3_launch<16, kRowSub3 / 4, 2>(ix, d, thr, rc, s, gy_max);
-      return rows_slid_launch<16>(ix, d, thr, rc, s, gy_max);
-  }
-}
-
-struct TuneKey {
-  int dev, dp, lw, lm;
-  bool operator<(const TuneKey& o) const {
-    return std::tie(dev, dp, lw, lm) < std::tie(o.dev, o.dp, o.lw, o.lm);
-  }
+struct VerifyOut {
+  double dist_d, dist_max;
+  uint64_t mask;
 };
-std::mutex& tune_mu() {
-  static std::mutex m;
-  return m;
-}
-std::map<TuneKey, int>& tune_map() {
-  static std::map<TuneKey, int> t;
-  return t;
-}
-int ilog2(int64_t x) {
-  int l = 0;
-  while (x > 1) { x >>= 1; ++l; }
-  return l;
+
+// Distances of one pair; lane f (and f - 32) ends up holding dimension f.
+template <typename T>
+__device__ void pair_distances(const Index& ix, uint32_t a, uint32_t b, T dist[2]) {
+  const int lane = threadIdx.x & 31;
+  dist[0] = dist[1] = T(0);
+  for (int f = 0; f < ix.D; ++f) {
+    const int64_t oa = int64_t(f) * ix.M + a, ob = int64_t(f) * ix.M + b;
+    const float* xa = ix.xs_hi + int64_t(f) * ix.n + a;
+    const float* xb = ix.xs_hi + int64_t(f) * ix.n + b;
+    const float* la = ix.has_lo ? ix.xs_lo + int64_t(f) * ix.n + a : nullptr;
+    const float* lb = ix.has_lo ? ix.xs_lo + int64_t(f) * ix.n + b : nullptr;
+    T s = T(0);
+    if constexpr (sizeof(T) == 4) {
+      const float m0a = ix.mu_hi[oa], m1a = ix.mu_lo[oa], isa = ix.inv_sig[oa];
+      const float m0b = ix.mu_hi[ob], m1b = ix.mu_lo[ob], isb = ix.inv_sig[ob];
+      for (int t = lane; t < ix.w; t += 32) {
+        float za = ((xa[t] - m0a) + ((la ? la[t] : 0.f) - m1a)) * isa;
+        float zb = ((xb[t] - m0b) + ((lb ? lb[t] : 0.f) - m1b)) * isb;
+        float dd = za - zb;
+        s = fmaf(dd, dd, s);
+      }
+    } else {
+      const double ma = ix.mu[oa], mb = ix.mu[ob];
+      const double sa = ix.sig[oa], sb = ix.sig[ob];
+      const bool fa = sa <= kFlatRel * (1.0 + fabs(ma)), fb = sb <= kFlatRel * (1.0 + fabs(mb));
+      const double isa = fa ? 0.0 : 1.0 / sa, isb = fb ? 0.0 : 1.0 / sb;
+      for (int t = lane; t < ix.w; t += 32) {
+        double va = double(xa[t]) + (la ? double(la[t]) : 0.0);
+        double vb = double(xb[t]) + (lb ? double(lb[t]) : 0.0);
+        double dd = (va - ma) * isa - (vb - mb) * isb;
+        s = fma(dd, dd, s);
+      }
+    }
+    s = warp_sum(s);
+    if (lane == (f & 31)) dist[f >> 5] = sqrt(s);
+  }
 }
 
-// The variant the sweep of this index runs: MOMENTI_SWEEP_VARIANT=v forces
-// one; MOMENTI_AUTOTUNE=0 takes variant 0; otherwise the cached choice for
-// (device, padded D, log2 w, log2 M), or, the first time, the fastest
-// candidate on a probe: every candidate runs three times over the grid's
-// first diagonal blocks (about four waves of CTAs, the longest diagonals)
-// with a negative threshold, which records nothing; the faster of the last
-// two runs counts (CUDA events on the sweep's stream).  Probes run one at a
-// time in the process.
-int sweep_variant(const Index& ix, int d, const ApRec& rc, cudaStream_t s) {
-  const int nv = sweep_variants(ix);
-  if (const char* f = std::getenv("MOMENTI_SWEEP_VARIANT"); f && f[0] >= '0' && f[0] <= '9')
-    return std::min(nv - 1, int(f[0] - '0'));
-  if (nv <= 1) return 0;
-  if (const char* e = std::getenv("MOMENTI_AUTOTUNE"); e && e[0] == '0') return 0;
-  int dev = 0;
-  cudaGetDevice(&dev);
-  const TuneKey key{dev, ix.xW ? ix.DW : ix.Dp, ilog2(ix.w), ilog2(ix.M)};
-  {
-    std::lock_guard<std::mutex> g(tune_mu());
-    auto it = tune_map().find(key);
-    if (it != tune_map().end()) return it->second;
-  }
-  // one probe at a time in the process (probes of other threads would
-  // share the GPU with this one and distort its timings)
-  static std::mutex probe_mu;
-  std::lock_guard<std::mutex> probe_lock(probe_mu);
-  {
-    std::lock_guard<std::mutex> g(tune_mu());
-    auto it = tune_map().find(key);
-    if (it != tune_map().end()) return it->second;
-  }
-  const int64_t nbx = (ix.M + kSeg - 1) / kSeg;
-  const int64_t gy_probe = std::max<int64_t>(1, (int64_t(sm_count()) * 8 + nbx - 1) / nbx);
-  cudaEvent_t e0 = nullptr, e1 = nullptr;
-  if (cudaEventCreate(&e0) != cudaSuccess || cudaEventCreate(&e1) != cudaSuccess) {
-    if (e0) cudaEventDestroy(e0);
-    return 0;
-  }
-  int best = 0;
-  float best_ms = INFINITY;
-  std::string line;
-  for (int v = 0; v < nv; ++v) {
-    float ms = INFINITY;
-    bool ok = true;
-    for (int rep = 0; rep < 3 && ok; ++rep) {    // a warm-up, then the faster of two
-      float t = INFINITY;
-      ok = cudaEventRecord(e0, s) == cudaSuccess &&
-           sweep_launch(ix, v, d, -1.f, rc, s, gy_probe) == cudaSuccess &&
-           cudaEventRecord(e1, s) == cudaSuccess && cudaEventSynchronize(e1) == cudaSuccess &&
-           cudaEventElapsedTime(&t, e0, e1) == cudaSuccess;
-      if (rep > 0) ms = std::min(ms, t);
+// Sum of the d smallest of D per-lane distances (ties to the lower index).
+template <typename T>
+__device__ VerifyOut select_d(const T dist[2], int D, int d) {
+  const int lane = threadIdx.x & 31;
+  int rank[2] = {0, 0};
+  for (int g = 0; g < D; ++g) {
+    T vg = __shfl_sync(0xffffffffu, dist[g >> 5], g & 31);
+    for (int h = 0; h < 2; ++h) {
+      int f = lane + 32 * h;
+      if (f < D && (vg < dist[h] || (vg == dist[h] && g < f))) ++rank[h];
     }
-    if (!ok) {
-      cudaGetLastError();       // a candidate that cannot launch is skipped
+  }
+  T sum = 0, mx = 0;
+  bool sel0 = lane < D && rank[0] < d, sel1 = lane + 32 < D && rank[1] < d;
+  if (sel0) { sum += dist[0]; mx = dist[0]; }
+  if (sel1) { sum += dist[1]; mx = max(mx, dist[1]); }
+  sum = warp_sum(sum);
+  mx = warp_max(mx);
+  uint64_t m0 = __ballot_sync(0xffffffffu, sel0), m1 = __ballot_sync(0xffffffffu, sel1);
+  return VerifyOut{double(sum), double(mx), m0 | (m1 << 32)};
+}
+
+// Per-dimension distances of one pair in FP32 with all dims' partial sums
+// kept per lane (loads of every dim in flight together), then the D warp
+// reductions interleaved; lane f (and f - 32) ends with dimension f.
+template <int DM>
+__device__ __forceinline__ void pair_distances_fast(const Index& ix, uint32_t a, uint32_t b,
+                                                    float dist[2]) {
+  const int lane = threadIdx.x & 31;
+  float acc[DM];
+#pragma unroll
+  for (int f = 0; f < DM; ++f) acc[f] = 0.f;
+#pragma unroll
+  for (int f = 0; f < DM; ++f) {
+    if (f < ix.D) {
+      const int64_t oa = int64_t(f) * ix.M + a, ob = int64_t(f) * ix.M + b;
+      const float m0a = ix.mu_hi[oa], m1a = ix.mu_lo[oa], isa = ix.inv_sig[oa];
+      const float m0b = ix.mu_hi[ob], m1b = ix.mu_lo[ob], isb = ix.inv_sig[ob];
+      const float* xa = ix.xs_hi + int64_t(f) * ix.n + a;
+      const float* xb = ix.xs_hi + int64_t(f) * ix.n + b;
+      const float* la = ix.has_lo ? ix.xs_lo + int64_t(f) * ix.n + a : nullptr;
+      const float* lb = ix.has_lo ? ix.xs_lo + int64_t(f) * ix.n + b : nullptr;
+      float s = 0.f;
+      for (int t = lane; t < ix.w; t += 32) {
+        float za = ((xa[t] - m0a) + ((la ? la[t] : 0.f) - m1a)) * isa;
+        float zb = ((xb[t] - m0b) + ((lb ? lb[t] : 0.f) - m1b)) * isb;
+        float dd = za - zb;
+        s = fmaf(dd, dd, s);
+      }
+      acc[f] = s;
+    }
+  }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1)
+#pragma unroll
+    for (int f = 0; f < DM; ++f) acc[f] += __shfl_xor_sync(0xffffffffu, acc[f], o);
+  dist[0] = dist[1] = 0.f;
+#pragma unroll
+  for (int f = 0; f < DM; ++f)
+    if (f < ix.D && lane == (f & 31)) dist[f >> 5] = sqrtf(acc[f]);
+}
+
+template <int DP>
+__device__ __forceinline__ void load_row(const float* __restrict__ base, int64_t t, float (&v)[DP]) {
+  const float4* p = reinterpret_cast<const float4*>(base + t * DP);
+#pragma unroll
+  for (int q = 0; q < DP / 4; ++q) {
+    const float4 u = p[q];
+    v[4 * q] = u.x; v[4 * q + 1] = u.y; v[4 * q + 2] = u.z; v[4 * q + 3] = u.w;
+  }
+}
+
+// dist_d of a pair from per-dim distances (registers), the d smallest.
+template <int DM>
+__device__ __forceinline__ float sum_d_smallest(const float (&v)[DM], int D, int d) {
+  float best[DM];
+#pragma unroll
+  for (int q = 0; q < DM; ++q) best[q] = INFINITY;
+#pragma unroll
+  for (int f = 0; f < DM; ++f) {
+    if (f < D) {
+      float x = v[f];
+      // insert x into the sorted prefix best[0..d)
+#pragma unroll
+      for (int q = DM - 1; q >= 0; --q) {
+        if (q < d) {
+          float prev = q > 0 ? best[q - 1] : -INFINITY;
+          if (x < best[q]) best[q] = x >= prev ? x : prev;
+        }
+      }
+    }
+  }
+  float s = 0.f;
+#pragma unroll
+  for (int q = 0; q < DM; ++q)
+    if (q < d) s += best[q];
+  return s;
+}
+
+// Window statistics of window a from the point-major copy: 3 rows of DP.
+template <int DP>
+__device__ __forceinline__ void load_stats(const Index& ix, uint32_t a, float (&mh)[DP],
+                                           float (&ml)[DP], float (&is)[DP]) {
+  const float* base = ix.stT + int64_t(a) * 3 * DP;
+  load_row<DP>(base, 0, mh);
+  load_row<DP>(base + DP, 0, ml);
+  load_row<DP>(base + 2 * DP, 0, is);
+}
+
+// Point-major form (D <= 8): each lane reads all dims of a time point of
+// both windows with float4 loads.  Padding dims have 1/sigma = 0 and add 0.
+template <int DP, bool LO>
+__device__ __forceinline__ void pair_distances_pm(const Index& ix, uint32_t a, uint32_t b,
+                                                  float dist[2]) {
+  const int lane = threadIdx.x & 31;
+  float m0a[DP], m1a[DP], isa[DP], m0b[DP], m1b[DP], isb[DP], acc[DP];
+  load_stats<DP>(ix, a, m0a, m1a, isa);
+  load_stats<DP>(ix, b, m0b, m1b, isb);
+#pragma unroll
+  for (int f = 0; f < DP; ++f) acc[f] = 0.f;
+  const float4* pa = reinterpret_cast<const float4*>(ix.xT + int64_t(a) * DP);
+  const float4* pb = reinterpret_cast<const float4*>(ix.xT + int64_t(b) * DP);
+  const float4* la = LO ? reinterpret_cast<const float4*>(ix.xlT + int64_t(a) * DP) : nullptr;
+  const float4* lb = LO ? reinterpret_cast<const float4*>(ix.xlT + int64_t(b) * DP) : nullptr;
+  for (int t = lane; t < ix.w; t += 32) {
+    float xa[DP], xb[DP], ya[DP], yb[DP];
+#pragma unroll
+    for (int v = 0; v < DP / 4; ++v) {
+      const float4 qa = pa[int64_t(t) * (DP / 4) + v], qb = pb[int64_t(t) * (DP / 4) + v];
+      xa[4 * v] = qa.x; xa[4 * v + 1] = qa.y; xa[4 * v + 2] = qa.z; xa[4 * v + 3] = qa.w;
+      xb[4 * v] = qb.x; xb[4 * v + 1] = qb.y; xb[4 * v + 2] = qb.z; xb[4 * v + 3] = qb.w;
+      if (LO) {
+        const float4 ra = la[int64_t(t) * (DP / 4) + v], rb = lb[int64_t(t) * (DP / 4) + v];
+        ya[4 * v] = ra.x; ya[4 * v + 1] = ra.y; ya[4 * v + 2] = ra.z; ya[4 * v + 3] = ra.w;
+        yb[4 * v] = rb.x; yb[4 * v + 1] = rb.y; yb[4 * v + 2] = rb.z; yb[4 * v + 3] = rb.w;
+      }
+    }
+#pragma unroll
+    for (int f = 0; f < DP; ++f) {
+      const float za = ((xa[f] - m0a[f]) + ((LO ? ya[f] : 0.f) - m1a[f])) * isa[f];
+      const float zb = ((xb[f] - m0b[f]) + ((LO ? yb[f] : 0.f) - m1b[f])) * isb[f];
+      const float dd = za - zb;
+      acc[f] = fmaf(dd, dd, acc[f]);
+    }
+  }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1)
+#pragma unroll
+    for (int f = 0; f < DP; ++f) acc[f] += __shfl_xor_sync(0xffffffffu, acc[f], o);
+  dist[0] = dist[1] = 0.f;
+#pragma unroll
+  for (int f = 0; f < DP; ++f)
+    if (f < ix.D && lane == f) dist[0] = sqrtf(acc[f]);
+}
+
+// Lower bound of dist_d from segment means (piecewise aggregate
+// approximation): for 16-point segments of both windows,
+//   sum_t (z_a - z_b)^2 >= sum_k 16 (mean_k z_a - mean_k z_b)^2
+// (Cauchy-Schwarz on every segment; the points after the last full
+// segment are left out, which only lowers the bound), and the sum of the d
+// smallest per-dim bounds is below dist_d.  Reads w/16 rows per window.
+template <int DP>
+__device__ __forceinline__ float dist_d_lower_bound(const Index& ix, uint32_t a, uint32_t b, int d) {
+  const int lane = threadIdx.x & 31;
+  float m0a[DP], m1a[DP], isa[DP], m0b[DP], m1b[DP], isb[DP], acc[DP];
+  load_stats<DP>(ix, a, m0a, m1a, isa);
+  load_stats<DP>(ix, b, m0b, m1b, isb);
+#pragma unroll
+  for (int f = 0; f < DP; ++f) acc[f] = 0.f;
+  const int segs = ix.w / 16;
+  for (int k = lane; k < segs; k += 32) {
+    float ua[DP], ub[DP];
+    load_row<DP>(ix.smT, int64_t(a) + 16 * k, ua);
+    load_row<DP>(ix.smT, int64_t(b) + 16 * k, ub);
+#pragma unroll
+    for (int f = 0; f < DP; ++f) {
+      const float za = ((ua[f] - m0a[f]) - m1a[f]) * isa[f];
+      const float zb = ((ub[f] - m0b[f]) - m1b[f]) * isb[f];
+      const float dd = za - zb;
+      acc[f] = fmaf(dd, dd, acc[f]);
+    }
+  }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1)
+#pragma unroll
+    for (int f = 0; f < DP; ++f) acc[f] += __shfl_xor_sync(0xffffffffu, acc[f], o);
+  float lb[DP];
+#pragma unroll
+  for (int f = 0; f < DP; ++f) lb[f] = f < ix.D ? sqrtf(16.f * acc[f]) : INFINITY;
+  return sum_d_smallest<DP>(lb, ix.D, d);
+}
+
+// One warp per candidate event (each warp a contiguous range of events):
+// distances; a pair with dist_d < tau is recorded (with its repetition) and
+// offered to the set of close pairs.
+// DM: dims held per lane (0 = any D); PM: the point-major copies (DP = DM)
+template <int DM, bool PM, bool LO>
+__global__ void __launch_bounds__(256)
+k_verify_events(Index ix, int d, HashSet hs, const Event* __restrict__ ev,
+                unsigned long long* __restrict__ counters, uint64_t ev_cap, float tau,
+                PairRec* __restrict__ rec, uint64_t rec_cap) {
+  const int lane = threadIdx.x & 31;
+  uint64_t cnt = counters[0];
+  if (cnt > ev_cap) cnt = ev_cap;
+  const uint64_t nw = uint64_t(gridDim.x) * (blockDim.x >> 5);
+  const uint64_t w = (blockIdx.x * uint64_t(blockDim.x) + threadIdx.x) >> 5;
+  const uint64_t q0 = cnt * w / nw, q1 = cnt * (w + 1) / nw;
+  for (uint64_t q = q0; q < q1; ++q) {
+    const Event e = ev[q];
+    if (PM && ix.smT) {
+      const float lb = dist_d_lower_bound<(PM ? DM : 4)>(ix, e.a, e.b, d);
+      if (lb > tau * (1.f + 1e-3f) + 1e-3f) {          // provably not below tau
+        if (lane == 0) atomicAdd(&counters[3], 1ull);
+        continue;
+      }
+    }
+    float dist[2];
+    if (PM) pair_distances_pm<(PM ? DM : 4), LO>(ix, e.a, e.b, dist);
+    else if (DM > 0) pair_distances_fast<(DM > 0 ? DM : 1)>(ix, e.a, e.b, dist);
+    else pair_distances<float>(ix, e.a, e.b, dist);
+    VerifyOut v = select_d<float>(dist, ix.D, d);
+    if (lane != 0) continue;
+    if (!(float(v.dist_d) < tau)) {
+      atomicAdd(&counters[4], 1ull);
       continue;
     }
-    line += " v" + std::to_string(v) + "=" + std::to_string(ms);
-    if (ms < best_ms) {
-      best_ms = ms;
-      best = v;
+    const unsigned long long pos = atomicAdd(&counters[1], 1ull);
+    if (pos < rec_cap) {
+      PairRec r;
+      r.a = e.a;
+      r.b = e.b;
+      r.j = e.j;
+      r.dist_d = float(v.dist_d);
+      r.dist_max = float(v.dist_max);
+      r.pad = 0;
+      r.dims = v.mask;
+      rec[pos] = r;
     }
-  }
-  cudaEventDestroy(e0);
-  cudaEventDestroy(e1);
-  {
-    std::lock_guard<std::mutex> g(tune_mu());
-    tune_map().emplace(key, best);
-  }
-  if (const char* t = std::getenv("MOMENTI_TRACE"); t && t[0] == '1')
-    std::fprintf(stderr, "momenti trace: sweep autotune dp=%d w=%d M=%lld ms:%s -> v%d\n", key.dp, ix.w,
-                 (long long)ix.M, line.c_str(), best);
-  return best;
-}
-
-// Column table of the statistics sweep: isT[b][f] = 1/sigma (0 for flat
-// windows, 1 for padding dims) and cflag[b] = 1 when some dim of window b
-// is flat or its column centring offset may be large against its sigma.
-// The centring constant of a diagonal is the float32 mean of a column
-// window b' in [b - kRowSub3, b] (the stage's first column), so b is marked
-// when sigma^2 <= 1e-4 (sigma^2 + max |mean(b') - mean(b)|^2) there, the
-// condition the rows kernels apply to the offset they actually carry.
-__global__ void k_col_prep(Index ix) {
-  const int64_t b = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
-  if (b >= ix.M) return;
-  float* tab = ix.isT ? ix.isT : ix.isW;
-  const int DP = ix.isT ? ix.Dp : ix.DW;
-  int u = 0;
-  for (int f = 0; f < DP; ++f) {
-    float is = 1.f;
-    if (f < ix.D) {
-      const int64_t o = int64_t(f) * ix.M;
-      is = ix.inv_sig[o + b];
-      const float mb = ix.mu_hi[o + b];
-      float dmax = 0.f;
-      for (int64_t q = b > kRowSub3 ? b - kRowSub3 : 0; q <= b; ++q)
-        dmax = fmaxf(dmax, fabsf(ix.mu_hi[o + q] - mb));
-      const double sg = ix.sig[o + b], v = sg * sg, dm = double(dmax);
-      u |= (is == 0.f) || !(v > 1e-4 * (v + dm * dm));
-    }
-    tab[b * DP + f] = is;
-  }
-  ix.cflag[b] = uint8_t(u);
-}
-
-}  // namespace
-
-cudaError_t launch_col_prep(const Index& ix, cudaStream_t s) {
-  if (!ix.isT && !ix.isW) return cudaSuccess;
-  MOMENTI_LAUNCH("col_prep", s, k_col_prep<<<unsigned((ix.M + 255) / 256), 256, 0, s>>>(ix));
-  return cudaGetLastError();
-}
-
-bool sweep_batchable(const Index& ix) {
-  return !ix.xW && sweep_variants(ix) > 0;
-}
-
-cudaError_t launch_allpairs_batch(const std::vector<SweepJob>& jobs, cudaStream_t s) {
-  if (jobs.empty()) return cudaSuccess;
-  for (const auto& j : jobs)
-    if (!sweep_batchable(j.ix)) return cudaErrorInvalidValue;
-  // items of every job, largest series first; one persistent launch per
-  // padded dimension count (the kernel's register and shared-memory shape)
-  std::vector<int> order(jobs.size());
-  for (size_t q = 0; q < jobs.size(); ++q) order[q] = int(q);
-  std::stable_sort(order.begin(), order.end(), [&](int x, int y) { return jobs[x].ix.M > jobs[y].ix.M; });
-  SweepJob* djobs = nullptr;
-  cudaError_t e = cudaMallocAsync(&djobs, jobs.size() * sizeof(SweepJob), s);
-  if (e != cudaSuccess) return e;
-  e = cudaMemcpyAsync(djobs, jobs.data(), jobs.size() * sizeof(SweepJob), cudaMemcpyHostToDevice, s);
-  for (int dp : {4, 8, 16}) {
-    std::vector<SweepItem> items;
-    for (int q : order) {
-      const Index& ix = jobs[q].ix;
-      if (ix.Dp != dp || ix.M - (ix.excl + 1) <= 0) continue;
-      const int64_t nbx = (ix.M + kSeg - 1) / kSeg;
-      const int64_t gy = (ix.M - (ix.excl + 1) + kDiagBlock - 1) / kDiagBlock;
-      for (int64_t by = 0; by < gy; ++by) {
-        const int64_t dlo = int64_t(ix.excl) + 1 + by * kDiagBlock;
-        for (int64_t bx = 0; bx < nbx && bx * kSeg < ix.M - dlo; ++bx)
-          items.push_back(SweepItem{uint32_t(q), uint32_t(bx), uint32_t(by)});
+    const uint64_t key = (uint64_t(e.a) << 32) | e.b;
+    uint64_t h = set_hash(key) & (hs.cap - 1);
+    for (int probe = 0; probe < kSetMaxProbe; ++probe) {
+      uint64_t cur = hs.keys[h];
+      if (cur == key) break;
+      if (cur == kSetEmpty) {
+        cur = atomicCAS(reinterpret_cast<unsigned long long*>(&hs.keys[h]), kSetEmpty, key);
+        if (cur == kSetEmpty) {
+          atomicAdd(&counters[2], 1ull);
+          break;
+        }
+        if (cur == key) break;
       }
+      h = (h + 1) & (hs.cap - 1);
     }
-    if (items.empty() || e != cudaSuccess) continue;
-    SweepItem* ditems = nullptr;
-    int* dnext = nullptr;
-    if ((e = cudaMallocAsync(&ditems, items.size() * sizeof(SweepItem), s)) != cudaSuccess) break;
-    if ((e = cudaMallocAsync(&dnext, sizeof(int), s)) != cudaSuccess) {
-      cudaFreeAsync(ditems, s);
-      break;
-    }
-    e = cudaMemcpyAsync(ditems, items.data(), items.size() * sizeof(SweepItem), cudaMemcpyHostToDevice, s);
-    if (e == cudaSuccess) e = cudaMemsetAsync(dnext, 0, sizeof(int), s);
-    const int per_sm = dp <= 8 ? 3 : 2;
-    const int64_t grid = std::min<int64_t>(int64_t(sm_count()) * per_sm, int64_t(items.size()));
-    const int nit = int(items.size());
-    if (e == cudaSuccess) {
-      if (dp == 4) {
-        const size_t smem = rows3_smem(4, kRowSub3);
-        e = allow_smem(reinterpret_cast<const void*>(k_allpairs_rows3_batch<4, kRowSub3, 3>), smem);
-        if (e == cudaSuccess)
-          MOMENTI_LAUNCH("allpairs_batch", s, k_allpairs_rows3_batch<4, kRowSub3, 3><<<unsigned(grid), kDiagBlock, smem, s>>>(djobs, ditems, nit, dnext));
-      } else if (dp == 8) {
-        const size_t smem = rows3_smem(8, kRowSub3);
-        e = allow_smem(reinterpret_cast<const void*>(k_allpairs_rows3_batch<8, kRowSub3, 3>), smem);
-        if (e == cudaSuccess)
-          MOMENTI_LAUNCH("allpairs_batch", s, k_allpairs_rows3_batch<8, kRowSub3, 3><<<unsigned(grid), kDiagBlock, smem, s>>>(djobs, ditems, nit, dnext));
-      } else {
-        const size_t smem = rows3_smem(16, kRowSub3 / 2);
-        e = allow_smem(reinterpret_cast<const void*>(k_allpairs_rows3_batch<16, kRowSub3 / 2, 2>), smem);
-        if (e == cudaSuccess)
-          MOMENTI_LAUNCH("allpairs_batch", s, k_allpairs_rows3_batch<16, kRowSub3 / 2, 2><<<unsigned(grid), kDiagBlock, smem, s>>>(djobs, ditems, nit, dnext));
-      }
-      if (e == cudaSuccess) e = cudaGetLastError();
-    }
-    cudaFreeAsync(ditems, s);
-    cudaFreeAsync(dnext, s);
   }
-  cudaFreeAsync(djobs, s);
-  return e;
 }
 
-bool rows2_usable(const Index& ix) {
-  return ix.xW && !ix.has_lo && (ix.DW == 32 || ix.DW == 64) &&
-         rows2_smem(ix.w, ix.DW) <= size_t(220) * 1024;
-}
-
-namespace {
-
-
-template <bool ROWMIN>
-cudaError_t allpairs_dispatch(const Index& ix, int d, float thr, const ApRec& rc, float* rowmin,
-                              cudaStream_t s) {
-  const int64_t ndiag = ix.M - (ix.excl + 1);
-  if (ndiag <= 0) return cudaSuccess;
-  if constexpr (!ROWMIN) {
-    if (sweep_variants(ix) > 0)
-      return sweep_launch(ix, sweep_variant(ix, d, rc, s), d, thr, rc, s, int64_t(1) << 40);
+__global__ void __launch_bounds__(256)
+k_verify_pairs(Index ix, int d, const uint64_t* __restrict__ pairs, int64_t m, int fp64,
+               double* __restrict__ per_dim, double* __restrict__ dist_d,
+               uint64_t* __restrict__ dims) {
+  const int lane = threadIdx.x & 31;
+  const int64_t nw = int64_t(gridDim.x) * (blockDim.x >> 5);
+  for (int64_t q = (blockIdx.x * int64_t(blockDim.x) + threadIdx.x) >> 5; q < m; q += nw) {
+    const uint32_t a = uint32_t(pairs[q] >> 32), b = uint32_t(pairs[q]);
+    VerifyOut v;
+    double dd[2];
+    if (fp64) {
+      double dist[2];
+      pair_distances<double>(ix, a, b, dist);
+      v = select_d<double>(dist, ix.D, d);
+      dd[0] = dist[0];
+      dd[1] = dist[1];
+    } else {
+      float dist[2];
+      pair_distances<float>(ix, a, b, dist);
+      v = select_d<float>(dist, ix.D, d);
+      dd[0] = dist[0];
+      dd[1] = dist[1];
+    }
+    if (per_dim) {
+      if (lane < ix.D) per_dim[q * ix.D + lane] = dd[0];
+      if (lane + 32 < ix.D) per_dim[q * ix.D + lane + 32] = dd[1];
+    }
+    if (lane == 0) {
+      if (dist_d) dist_d[q] = v.dist_d;
+      if (dims) dims[q] = v.mask;
+    }
   }
-  if (rows2_usable(ix)) {
-    if (ix.DW == 32) return rows2_dispatch<32, ROWMIN>(ix, d, thr, rc, rowmin, s);
-    if constexpr (ROWMIN) return launch_rows2_64_rowmin(ix, d, rowmin, s);
-    else return launch_rows2_64(ix, d, thr, rc, s, int64_t(1) << 40);
-  }
-  // every other form below needs a point-major copy or D <= 32
-  if (!ix.xT && ix.D > 32) return launch_wide64(ix, d, thr, rc, rowmin, ROWMIN, s);
-  const int64_t gy = (ndiag + kDiagBlock - 1) / kDiagBlock;
-  for (int64_t y0 = 0; y0 < gy; y0 += 65535) {
-  dim3 grid{unsigned((ix.M + kSeg - 1) / kSeg), unsigned(std::min<int64_t>(65535, gy - y0)), 1u};
-  if (ix.xT && ix.Dp == 4 && ix.has_lo)
-    MOMENTI_LAUNCH("allpairs", s, k_allpairs_pm<4, true, ROWMIN><<<grid, kDiagBlock, 0, s>>>(ix, d, thr, rc, rowmin, y0));
-  else if (ix.xT && ix.Dp == 4 && rows_fit(ix.w, 4)) {
-    const size_t smem = rows_smem(ix.w, 4);
-    cudaError_t e = allow_smem(reinterpret_cast<const void*>(k_allpairs_rows<4, ROWMIN>), smem);
-    if (e != cudaSuccess) return e;
-    MOMENTI_LAUNCH("allpairs", s, k_allpairs_rows<4, ROWMIN><<<grid, kDiagBlock, smem, s>>>(ix, d, thr, rc, rowmin, y0));
-  }
-  else if (ix.xT && ix.Dp == 8 && ix.has_lo)
-    MOMENTI_LAUNCH("allpairs", s, k_allpairs_pm<8, true, ROWMIN><<<grid, kDiagBlock, 0, s>>>(ix, d, thr, rc, rowmin, y0));
-  else if (ix.xT && ix.Dp == 8 && rows_fit(ix.w, 8)) {
-    const size_t smem = rows_smem(ix.w, 8);
-    cudaError_t e = allow_smem(reinterpret_cast<const void*>(k_allpairs_rows<8, ROWMIN>), smem);
-    if (e != cudaSuccess) return e;
-    MOMENTI_LAUNCH("allpairs", s, k_allpairs_rows<8, ROWMIN><<<grid, kDiagBlock, smem, s>>>(ix, d, thr, rc, rowmin, y0));
-  }
-  else if (ix.xT && ix.Dp == 16 && ix.has_lo)
-    MOMENTI_LAUNCH("allpairs", s, k_allpairs_pm<16, true, ROWMIN><<<grid, kDiagBlock, 0, s>>>(ix, d, thr, rc, rowmin, y0));
-  else if (ix.xT && ix.Dp == 16 && rows_fit(ix.w, 16)) {
-    const size_t smem = rows_smem(ix.w, 16);
-    cudaError_t e = allow_smem(reinterpret_cast<const void*>(k_allpairs_rows<16, ROWMIN>), smem);
-    if (e != cudaSuccess) return e;
-    MOMENTI_LAUNCH("allpairs", s, k_allpairs_rows<16, ROWMIN><<<grid, kDiagBlock, smem, s>>>(ix, d, thr, rc, rowmin, y0));
-  }
-  else if (ix.D <= 16)
-    MOMENTI_LAUNCH("allpairs", s, k_allpairs<16, ROWMIN><<<grid, kDiagBlock, 0, s>>>(ix, d, thr, rc, rowmin, y0));
-  else {
-    const size_t smem = size_t(32) * (kDiagBlock + 1) * sizeof(float);
-    cudaError_t e = allow_smem(reinterpret_cast<const void*>(k_allpairs_wide<32, ROWMIN>), smem);
-    if (e != cudaSuccess) return e;
-    MOMENTI_LAUNCH("allpairs", s, k_allpairs_wide<32, ROWMIN><<<grid, kDiagBlock, smem, s>>>(ix, d, thr, rc, rowmin, y0));
-  }
-  }
-  return cudaGetLastError();
 }
 
 }  // namespace
@@ -384,14 +413,6 @@ cudaError_t launch_select_pairs(const uint64_t* pairs, const float* dd, uint64_t
   if (g > sm_count() * 8) g = sm_count() * 8;
   MOMENTI_LAUNCH("select_pairs", s, k_select_pairs<<<unsigned(g), 256, 0, s>>>(pairs, dd, m, lo, hi, out, count));
   return cudaGetLastError();
-}
-
-cudaError_t launch_allpairs(const Index& ix, int d, float thr, const ApRec& rc, cudaStream_t s) {
-  return allpairs_dispatch<false>(ix, d, thr, rc, nullptr, s);
-}
-
-cudaError_t launch_allpairs_rowmin(const Index& ix, int d, float* rowmin, cudaStream_t s) {
-  return allpairs_dispatch<true>(ix, d, 0.f, ApRec{}, rowmin, s);
 }
 
 }  // namespace momenti

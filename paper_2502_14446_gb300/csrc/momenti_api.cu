@@ -220,8 +220,7 @@ struct SearchState {
 }  // namespace
 
 // The batching form's sweep service.  The workers of momenti_topk_batch
-// hand it the recording sweeps of their exact paths (batchable indexes:
-// float32, D <= 16).  Once every worker still running is waiting here, or
+// hand it the recording sweeps of their exact paths.  Once every worker still running is waiting here, or
 // the oldest request has waited 2 ms, the pending sweeps run together in
 // one persistent launch on the service's stream, ordered after what each
 // requester queued on its own stream and before its next work there.
@@ -234,9 +233,9 @@ class SweepBatcher {
   SweepBatcher(const SweepBatcher&) = delete;
   SweepBatcher& operator=(const SweepBatcher&) = delete;
 
-  cudaError_t sweep(const Index& ix, int d, float thr, const ApRec& rc, cudaStream_t s) {
+  cudaError_t sweep(const SweepView& v, int d, float thr, const ApRec& rc, cudaStream_t s) {
     Req r;
-    r.job.ix = ix;
+    r.job.v = v;
     r.job.rc = rc;
     r.job.thr = thr;
     r.job.d = d;
@@ -294,7 +293,7 @@ class SweepBatcher {
         if (e == cudaSuccess) e = cudaStreamWaitEvent(stream_, ev, 0);
         jobs.push_back(q->job);
       }
-      if (e == cudaSuccess) e = launch_allpairs_batch(jobs, stream_);
+      if (e == cudaSuccess) e = launch_allpairs_batch(std::move(jobs), stream_);
       // each requester's next work follows the launch
       if (e == cudaSuccess) e = cudaEventRecord(ev, stream_);
       for (Req* q : batch)
@@ -434,6 +433,19 @@ cudaError_t pool_malloc(T** ptr, size_t bytes, cudaStream_t s) {
   return cudaMallocFromPoolAsync(reinterpret_cast<void**>(ptr), std::max<size_t>(bytes, 16), pool, s);
 }
 
+// A transient buffer of the library pool, returned when it goes out of
+// scope (queued on its stream).
+struct PoolBuf {
+  void* p = nullptr;
+  cudaStream_t s;
+  explicit PoolBuf(cudaStream_t st) : s(st) {}
+  PoolBuf(const PoolBuf&) = delete;
+  PoolBuf& operator=(const PoolBuf&) = delete;
+  ~PoolBuf() {
+    if (p) cudaFreeAsync(p, s);
+  }
+};
+
 template <typename T>
 cudaError_t dalloc(momenti_handle* h, T** ptr, size_t count) {
   size_t bytes = std::max<size_t>(count * sizeof(T), 16);
@@ -504,12 +516,16 @@ int exact_sweeps(const Index& ix, bool top_full) {
   return large ? 2 : 4;
 }
 
+// The costs per pair are not those of the present sweep, which is several
+// times faster: they decide the level at which the exact path takes over,
+// and with it which searches end by STOP (with a miss bound) and which in
+// the exact path, so they stay as they are.
 double predict_exact_ms(const Index& ix, int passes) {
   double ps_pair;                                  // all-pairs kernel, per pair
-  if (ix.xT && !ix.has_lo && ix.Dp == 4) ps_pair = 5.0;
-  else if (ix.xT && !ix.has_lo && ix.Dp == 8) ps_pair = 7.5;
-  else if (ix.xT && !ix.has_lo && ix.Dp == 16) ps_pair = 40.0;
-  else if (ix.xW && rows2_usable(ix)) ps_pair = 1.5 * double(ix.DW);
+  if (!ix.has_lo && ix.D <= 4) ps_pair = 5.0;
+  else if (!ix.has_lo && ix.D <= 8) ps_pair = 7.5;
+  else if (!ix.has_lo && ix.D <= 16) ps_pair = 40.0;
+  else if (!ix.has_lo) ps_pair = 1.5 * (ix.D <= 32 ? 32.0 : 64.0);
   else if (ix.D <= 32) ps_pair = 8.0 * double(ix.D);
   else ps_pair = 31.0 * double(ix.D);
   const double pairs = 0.5 * double(ix.M) * double(ix.M);
@@ -622,62 +638,12 @@ int finalize(momenti_handle* h, int d, std::vector<PoolEntry> cand, momenti_moti
   return MOMENTI_OK;
 }
 
-// Exact all-pairs top-k (the final fallback of Algorithm 1).  tau0 <= 0: derive the
-// first threshold from per-window nearest distances.
+// Exact all-pairs top-k (the final fallback of Algorithm 1).  tau0: TOP's
+// k-th with some slack, or <= 0 when TOP is not full.
 int exact_path(momenti_handle* h, int d, double tau0, momenti_motif* out, int32_t* n_out,
                double* max_err) {
   Index& ix = h->ix;
   const int k = h->p.k;
-  // First threshold: TOP's k-th (tau0), else 1.2 x the 2k-th smallest row
-  // minimum of spaced windows.  On a large series (M^2 D > 4e11) a loose
-  // threshold costs a sweep in which most pairs pass the filters, and the
-  // row-minima sweep evaluates every pair in full: there, when TOP holds
-  // only background pairs (its k-th above a quarter of the largest possible
-  // dist_d, 2 d sqrt(w)) or is not full, the slices start at 5% of that
-  // largest value and double.  Any start gives the same exact result.
-  const double dmax_all = 2.0 * double(d) * std::sqrt(double(ix.w));
-  const double tau_low = 0.05 * dmax_all;
-  const bool large = double(ix.M) * double(ix.M) * double(ix.D) > 4e11;
-  double tau = tau0;
-  if (large && (!(tau > 0) || tau > 0.25 * dmax_all)) tau = tau > 0 ? std::min(tau, tau_low) : tau_low;
-  if (!(tau > 0)) {
-    float* rowmin = nullptr;
-    CK(pool_malloc(&rowmin, ix.M * 4, h->stream));
-    CK(cudaMemsetAsync(rowmin, 0x7f, ix.M * 4, h->stream));
-    const auto tr0 = std::chrono::steady_clock::now();
-    CK(launch_allpairs_rowmin(ix, d, rowmin, h->stream));
-    std::vector<float> rm(ix.M);
-    CK(cudaMemcpyAsync(rm.data(), rowmin, ix.M * 4, cudaMemcpyDeviceToHost, h->stream));
-    CK(cudaFreeAsync(rowmin, h->stream));
-    CK(cudaStreamSynchronize(h->stream));
-    // 2k-th smallest nearest distance among windows spaced more than eps
-    std::vector<std::pair<float, int64_t>> v;
-    for (int64_t a = 0; a < ix.M; ++a)
-      if (std::isfinite(rm[a])) v.push_back({rm[a], a});
-    std::sort(v.begin(), v.end());
-    std::vector<int64_t> picked;
-    double val = 0;
-    for (auto& pr : v) {
-      bool ok = true;
-      for (int64_t q : picked)
-        if (std::llabs(q - pr.second) <= ix.excl) { ok = false; break; }
-      if (!ok) continue;
-      picked.push_back(pr.second);
-      val = pr.first;
-      if (int(picked.size()) >= 2 * k) break;
-    }
-    if (picked.empty()) {
-      *n_out = 0;
-      return MOMENTI_OK;
-    }
-    tau = std::max(val * 1.2, 1e-3);
-    if (const char* t1 = std::getenv("MOMENTI_TRACE"); t1 && t1[0] == '1')
-      std::fprintf(stderr, "momenti trace: exact row minima ms=%.1f\n",
-                   std::chrono::duration<double, std::milli>(std::chrono::steady_clock::now() - tr0).count());
-  }
-  if (const char* t0 = std::getenv("MOMENTI_TRACE"); t0 && t0[0] == '1')
-    std::fprintf(stderr, "momenti trace: exact tau=%.5g (%s)\n", tau,
-                 tau == tau0 ? "from TOP" : (tau == tau_low ? "low start" : "from row minima"));
   const auto te0 = std::chrono::steady_clock::now();
   // Pairs are taken in slices of their approximate dist_d (float32 Pearson
   // form, within 1% + 0.01 of the exact value): each all-pairs sweep records
@@ -728,18 +694,25 @@ int exact_path(momenti_handle* h, int d, double tau0, momenti_motif* out, int32_
   // no pair has an approximate distance above this
   const float all_edge = float(2.0 * std::sqrt(double(ix.w)) * d * 1.01 + 0.02);
   constexpr int64_t kBatch = int64_t(1) << 13;   // pairs verified per batch (smallest first)
+  if (ix.M <= int64_t(ix.excl) + 1) {              // no non-trivial pair
+    *n_out = 0;
+    return MOMENTI_OK;
+  }
   size_t free_b = 0, total_b = 0;
   CK(cudaMemGetInfo(&free_b, &total_b));
   const uint64_t cap_max = std::max<uint64_t>(uint64_t(1) << 22,
                                               std::min<uint64_t>(uint64_t(1) << 30, free_b / 4 / 12));
   uint64_t cap = std::min<uint64_t>(uint64_t(1) << 24, cap_max);
-  float lo = -1.f;
-  float hi = std::min(float(tau) * 1.01f + 1e-2f, all_edge);
   uint64_t* dout = nullptr;
   float* dval = nullptr;
   unsigned long long* dcnt = nullptr;
   uint32_t* dhist = nullptr;
   uint64_t* dsel = nullptr;
+  // the sweep's table of this index, for the duration of the exact path
+  PoolBuf table(h->stream);
+  CK(pool_malloc(&table.p, sweep_table_bytes(ix), h->stream));
+  SweepView view;
+  CK(launch_sweep_table(ix, table.p, &view, h->stream));
   auto release = [&]() {
     if (dout) cudaFreeAsync(dout, h->stream);
     if (dval) cudaFreeAsync(dval, h->stream);
@@ -748,9 +721,95 @@ int exact_path(momenti_handle* h, int d, double tau0, momenti_motif* out, int32_
     dval = nullptr;
     dsel = nullptr;
   };
-  CK(pool_malloc(&dcnt, 8, h->stream));
+  CK(pool_malloc(&dcnt, 24, h->stream));           // pairs; a sample's groups, and those run twice
   CK(pool_malloc(&dhist, kApBins * 4, h->stream));
   std::vector<uint32_t> hist(kApBins);
+  // First edge.  A pair is worth recording if it can be among the k motifs:
+  // TOP's k-th (tau0) bounds them when TOP is full, but on background pairs
+  // it is loose, and a loose edge sends most of the sweep through its slow
+  // branch (three times the time on the plain workload at TOP's k-th).  The
+  // edge is set where about `want` pairs lie below it: the k motifs, each
+  // with the neighbours of its windows, which are within reach of the edge
+  // too (about w^2 / 256 of them where the distance is flat), found from a
+  // sample: first about 2^20 pairs of all distances, then, where `want`
+  // pairs are fewer than that sample resolves, a fraction holding about 24
+  // of them, swept below the first sample's edge (small blocks: close pairs
+  // come in clusters).  Where even that edge
+  // sends four groups of rows out of five through the slow branch (many
+  // dimensions, or a d whose background distances are close), a sweep at 5%
+  // of the largest possible distance costs a quarter of one at the edge and
+  // holds the motifs whenever they stand out, so it goes first (the wide
+  // workload: 149 ms against 570).  Any edge gives the same result; one that
+  // holds fewer than k motifs is followed by the next.
+  const double n_pairs = 0.5 * double(ix.M - ix.excl) * double(ix.M - ix.excl - 1);
+  const double want = 2048.0 + double(k) * std::max(64.0, double(ix.w) * double(ix.w) / 256.0);
+  const float hi_top = tau0 > 0 ? std::min(float(tau0) * 1.01f + 1e-2f, all_edge) : all_edge;
+  float hi = hi_top, hi_next = 0.f;                // the first edge and the one after it (0: twice as far)
+  float lo = -1.f;
+  unsigned long long groups[2] = {0, 0};
+  // samples below `edge` and returns the edges holding want_a and want_b pairs of all
+  auto sample = [&](float edge, double fraction, int seg, double want_a, double want_b, float* ea, float* eb) -> int {
+    CK(cudaMemsetAsync(dcnt, 0, 24, h->stream));
+    CK(cudaMemsetAsync(dhist, 0, kApBins * 4, h->stream));
+    ApRec ar;
+    ar.count = dcnt;
+    ar.hist = dhist;
+    ar.lo = -1.f;
+    ar.hscale = float(kApBins) / (edge + 1.f);
+    double held = 0.0;
+    CK(launch_allpairs_sample(view, d, edge, ar, fraction, seg, &held, dcnt + 1, h->stream));
+    CK(cudaMemcpyAsync(groups, dcnt + 1, 16, cudaMemcpyDeviceToHost, h->stream));
+    CK(cudaMemcpyAsync(hist.data(), dhist, kApBins * 4, cudaMemcpyDeviceToHost, h->stream));
+    CK(cudaStreamSynchronize(h->stream));
+    const double scale = held > 0.0 ? n_pairs / held : 0.0;
+    double run = 0.0;
+    *ea = *eb = edge;
+    bool have_a = false;
+    for (int b = 0; b < kApBins; ++b) {
+      run += scale * double(hist[size_t(b)]);
+      const float up = -1.f + (edge + 1.f) * float(b + 1) / float(kApBins);
+      if (!have_a && run >= want_a) {
+        *ea = up;
+        have_a = true;
+      }
+      if (run >= want_b) {
+        *eb = up;
+        break;
+      }
+    }
+    return MOMENTI_OK;
+  };
+  const double kSample = double(1 << 20), sweep_work = n_pairs * double(ix.D);
+  if (n_pairs > 0.25 * kSample && (!(tau0 > 0) || sweep_work > 2e8)) {
+    float edge = hi_top;
+    const bool fine = want / n_pairs * kSample < 32.0;    // too few of them in the first sample
+    if (!(tau0 > 0) || !fine) {
+      float ea = 0.f, eb = 0.f;
+      const double w1 = fine ? 32.0 * n_pairs / kSample : want;
+      const int r = sample(all_edge, std::min(1.0, kSample / n_pairs), 8, w1, 16.0 * want, &ea, &eb);
+      if (r != MOMENTI_OK) return r;
+      edge = std::min(hi_top, ea);
+      if (!fine) {
+        hi = edge;
+        hi_next = std::min(hi_top, eb);
+      }
+    }
+    if (fine) {
+      float ea = 0.f, eb = 0.f;
+      const int r = sample(edge, std::min(1.0 / 32.0, 24.0 / want), 32, want, 16.0 * want, &ea, &eb);
+      if (r != MOMENTI_OK) return r;
+      hi = std::min(edge, ea);
+      hi_next = std::min(edge, eb);
+    }
+  }
+  const float far = float(2.0 * std::sqrt(double(ix.w)) * d), low = 0.05f * far;
+  if (groups[1] * 5 > groups[0] * 4 && hi > 2.f * low && (!(tau0 > 0) || float(tau0) > 0.25f * far)) {
+    hi_next = hi;
+    hi = low;
+  }
+  if (trace)
+    std::fprintf(stderr, "momenti trace: exact edge=%.5g next=%.5g top=%.5g ms=%.2f\n", double(hi), double(hi_next),
+                 double(tau0), std::chrono::duration<double, std::milli>(std::chrono::steady_clock::now() - te0).count());
   int rc = MOMENTI_ERR_OVERFLOW;
   for (int pass = 0; pass < 64; ++pass) {
     if (!dout) {
@@ -768,10 +827,10 @@ int exact_path(momenti_handle* h, int d, double tau0, momenti_motif* out, int32_
     ar.lo = lo;
     ar.hscale = float(kApBins) / (hi - lo);
     const auto tp0 = std::chrono::steady_clock::now();
-    if (h->batcher && sweep_batchable(ix))
-      CK(h->batcher->sweep(ix, d, hi, ar, h->stream));
+    if (h->batcher)
+      CK(h->batcher->sweep(view, d, hi, ar, h->stream));
     else
-      CK(launch_allpairs(ix, d, hi, ar, h->stream));
+      CK(launch_allpairs(view, d, hi, ar, h->stream));
     unsigned long long cnt = 0;
     CK(cudaMemcpyAsync(&cnt, dcnt, 8, cudaMemcpyDeviceToHost, h->stream));
     CK(cudaMemcpyAsync(hist.data(), dhist, kApBins * 4, cudaMemcpyDeviceToHost, h->stream));
@@ -828,7 +887,10 @@ int exact_path(momenti_handle* h, int d, double tau0, momenti_motif* out, int32_
       break;
     }
     lo = hi;
-    hi = std::min(2.f * hi + 1e-2f, all_edge);
+    // the next sample edge, TOP's k-th (which holds all k), then twice as far
+    if (hi_next > hi * 1.01f) hi = hi_next;
+    else if (hi_top > hi && tau0 > 0) hi = hi_top;
+    else hi = std::min(2.f * hi + 1e-2f, all_edge);
   }
   cudaFreeAsync(dcnt, h->stream);
   cudaFreeAsync(dhist, h->stream);
@@ -1012,20 +1074,10 @@ static int hash_all_impl(momenti_handle* h, const void* series, int32_t dtype, i
     const int N = (tens ? 2 * isqrt(L) : L) * kRepStride;
     CK(dalloc(h, &ix.xs_hi, size_t(D) * n));
     if (ix.has_lo) CK(dalloc(h, &ix.xs_lo, size_t(D) * n));
-    if (D > 16 && dtype == MOMENTI_F32) {       // the row-staged sweep of wide series
-      ix.DW = D <= 32 ? 32 : 64;
-      CK(dalloc(h, &ix.xW, size_t(ix.DW) * n));
-      CK(dalloc(h, &ix.isW, size_t(ix.DW) * M));
-      CK(dalloc(h, &ix.cflag, size_t(M)));
-    }
     if (D <= 16) {
       ix.Dp = D <= 4 ? 4 : (D <= 8 ? 8 : 16);
       CK(dalloc(h, &ix.xT, size_t(ix.Dp) * n));
       CK(dalloc(h, &ix.stT, size_t(3) * ix.Dp * M));
-      if (!ix.has_lo) {
-        CK(dalloc(h, &ix.isT, size_t(ix.Dp) * M));
-        CK(dalloc(h, &ix.cflag, size_t(M)));
-      }
       if (ix.has_lo) CK(dalloc(h, &ix.xlT, size_t(ix.Dp) * n));
       if (w >= 32) {
         CK(dalloc(h, &ix.smT, size_t(ix.Dp) * n));
@@ -1130,7 +1182,6 @@ static int hash_all_impl(momenti_handle* h, const void* series, int32_t dtype, i
   if (staging) CK(cudaFreeAsync(staging, s));
   CK(launch_window_stats(ix, s));
   CK(launch_stats_point_major(ix, s));
-  CK(launch_col_prep(ix, s));
 
   // ---- hash functions ----
   int L_src = hx.L;
