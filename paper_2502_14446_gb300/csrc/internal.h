@@ -133,7 +133,7 @@ struct SortItem {
 // already in order).
 struct SortChunk {
   uint32_t seg, start, size;
-  uint8_t lcp0, buf, equal, pad;
+  uint8_t lcp0, buf, equal, t;   // t: the hash value the range was partitioned by
 };
 struct SortCaps {
   int64_t item_cap = 0, tile_cap = 0, chunk_cap = 0;

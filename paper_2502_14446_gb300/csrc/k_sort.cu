@@ -8,8 +8,7 @@
 // never moves an entry out of its item, so every entry lands in its final
 // position's bucket.  Buckets of at most kLocalMax entries are packed, in
 // order, into chunks that one CTA then sorts completely in shared memory
-// (a stable least-significant-digit sort over the bytes that vary inside
-// the chunk); larger buckets become the items of level t + 1.  After level
+// by (key, window); larger buckets become the items of level t + 1.  After level
 // K - 1 every bucket holds equal keys and is already in order.  On the
 // hash strings of z-normalised windows one level usually suffices: the
 // largest bucket of the first hash value holds a few percent of the
@@ -43,10 +42,13 @@ constexpr int kWarps = kThreads / 32;
 constexpr int kWarpSpan = kTile / kWarps;      // 256 entries per warp
 constexpr int kRounds = kWarpSpan / 32;        // 8
 
-constexpr int kLocalThreads = 128;
+constexpr int kLocalThreads = 256;
+constexpr int kLocalBlocks = 4;                              // CTAs per SM (64 registers a thread)
 constexpr int kLocalWarps = kLocalThreads / 32;
-constexpr int kLocalRounds = kSortLocalMax / (kLocalWarps * 32);   // 16
-static_assert(kSortLocalMax <= 65536, "chunk ranks travel as 16-bit values");
+constexpr int kLocalItems = kSortLocalMax / kLocalThreads;   // 8 per thread
+constexpr int kBinBits = 11;                                 // bins of a chunk: about one per entry
+constexpr int kBins = 1 << kBinBits;
+static_assert(kBins % kLocalThreads == 0 && kSortLocalMax <= 4096, "bin and rank travel in one word");
 
 // counters: [2 t] items and [2 t + 1] tiles of level t (t = 0..8), then
 constexpr int kCntChunks = 20;   // chunks for the shared-memory sort
@@ -154,144 +156,147 @@ __global__ void __launch_bounds__(kThreads) k_sort_hist(Level lv) {
       if (p < end) atomicAdd(&h[lv.digit(k[r])], 1u);
     }
     __syncthreads();
-    const uint32_t nti = ntiles(it.size);
-    uint32_t* out = lv.hist + int64_t(it.hist0) * 256;
-    for (int d = threadIdx.x; d < 256; d += kThreads) out[int64_t(d) * nti + tt] = h[d];
+    uint32_t* out = lv.hist + (int64_t(it.hist0) + tt) * 256;
+    for (int d = threadIdx.x; d < 256; d += kThreads) out[d] = h[d];
     __syncthreads();
   }
 }
 
-// Exclusive scan over the digit-major (digit, tile) counts of one item, then
-// the item's buckets become chunks (at most kSortLocalMax entries, packed in
-// order) or items of the next level.
+// Exclusive scan over the (digit, tile) counts of one item, digit-major (a
+// thread per digit walks the tiles, whose rows of 256 counts it reads
+// together with its neighbours), then the item's buckets become chunks (at
+// most kSortLocalMax entries, packed greedily in digit order) or items of
+// the next level.  The greedy packing is a chain of "next chunk starts at
+// digit e" steps: every thread finds its e by a binary search in the bucket
+// starts, one thread follows the chain (one step per chunk), and all write
+// the chunks.  (One thread walking the 256 digits twice took 8 us of a
+// block: 15.5 ms of a wide index's 118 ms of sorting.)
 __global__ void __launch_bounds__(256) k_sort_scan(Level lv) {
-  __shared__ uint32_t tot[256], bstart[256];
+  __shared__ uint32_t pre[257];              // bucket starts, relative to the item
+  __shared__ uint32_t wsum[8], bigm[8];      // per warp: total, mask of large buckets
+  __shared__ uint16_t nxt[256];
+  __shared__ uint8_t head[256];              // a chunk or item starts at this digit
+  __shared__ uint32_t chunk0;
   const uint32_t ni = min(lv.cnt[2 * lv.t], lv.item_cap);
-  const int d = threadIdx.x;
+  const int d = threadIdx.x, lane = d & 31, warp = d >> 5;
+  const bool last_level = lv.t + 1 >= lv.K;
   for (uint32_t item = blockIdx.x; item < ni; item += gridDim.x) {
     const SortItem it = lv.items[item];
     const uint32_t tiles = ntiles(it.size);
     if (it.seg >= uint32_t(lv.segs) || int64_t(it.start) + it.size > lv.M ||
         int64_t(it.hist0) + tiles > int64_t(lv.tile_cap))
       continue;                                   // only after an overflow
-    uint32_t* hs = lv.hist + int64_t(it.hist0) * 256 + int64_t(d) * tiles;
-    uint32_t s = 0;
-    uint32_t t0 = 0;
+    uint32_t* hs = lv.hist + int64_t(it.hist0) * 256 + d;
+    uint32_t s = 0, t0 = 0;
     for (; t0 + 8 <= tiles; t0 += 8) {          // eight independent loads in flight
       uint32_t c[8];
 #pragma unroll
-      for (int q = 0; q < 8; ++q) c[q] = hs[t0 + q];
+      for (int q = 0; q < 8; ++q) c[q] = hs[(t0 + q) * 256];
 #pragma unroll
       for (int q = 0; q < 8; ++q) s += c[q];
     }
-    for (; t0 < tiles; ++t0) s += hs[t0];
-    tot[d] = s;
-    bstart[d] = s;
-    __syncthreads();
-    // Hillis-Steele inclusive scan of the 256 digit totals
-    for (int off = 1; off < 256; off <<= 1) {
-      uint32_t v = d >= off ? bstart[d - off] : 0u;
-      __syncthreads();
-      bstart[d] += v;
-      __syncthreads();
+    for (; t0 < tiles; ++t0) s += hs[t0 * 256];
+    // exclusive scan of the 256 digit totals
+    uint32_t incl = s;
+    for (int o = 1; o < 32; o <<= 1) {
+      const uint32_t u = __shfl_up_sync(0xffffffffu, incl, o);
+      if (lane >= o) incl += u;
     }
-    uint32_t run = bstart[d] - s;   // exclusive, relative to the item's start
+    const bool big = s > uint32_t(kSortLocalMax);
+    const uint32_t bm = __ballot_sync(0xffffffffu, big);
+    if (lane == 31) {
+      wsum[warp] = incl;
+      bigm[warp] = bm;
+    }
+    head[d] = 0;
     __syncthreads();
-    bstart[d] = run;
-    uint32_t t1 = 0;
-    for (; t1 + 8 <= tiles; t1 += 8) {
+    uint32_t before = 0;
+#pragma unroll
+    for (int q = 0; q < 8; ++q) before += q < warp ? wsum[q] : 0u;
+    const uint32_t start = before + incl - s;
+    pre[d] = start;
+    if (d == 255) pre[256] = start + s;
+    uint32_t run = start;
+    t0 = 0;
+    for (; t0 + 8 <= tiles; t0 += 8) {
       uint32_t c[8];
 #pragma unroll
-      for (int q = 0; q < 8; ++q) c[q] = hs[t1 + q];
+      for (int q = 0; q < 8; ++q) c[q] = hs[(t0 + q) * 256];
 #pragma unroll
       for (int q = 0; q < 8; ++q) {
-        hs[t1 + q] = run;
+        hs[(t0 + q) * 256] = run;
         run += c[q];
       }
     }
-    for (; t1 < tiles; ++t1) {
-      uint32_t c = hs[t1];
-      hs[t1] = run;
+    for (; t0 < tiles; ++t0) {
+      const uint32_t c = hs[t0 * 256];
+      hs[t0 * 256] = run;
       run += c;
     }
     __syncthreads();
+    // where the chunk that starts at digit d ends: before the next large
+    // bucket, and while at most kSortLocalMax entries are in it
+    int e = d + 1;
+    if (!big) {
+      int stop = 256;
+      for (int q = 7; q >= warp; --q) {
+        const uint32_t m = q == warp ? bigm[q] & ~((1u << lane) - 1u) : bigm[q];
+        if (m) stop = q * 32 + __ffs(m) - 1;
+      }
+      int hi = stop;
+      while (e < hi) {
+        const int mid = (e + hi + 1) >> 1;
+        if (pre[mid] - start <= uint32_t(kSortLocalMax)) e = mid;
+        else hi = mid - 1;
+      }
+    }
+    nxt[d] = uint16_t(e);
+    __syncthreads();
+    if (d == 0)
+      for (int g = 0; g < 256; g = nxt[g]) head[g] = 1;
+    __syncthreads();
+    const uint32_t size = pre[e] - start;
+    const bool lead = head[d] != 0 && size > 0;
+    const bool is_item = lead && big && !last_level;
+    const bool is_chunk = lead && !is_item;
+    // a bucket's first entry shares t hash values with its predecessor (the
+    // item's own first entry keeps the item's count)
+    const uint32_t l0 = start == 0 ? it.lcp0 : uint32_t(lv.t);
+    const uint32_t cm = __ballot_sync(0xffffffffu, is_chunk);
+    if (lane == 0) wsum[warp] = __popc(cm);
+    __syncthreads();
     if (d == 0) {
-      // classification, in digit order: a bucket's first entry shares t
-      // hash values with its predecessor (the item's own first entry keeps
-      // the item's count).  Two walks over the digits: the first counts the
-      // chunks and items this item makes, so that one atomic reserves their
-      // slots; the second writes them.
-      const bool last_level = lv.t + 1 >= lv.K;
-      uint32_t n_chunks = 0, n_items = 0, n_tiles = 0, chunk0 = 0, item0 = 0, tile0 = 0;
-      for (int pass = 0; pass < 2; ++pass) {
-        uint32_t nch = 0, nit = 0, ntl = 0;
-        uint32_t c_start = 0, c_size = 0, c_lcp = 0;
-        bool open = false, first = true;
-        auto emit = [&](uint32_t st, uint32_t sz, uint32_t l0, uint32_t equal) {
-          if (pass == 1) {
-            const uint32_t slot = chunk0 + nch;
-            if (slot < lv.chunk_cap) {
-              SortChunk ch;
-              ch.seg = it.seg;
-              ch.start = st;
-              ch.size = sz;
-              ch.lcp0 = uint8_t(l0);
-              ch.buf = uint8_t(lv.t & 1);
-              ch.equal = uint8_t(equal);
-              ch.pad = 0;
-              lv.chunks[slot] = ch;
-            } else {
-              lv.cnt[kCntOverflow] = 1u;
-            }
-          }
-          ++nch;
-        };
-        for (int g = 0; g < 256; ++g) {
-          const uint32_t sz = tot[g];
-          if (!sz) continue;
-          const uint32_t l0 = first ? it.lcp0 : uint32_t(lv.t);
-          first = false;
-          const uint32_t st = it.start + bstart[g];
-          if (sz > uint32_t(kSortLocalMax)) {
-            if (open) emit(c_start, c_size, c_lcp, 0u);
-            open = false;
-            if (last_level) {
-              emit(st, sz, l0, 1u);            // equal keys: already in order
-            } else {
-              const uint32_t nt = ntiles(sz);
-              if (pass == 1) {
-                const uint32_t slot = item0 + nit, tb = tile0 + ntl;
-                if (slot < lv.item_cap && tb + nt <= lv.tile_cap) {
-                  lv.items_next[slot] = SortItem{it.seg, st, sz, tb, l0, {0u, 0u, 0u}};
-                  for (uint32_t q = 0; q < nt; ++q) lv.tile_next[tb + q] = (uint64_t(q) << 32) | slot;
-                } else {
-                  lv.cnt[kCntOverflow] = 1u;
-                }
-              }
-              ++nit;
-              ntl += nt;
-            }
-          } else if (open && c_size + sz <= uint32_t(kSortLocalMax)) {
-            c_size += sz;
-          } else {
-            if (open) emit(c_start, c_size, c_lcp, 0u);
-            open = true;
-            c_start = st;
-            c_size = sz;
-            c_lcp = l0;
-          }
-        }
-        if (open) emit(c_start, c_size, c_lcp, 0u);
-        if (pass == 0) {
-          n_chunks = nch;
-          n_items = nit;
-          n_tiles = ntl;
-          if (n_chunks) chunk0 = atomicAdd(&lv.cnt[kCntChunks], n_chunks);
-          if (n_items) {
-            item0 = atomicAdd(&lv.cnt[2 * (lv.t + 1)], n_items);
-            tile0 = atomicAdd(&lv.cnt[2 * (lv.t + 1) + 1], n_tiles);
-          }
-        }
+      uint32_t n = 0;
+      for (int q = 0; q < 8; ++q) n += wsum[q];
+      chunk0 = n ? atomicAdd(&lv.cnt[kCntChunks], n) : 0u;
+    }
+    __syncthreads();
+    if (is_chunk) {
+      uint32_t slot = chunk0 + __popc(cm & ((1u << lane) - 1u));
+      for (int q = 0; q < warp; ++q) slot += wsum[q];
+      if (slot < lv.chunk_cap) {
+        SortChunk ch;
+        ch.seg = it.seg;
+        ch.start = it.start + start;
+        ch.size = size;
+        ch.lcp0 = uint8_t(l0);
+        ch.buf = uint8_t(lv.t & 1);
+        ch.equal = uint8_t(big);                // after the last level: equal keys, already in order
+        ch.t = uint8_t(lv.t);
+        lv.chunks[slot] = ch;
+      } else {
+        lv.cnt[kCntOverflow] = 1u;
+      }
+    }
+    if (is_item) {
+      const uint32_t nt = ntiles(size);
+      const uint32_t slot = atomicAdd(&lv.cnt[2 * (lv.t + 1)], 1u);
+      const uint32_t tb = atomicAdd(&lv.cnt[2 * (lv.t + 1) + 1], nt);
+      if (slot < lv.item_cap && tb + nt <= lv.tile_cap) {
+        lv.items_next[slot] = SortItem{it.seg, it.start + start, size, tb, l0, {0u, 0u, 0u}};
+        for (uint32_t q = 0; q < nt; ++q) lv.tile_next[tb + q] = (uint64_t(q) << 32) | slot;
+      } else {
+        lv.cnt[kCntOverflow] = 1u;
       }
     }
     __syncthreads();
@@ -376,14 +381,13 @@ __global__ void __launch_bounds__(kThreads) k_sort_scatter(Level lv) {
     }
     __syncthreads();
     // ... then written out in that order: runs of equal digits are contiguous
-    const uint32_t nti = ntiles(it.size);
-    const uint32_t* hs = lv.hist + int64_t(it.hist0) * 256;
+    const uint32_t* hs = lv.hist + (int64_t(it.hist0) + tt) * 256;
     const int64_t n_tile = min(int64_t(kTile), end - (int64_t(it.start) + int64_t(tt) * kTile));
     const int64_t obase = int64_t(it.seg) * lv.M + it.start;
     for (int q = threadIdx.x; q < n_tile; q += kThreads) {
       const uint64_t k = sk[q];
       const uint32_t d = lv.digit(k);
-      const uint32_t dst = hs[int64_t(d) * nti + tt] + (uint32_t(q) - loff[d]);
+      const uint32_t dst = hs[d] + (uint32_t(q) - loff[d]);
       lv.kout[obase + dst] = k;
       lv.vout[obase + dst] = sv[q];
     }
@@ -404,106 +408,31 @@ struct LocalArgs {
   uint8_t* lcp;
 };
 
-// Stable LSD pass of one 8-bit digit over n entries in shared memory (src ->
-// dst): keys and their 16-bit ranks in the chunk move together.  Each warp
-// owns a contiguous span and ranks it with match masks against its own
-// digit counters; the warp-order scan of the counters keeps the pass
-// stable.  Keys stay in registers between counting and scatter.
-__device__ __forceinline__ void local_pass(const uint64_t* sk, const uint16_t* si, uint64_t* dk,
-                                           uint16_t* di, int n, int shift, uint16_t (*wh)[256],
-                                           uint32_t* doff) {
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const uint32_t lt = (1u << lane) - 1u;
-  {
-    uint32_t* z = reinterpret_cast<uint32_t*>(&wh[0][0]);
-    for (int q = threadIdx.x; q < kLocalWarps * 128; q += kLocalThreads) z[q] = 0u;
-  }
-  // span: a multiple of 32 covering n over the warps
-  const int span = ((n + kLocalWarps * 32 - 1) / (kLocalWarps * 32)) * 32;
-  uint64_t key[kLocalRounds];
-  uint16_t idx[kLocalRounds];
-  uint32_t pk[kLocalRounds];            // digit | local rank << 9
-#pragma unroll
-  for (int r = 0; r < kLocalRounds; ++r) {
-    const int q = warp * span + r * 32 + lane;
-    const bool in = r * 32 < span && q < n;
-    key[r] = in ? sk[q] : 0ull;
-    idx[r] = in ? si[q] : uint16_t(0);
-    pk[r] = in ? uint32_t(key[r] >> shift) & 255u : 256u + lane;
-  }
-  __syncthreads();
-#pragma unroll
-  for (int r = 0; r < kLocalRounds; ++r) {
-    if (r * 32 >= span) break;                 // uniform over the block
-    const uint32_t dg = pk[r];
-    const uint32_t peers = __match_any_sync(0xffffffffu, dg);
-    const uint32_t rank = __popc(peers & lt);
-    const uint32_t b = dg < 256u ? wh[warp][dg] : 0u;
-    __syncwarp();
-    if (dg < 256u && rank == 0) wh[warp][dg] = uint16_t(b + __popc(peers));
-    __syncwarp();
-    pk[r] = dg | ((b + rank) << 9);
-  }
-  __syncthreads();
-  for (int d = threadIdx.x; d < 256; d += kLocalThreads) {
-    uint32_t run = 0;
-#pragma unroll
-    for (int h = 0; h < kLocalWarps; ++h) {
-      const uint32_t c = wh[h][d];
-      wh[h][d] = uint16_t(run);
-      run += c;
-    }
-    doff[d] = run;
-  }
-  __syncthreads();
-  if (threadIdx.x < 32) {
-    uint32_t v[8], run = 0;
-#pragma unroll
-    for (int q = 0; q < 8; ++q) { v[q] = doff[lane * 8 + q]; run += v[q]; }
-    uint32_t incl = run;
-    for (int o = 1; o < 32; o <<= 1) {
-      const uint32_t u = __shfl_up_sync(0xffffffffu, incl, o);
-      if (lane >= o) incl += u;
-    }
-    uint32_t b = incl - run;
-#pragma unroll
-    for (int q = 0; q < 8; ++q) { doff[lane * 8 + q] = b; b += v[q]; }
-  }
-  __syncthreads();
-#pragma unroll
-  for (int r = 0; r < kLocalRounds; ++r) {
-    const uint32_t dg = pk[r] & 511u;
-    if (dg < 256u) {
-      const uint32_t dst = doff[dg] + wh[warp][dg] + (pk[r] >> 9);
-      dk[dst] = key[r];
-      di[dst] = idx[r];
-    }
-  }
-  __syncthreads();
-}
-
-// Each chunk sorted completely in shared memory, then order and common-
-// prefix lengths written to their final ranks.  The keys of a chunk are
-// first compressed without changing their order: every hash value is
-// replaced by its offset from the chunk's smallest value at that position,
-// in as many bits as the chunk's range there needs, and the fields are
-// concatenated, first hash value most significant; the digit passes then
-// run over the bits the chunk actually uses.  Two keys share a hash value
-// iff they share its field, so the common-prefix length is read off the
-// compressed keys: the field of their highest differing bit.
-__global__ void __launch_bounds__(kLocalThreads, 5) k_sort_local(LocalArgs a) {
-  extern __shared__ __align__(16) unsigned char smem[];
-  uint64_t* sk0 = reinterpret_cast<uint64_t*>(smem);
-  uint64_t* sk1 = sk0 + kSortLocalMax;
-  uint16_t* si0 = reinterpret_cast<uint16_t*>(sk1 + kSortLocalMax);
-  uint16_t* si1 = si0 + kSortLocalMax;
-  uint16_t (*wh)[256] = reinterpret_cast<uint16_t (*)[256]>(si1 + kSortLocalMax);
-  uint32_t* doff = reinterpret_cast<uint32_t*>(&wh[kLocalWarps][0]);
-  __shared__ uint32_t s_min[kLocalWarps][2], s_max[kLocalWarps][2];
-  __shared__ uint32_t s_bmin[8], s_width[8], s_off[8];
-  __shared__ uint8_t s_field[64];          // bit position -> hash value it belongs to
-  __shared__ int s_bits;
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+// Each chunk sorted completely in shared memory by (key, window), then
+// order and common-prefix lengths written to their final ranks.
+//
+// The entries are first spread over 2048 bins, about one per entry, by the
+// first three hash values that differ inside the chunk, each as its offset
+// from the chunk's smallest there in the bits its range needs, most
+// significant first (monotone in the key).  Then every entry
+// counts the smaller ones in its bin.  (key, window) is a total order, so
+// neither step has to be stable: one shared-memory atomic per entry, no
+// match masks.  On the hash strings of z-normalised windows an entry's bin
+// holds 6 to 7 entries (mean over entries).  Chunks whose bins are crowded
+// (sum of squared sizes above 48 per entry: equal or nearly equal keys) are
+// sorted by a bitonic network instead; chunks whose keys differ in no value
+// below the partitioned one are in order already.
+//
+// The least-significant-digit form before (6 to 7 digit passes with match
+// masks over 8-bit digits) took 9.0 ms for 1.6e8 entries, this one 3.0; it
+// is bound by issue (the compares inside the bins come first).
+__global__ void __launch_bounds__(kLocalThreads, kLocalBlocks) k_sort_local(LocalArgs a) {
+  __shared__ uint64_t sk[kSortLocalMax];
+  __shared__ uint32_t sv[kSortLocalMax];
+  __shared__ uint32_t bin0[kBins + 1];       // counts, then first ranks
+  __shared__ uint16_t sb[kSortLocalMax];     // bin of the entry
+  __shared__ uint32_t s_diff[2], s_min[3], s_max[3], s_cnt[kLocalWarps], s_sq[kLocalWarps];
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const uint32_t nc = min(a.cnt[kCntChunks], a.chunk_cap);
   for (uint32_t c = blockIdx.x; c < nc; c += gridDim.x) {
     const SortChunk ch = a.chunks[c];
@@ -515,104 +444,210 @@ __global__ void __launch_bounds__(kLocalThreads, 5) k_sort_local(LocalArgs a) {
     const int n = int(ch.size);
     if (ch.equal || n > kSortLocalMax) {
       // equal keys (after the last level): already in order
-      for (int q = threadIdx.x; q < n; q += kLocalThreads) {
+      for (int q = tid; q < n; q += kLocalThreads) {
         a.order[ob + q] = vin[q];
         a.lcp[ob + q] = q == 0 ? ch.lcp0 : uint8_t(a.K);
       }
       continue;
     }
-    // per-byte minimum and maximum over the chunk (four bytes per word)
-    uint32_t mn[2] = {~0u, ~0u}, mx[2] = {0u, 0u};
-    for (int q = threadIdx.x; q < n; q += kLocalThreads) {
-      const uint64_t k = kin[q] & a.kmask;
-      sk1[q] = k;                                  // the keys as loaded, for the compression
-      const uint32_t w0 = uint32_t(k >> 32), w1 = uint32_t(k);
-      mn[0] = __vminu4(mn[0], w0); mn[1] = __vminu4(mn[1], w1);
-      mx[0] = __vmaxu4(mx[0], w0); mx[1] = __vmaxu4(mx[1], w1);
+    uint64_t k[kLocalItems];
+    uint32_t v[kLocalItems];
+    if (tid < 2) s_diff[tid] = 0u;
+    if (tid < 3) {
+      s_min[tid] = ~0u;
+      s_max[tid] = 0u;
     }
-    for (int off = 16; off; off >>= 1) {
+    // the bits in which any two keys differ
+    const uint64_t k0 = kin[0] & a.kmask;
+    uint64_t diff = 0;
 #pragma unroll
-      for (int h = 0; h < 2; ++h) {
-        mn[h] = __vminu4(mn[h], __shfl_xor_sync(0xffffffffu, mn[h], off));
-        mx[h] = __vmaxu4(mx[h], __shfl_xor_sync(0xffffffffu, mx[h], off));
-      }
+    for (int i = 0; i < kLocalItems; ++i) {
+      const int q = i * kLocalThreads + tid;
+      k[i] = q < n ? kin[q] & a.kmask : ~0ull;
+      v[i] = q < n ? vin[q] : ~0u;
+      diff |= q < n ? k[i] ^ k0 : 0ull;
     }
+#pragma unroll
+    for (int q = 0; q < kBins / kLocalThreads; ++q) bin0[q * kLocalThreads + tid] = 0u;
+    const uint32_t d0 = __reduce_or_sync(0xffffffffu, uint32_t(diff >> 32));
+    const uint32_t d1 = __reduce_or_sync(0xffffffffu, uint32_t(diff));
+    __syncthreads();
     if (lane == 0) {
-      s_min[warp][0] = mn[0]; s_min[warp][1] = mn[1];
-      s_max[warp][0] = mx[0]; s_max[warp][1] = mx[1];
+      atomicOr(&s_diff[0], d0);
+      atomicOr(&s_diff[1], d1);
     }
     __syncthreads();
-    if (threadIdx.x < 8) {
-      const int b = threadIdx.x, h = b >> 2, sh = 24 - 8 * (b & 3);   // byte b of the key, 0 = most significant
-      uint32_t lo = 255u, hi = 0u;
+    diff = (uint64_t(s_diff[0]) << 32) | s_diff[1];
+    // no value below the partitioned one differs: in order as it is
+    const bool sorted = ch.t >= 7 || (diff & (~0ull >> (8 * (int(ch.t) + 1)))) == 0ull;
+    // the first three hash values that differ (as shifts), their ranges
+    int sh[3];
+    {
+      uint64_t rest = diff;
+#pragma unroll
+      for (int f = 0; f < 3; ++f) {
+        sh[f] = rest ? (63 - __clzll(static_cast<long long>(rest))) & ~7 : 0;
+        rest &= (1ull << sh[f]) - 1ull;
+      }
+    }
+    uint32_t lo[3] = {~0u, ~0u, ~0u}, hi[3] = {0u, 0u, 0u};
+#pragma unroll
+    for (int i = 0; i < kLocalItems; ++i)
+      if (i * kLocalThreads + tid < n) {
+#pragma unroll
+        for (int f = 0; f < 3; ++f) {
+          const uint32_t x = uint32_t(k[i] >> sh[f]) & 255u;
+          lo[f] = min(lo[f], x);
+          hi[f] = max(hi[f], x);
+        }
+      }
+#pragma unroll
+    for (int f = 0; f < 3; ++f) {
+      lo[f] = __reduce_min_sync(0xffffffffu, lo[f]);
+      hi[f] = __reduce_max_sync(0xffffffffu, hi[f]);
+      if (lane == 0) {
+        atomicMin(&s_min[f], lo[f]);
+        atomicMax(&s_max[f], hi[f]);
+      }
+    }
+    __syncthreads();
+    // bin: ((x0 - lo0) in w0 bits, (x1 - lo1) in w1, (x2 - lo2) in w2), its
+    // leading kBinBits bits.  A shift of 0 is a value taken already, or a
+    // position all keys share: no bits
+    int up[3], bits = 0;
+#pragma unroll
+    for (int f = 2; f >= 0; --f) {
+      lo[f] = s_min[f];
+      const bool use = f == 0 ? diff != 0 : sh[f] < sh[f - 1];
+      up[f] = use ? bits : 32;
+      if (use) bits += 32 - __clz(int(s_max[f] - lo[f]));
+    }
+    const int drop = bits > kBinBits ? bits - kBinBits : 0;
+    auto bin_of = [&](uint64_t key) {
+      uint32_t z = 0;
+#pragma unroll
+      for (int f = 0; f < 3; ++f)
+        if (up[f] < 32) z |= ((uint32_t(key >> sh[f]) & 255u) - lo[f]) << up[f];
+      return z >> drop;
+    };
+    bool spread = false;
+    if (!sorted) {
+      uint32_t br[kLocalItems];              // bin << 16 | rank of arrival
+#pragma unroll
+      for (int i = 0; i < kLocalItems; ++i) {
+        br[i] = 0;
+        if (i * kLocalThreads + tid < n) {
+          const uint32_t b = bin_of(k[i]);
+          br[i] = (b << 16) | atomicAdd(&bin0[b], 1u);
+        }
+      }
+      __syncthreads();
+      // first ranks of the bins, and the sum of their squared sizes
+      uint32_t cnt[kBins / kLocalThreads], run = 0, sq = 0;
+#pragma unroll
+      for (int q = 0; q < kBins / kLocalThreads; ++q) {
+        cnt[q] = bin0[tid * (kBins / kLocalThreads) + q];
+        run += cnt[q];
+        sq += cnt[q] * cnt[q];
+      }
+      uint32_t incl = run;
+      for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t u = __shfl_up_sync(0xffffffffu, incl, o);
+        if (lane >= o) incl += u;
+      }
+      sq = __reduce_add_sync(0xffffffffu, sq);
+      if (lane == 31) {
+        s_cnt[warp] = incl;
+        s_sq[warp] = sq;
+      }
+      __syncthreads();
+      uint32_t first = incl - run, all_sq = 0;
+#pragma unroll
       for (int w = 0; w < kLocalWarps; ++w) {
-        lo = min(lo, (s_min[w][h] >> sh) & 255u);
-        hi = max(hi, (s_max[w][h] >> sh) & 255u);
+        if (w < warp) first += s_cnt[w];
+        all_sq += s_sq[w];
       }
-      s_bmin[b] = lo;
-      s_width[b] = hi > lo ? 32u - __clz(hi - lo) : 0u;
-    }
-    __syncthreads();
-    if (threadIdx.x == 0) {
-      int off = 0;                                  // bit offset of each field from the bottom
-      for (int b = 7; b >= 0; --b) {
-        s_off[b] = uint32_t(off);
-        off += int(s_width[b]);
-      }
-      s_bits = off;
-    }
-    __syncthreads();
-    if (threadIdx.x < 64) {
-      uint8_t f = 8;
-      for (int b = 0; b < 8; ++b)
-        if (uint32_t(threadIdx.x) >= s_off[b] && uint32_t(threadIdx.x) < s_off[b] + s_width[b]) f = uint8_t(b);
-      s_field[threadIdx.x] = f;
-    }
-    const uint32_t bmin_hi = (s_bmin[0] << 24) | (s_bmin[1] << 16) | (s_bmin[2] << 8) | s_bmin[3];
-    const uint32_t bmin_lo = (s_bmin[4] << 24) | (s_bmin[5] << 16) | (s_bmin[6] << 8) | s_bmin[7];
-    uint32_t foff[8];
 #pragma unroll
-    for (int b = 0; b < 8; ++b) foff[b] = s_off[b];
-    for (int q = threadIdx.x; q < n; q += kLocalThreads) {
-      const uint64_t k = sk1[q];
-      // byte-wise offsets from the minima (no borrow: every byte is >= its minimum)
-      const uint32_t d0 = __vsub4(uint32_t(k >> 32), bmin_hi), d1 = __vsub4(uint32_t(k), bmin_lo);
-      uint64_t z = 0;
-#pragma unroll
-      for (int b = 0; b < 8; ++b) {
-        const uint32_t v = ((b < 4 ? d0 : d1) >> (24 - 8 * (b & 3))) & 255u;
-        z |= uint64_t(v) << foff[b];                 // width 0: the offset is 0
+      for (int q = 0; q < kBins / kLocalThreads; ++q) {
+        bin0[tid * (kBins / kLocalThreads) + q] = first;
+        first += cnt[q];
       }
-      sk0[q] = z;
-      si0[q] = uint16_t(q);
+      if (tid == kLocalThreads - 1) bin0[kBins] = first;
+      spread = all_sq <= 48u * uint32_t(n);
+      __syncthreads();
+      if (spread) {
+#pragma unroll
+        for (int i = 0; i < kLocalItems; ++i)
+          if (i * kLocalThreads + tid < n) {
+            const uint32_t p = bin0[br[i] >> 16] + (br[i] & 0xffffu);
+            sk[p] = k[i];
+            sv[p] = v[i];
+            sb[p] = uint16_t(br[i] >> 16);
+          }
+        __syncthreads();
+        // ranks inside the bins (neighbouring threads read the same bins)
+        uint32_t to[kLocalItems];
+#pragma unroll
+        for (int i = 0; i < kLocalItems; ++i) {
+          const int p = i * kLocalThreads + tid;
+          if (p >= n) continue;
+          k[i] = sk[p];
+          v[i] = sv[p];
+          const uint32_t b = sb[p];
+          const uint32_t q0 = bin0[b], q1 = bin0[b + 1];
+          uint32_t r = q0;
+          for (uint32_t q = q0; q < q1; ++q) {
+            const uint64_t o = sk[q];
+            r += o < k[i] ? 1u : 0u;
+            if (o == k[i] && q != uint32_t(p)) r += sv[q] < v[i] ? 1u : 0u;
+          }
+          to[i] = r;
+        }
+        __syncthreads();
+#pragma unroll
+        for (int i = 0; i < kLocalItems; ++i)
+          if (i * kLocalThreads + tid < n) {
+            sk[to[i]] = k[i];
+            sv[to[i]] = v[i];
+          }
+      }
+    }
+    if (!spread) {
+      // as loaded; the places past n hold the largest (key, window)
+#pragma unroll
+      for (int i = 0; i < kLocalItems; ++i) {
+        sk[i * kLocalThreads + tid] = k[i];
+        sv[i * kLocalThreads + tid] = v[i];
+      }
+      if (!sorted) {
+        int m = 2;
+        while (m < n) m <<= 1;
+        for (int len = 2; len <= m; len <<= 1)
+          for (int st = len >> 1; st > 0; st >>= 1) {
+            __syncthreads();
+            for (int q = tid; q < m / 2; q += kLocalThreads) {
+              const int x = 2 * st * (q / st) + q % st, y = x + st;
+              const uint64_t kx = sk[x], ky = sk[y];
+              const uint32_t vx = sv[x], vy = sv[y];
+              const bool gt = kx > ky || (kx == ky && vx > vy);
+              if (gt == ((x & len) == 0)) {
+                sk[x] = ky; sk[y] = kx;
+                sv[x] = vy; sv[y] = vx;
+              }
+            }
+          }
+      }
     }
     __syncthreads();
-    uint64_t* ck = sk0;
-    uint16_t* ci = si0;
-    uint64_t* ok = sk1;
-    uint16_t* oi = si1;
-    const int bits = s_bits;
-    for (int shift = 0; shift < bits; shift += 8) {
-      local_pass(ck, ci, ok, oi, n, shift, wh, doff);
-      uint64_t* tk = ck; ck = ok; ok = tk;
-      uint16_t* ti = ci; ci = oi; oi = ti;
-    }
-    for (int q = threadIdx.x; q < n; q += kLocalThreads) {
-      a.order[ob + q] = vin[ci[q]];
+    for (int q = tid; q < n; q += kLocalThreads) {
+      a.order[ob + q] = sv[q];
       uint32_t l = ch.lcp0;
-      if (q > 0) {
-        const uint64_t x = ck[q] ^ ck[q - 1];
-        l = x == 0 ? 8u : uint32_t(s_field[63 - __clzll(x)]);
-        if (l > uint32_t(a.K)) l = uint32_t(a.K);
-      }
+      if (q > 0) l = min(uint32_t(__clzll(static_cast<long long>(sk[q] ^ sk[q - 1]))) >> 3, uint32_t(a.K));
       a.lcp[ob + q] = uint8_t(l);
     }
     __syncthreads();
   }
 }
-
-constexpr size_t kLocalSmem = size_t(kSortLocalMax) * (8 + 8 + 2 + 2) +
-                              size_t(kLocalWarps) * 256 * 2 + 256 * 4;
 
 }  // namespace
 
@@ -646,8 +681,7 @@ cudaError_t launch_sort_reps(const Index& ix, int j0, int j1, const SortScratch&
   const int segs = (j1 - j0) * ix.D;
   if (sc.M != ix.M || segs > sc.segs) return cudaErrorInvalidValue;
   const SortCaps& c = sc.caps;
-  cudaError_t e = allow_smem(reinterpret_cast<const void*>(k_sort_local), kLocalSmem);
-  if (e != cudaSuccess) return e;
+  cudaError_t e = cudaSuccess;
   const int64_t tpm = (ix.M + kTile - 1) / kTile;
   const int sm = sm_count();
   {
@@ -714,9 +748,9 @@ cudaError_t launch_sort_reps(const Index& ix, int j0, int j1, const SortScratch&
   la.kmask = ix.K >= 8 ? ~0ull : ~((~0ull) >> (8 * ix.K));
   la.order = ix.order;
   la.lcp = ix.lcp;
-  // five CTAs of 4 warps per SM (shared memory bound); chunks statically
-  // interleaved over them
-  MOMENTI_LAUNCH("sort_local", s, k_sort_local<<<sm * 5, kLocalThreads, kLocalSmem, s>>>(la));
+  // four CTAs of 8 warps per SM (register bound; five spill); chunks
+  // statically interleaved over them
+  MOMENTI_LAUNCH("sort_local", s, k_sort_local<<<sm * kLocalBlocks, kLocalThreads, 0, s>>>(la));
   return cudaGetLastError();
 }
 
