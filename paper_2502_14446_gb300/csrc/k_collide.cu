@@ -38,28 +38,48 @@ struct Seg {
   }
 };
 
-// One warp per (segment, chunk): the last bucket start in the chunk (or -1)
-// and whether any rank of the chunk continues the bucket of its predecessor.
+// Which of the ranks p0 .. p0 + 31 of a segment (M prefix lengths at L, of
+// any alignment; ranks past M: no) share at least i hash values with their
+// predecessor: bit q for rank p0 + q.  Whole words, shifted into place; a
+// byte of a word is >= i iff byte + 128 - i has its top bit set (bytes are
+// 0..8, so no carry crosses a byte), and the four top bits are gathered by a
+// multiplication.  About two instructions a rank; a byte a lane took fifteen.
+__device__ __forceinline__ uint32_t join_mask(const uint8_t* L, int64_t p0, int64_t M, int i) {
+  if (p0 >= M) return 0u;
+  const uintptr_t at = reinterpret_cast<uintptr_t>(L + p0);
+  const uint32_t* w = reinterpret_cast<const uint32_t*>(at & ~uintptr_t(3));
+  const uint32_t sh = uint32_t(at & 3) * 8u;
+  const uint32_t* end = reinterpret_cast<const uint32_t*>(L + M);    // words starting before the segment's end
+  uint32_t x[9];
+#pragma unroll
+  for (int k = 0; k < 9; ++k) x[k] = w + k < end ? __ldg(w + k) : 0u;
+  const uint32_t add = 0x01010101u * uint32_t(128 - i);
+  uint32_t m = 0;
+#pragma unroll
+  for (int k = 0; k < 8; ++k) {
+    const uint32_t y = ((__funnelshift_r(x[k], x[k + 1], sh) + add) >> 7) & 0x01010101u;
+    m |= ((y * 0x01020408u) >> 24) << (4 * k);
+  }
+  const int64_t left = M - p0;
+  return left >= 32 ? m : m & ((1u << left) - 1u);
+}
+
+// One thread per (segment, chunk): the last bucket start in the chunk (or
+// -1) and whether any rank of the chunk continues the bucket of its
+// predecessor.
 __global__ void k_chunk_agg(const uint8_t* __restrict__ lcp, Seg sg, int segs, int i, int d,
                             int32_t* __restrict__ cagg, uint64_t* __restrict__ ntile) {
-  const int64_t gw = (blockIdx.x * int64_t(blockDim.x) + threadIdx.x) >> 5;
-  const int lane = threadIdx.x & 31;
-  if (gw >= int64_t(segs) * sg.C) return;
-  const int seg = int(gw / sg.C);
-  const int64_t c = gw - int64_t(seg) * sg.C;
-  const uint8_t* L = lcp + sg.base(seg);
-  const int64_t p = c * 32 + lane;
-  const bool valid = p < sg.M;
-  const int l = valid ? int(L[p]) : 0;
-  const unsigned st = __ballot_sync(0xffffffffu, valid && l < i);
+  const int64_t q = blockIdx.x * int64_t(blockDim.x) + threadIdx.x;
+  if (q >= int64_t(segs) * sg.C) return;
+  const int seg = int(q / sg.C);
+  const int64_t c = q - int64_t(seg) * sg.C;
+  const uint32_t ge = join_mask(lcp + sg.base(seg), c * 32, sg.M, i);
+  const int64_t left = sg.M - c * 32;
+  const uint32_t st = ~ge & (left >= 32 ? ~0u : (1u << left) - 1u);
   // a pair handled from dim f needs d - 1 more colliding dims above f
   const int f = seg - (seg / sg.D) * sg.D;
-  const bool useful = f <= sg.D - d;
-  const unsigned jn = __ballot_sync(0xffffffffu, valid && l >= i && useful);
-  if (lane == 0) {
-    cagg[gw] = st ? int32_t(c * 32 + 31 - __clz(int(st))) : -1;
-    ntile[gw] = jn ? 1u : 0u;
-  }
+  cagg[q] = st ? int32_t(c * 32 + 31 - __clz(int(st))) : -1;
+  ntile[q] = ge && f <= sg.D - d ? 1u : 0u;
 }
 
 // One block per segment: bucket start of each chunk's first rank (exclusive
@@ -218,6 +238,57 @@ __device__ __forceinline__ uint64_t zero_bytes(uint64_t x) {
   return ~(y | x | L7);
 }
 
+// The four byte planes of four words (byte 3 - h of word e becomes byte e of
+// plane h): eight byte permutations.
+__device__ __forceinline__ void transpose4(const uint32_t (&h)[4], uint32_t (&pl)[4]) {
+  const uint32_t a = __byte_perm(h[0], h[1], 0x6273), b = __byte_perm(h[0], h[1], 0x4051);
+  const uint32_t c = __byte_perm(h[2], h[3], 0x6273), e = __byte_perm(h[2], h[3], 0x4051);
+  pl[0] = __byte_perm(a, c, 0x5410);
+  pl[1] = __byte_perm(a, c, 0x7632);
+  pl[2] = __byte_perm(b, e, 0x5410);
+  pl[3] = __byte_perm(b, e, 0x7632);
+}
+
+// Byte planes 0..NQ-1 of eight keys of a window, dims f0 .. f0 + 7 of D at
+// kw (plane h: byte e = hash value h of dim f0 + e; dims past D give 0).
+// Keys hold zero bytes past their K values.
+template <int NQ>
+__device__ __forceinline__ void planes8(const uint64_t* kw, int f0, int D, uint64_t (&pl)[NQ]) {
+  uint32_t hi[2][4], lo[2][4];
+#pragma unroll
+  for (int e = 0; e < 8; ++e) hi[e >> 2][e & 3] = lo[e >> 2][e & 3] = 0u;
+  if ((D & 1) == 0) {                              // rows of whole 16-byte units
+#pragma unroll
+    for (int e = 0; e < 8; e += 2)
+      if (f0 + e < D) {
+        const uint4 q = __ldg(reinterpret_cast<const uint4*>(kw + f0 + e));
+        hi[e >> 2][e & 3] = q.y;
+        hi[e >> 2][(e & 3) + 1] = q.w;
+        lo[e >> 2][e & 3] = q.x;
+        lo[e >> 2][(e & 3) + 1] = q.z;
+      }
+  } else {
+#pragma unroll
+    for (int e = 0; e < 8; ++e)
+      if (f0 + e < D) {
+        const uint2 q = __ldg(reinterpret_cast<const uint2*>(kw + f0 + e));
+        hi[e >> 2][e & 3] = q.y;
+        lo[e >> 2][e & 3] = q.x;
+      }
+  }
+  uint32_t p0[4], p1[4];
+  transpose4(hi[0], p0);
+  transpose4(hi[1], p1);
+#pragma unroll
+  for (int h = 0; h < (NQ < 4 ? NQ : 4); ++h) pl[h] = (uint64_t(p1[h]) << 32) | p0[h];
+  if constexpr (NQ > 4) {
+    transpose4(lo[0], p0);
+    transpose4(lo[1], p1);
+#pragma unroll
+    for (int h = 4; h < (NQ < 8 ? NQ : 8); ++h) pl[h] = (uint64_t(p1[h - 4]) << 32) | p0[h - 4];
+  }
+}
+
 // Per warp: the 64 windows of a tile (32 row ranks, 32 column ranks) as
 // byte planes: word (t, g) of a window holds byte t (hash value t) of the
 // keys of dims 8g .. 8g+7, dim 8g+e in byte e.  Equality of the length-i
@@ -267,13 +338,7 @@ __global__ void __launch_bounds__(128) k_collide(CollideArgs g) {
       uint64_t pw[NPMAX];
 #pragma unroll
       for (int q = 0; q < NPMAX; ++q) pw[q] = 0;
-      for (int ee = 0; ee < 8; ++ee) {
-        const int ff = gg * 8 + ee;
-        if (ff >= D || !ok) break;
-        const uint64_t key = kw[ff];
-#pragma unroll
-        for (int q = 0; q < NPMAX; ++q) pw[q] |= ((key >> (56 - 8 * q)) & 0xFFull) << (8 * ee);
-      }
+      if (ok) planes8<NPMAX>(kw, gg * 8, D, pw);
 #pragma unroll
       for (int q = 0; q < NPMAX; ++q)
         if (q < NP) sp[(q * G + gg) * 64 + r] = pw[q];
@@ -335,9 +400,10 @@ __global__ void __launch_bounds__(128) k_collide(CollideArgs g) {
       int W = 0;
       if (emit) {
         if (G == 1) {
-          uint64_t m = valid0;
+          uint64_t x = 0;
 #pragma unroll
-          for (int q = 0; q < I; ++q) m &= zero_bytes(rp[q] ^ sp[q * 64 + 32 + cc]);
+          for (int q = 0; q < I; ++q) x |= rp[q] ^ sp[q * 64 + 32 + cc];
+          const uint64_t m = valid0 & zero_bytes(x);
           emit = (m & lowmask) == 0;
           W = __popcll(m);
           if (emit && W >= g.d && lvl_dup) {
@@ -350,9 +416,10 @@ __global__ void __launch_bounds__(128) k_collide(CollideArgs g) {
             const int nvalid = min(8, D - gg * 8);
             uint64_t m = nvalid == 8 ? 0x8080808080808080ull
                                      : (0x8080808080808080ull & ((1ull << (8 * nvalid)) - 1));
+            uint64_t x = 0;
 #pragma unroll
-            for (int q = 0; q < I; ++q)
-              m &= zero_bytes(sp[(q * G + gg) * 64 + lane] ^ sp[(q * G + gg) * 64 + 32 + cc]);
+            for (int q = 0; q < I; ++q) x |= sp[(q * G + gg) * 64 + lane] ^ sp[(q * G + gg) * 64 + 32 + cc];
+            m &= zero_bytes(x);
             if (gg < gf) low = m != 0;
             else if (gg == gf) low = (m & ((1ull << (8 * ef)) - 1)) != 0;
             W += __popcll(m);
@@ -408,31 +475,42 @@ __global__ void __launch_bounds__(128) k_collide(CollideArgs g) {
 // list 1 9..32 (a warp each, counts[2]), list 2 5..8 (8 lanes each,
 // counts[3]), list 3 2..4 (4 lanes each, counts[4]); counts[1] = the
 // largest bucket.
-__global__ void k_bucket_jobs(const uint8_t* __restrict__ lcp, Seg sg, int segs, int i, int d,
-                              BucketJob* __restrict__ jobs, uint64_t job_cap,
-                              unsigned long long* __restrict__ counts) {
+// A lane takes 32 ranks as a bit mask (join_mask), its bucket starts are the
+// clear bits followed by a set one, and a warp takes room in the four lists
+// for its 1024 ranks at once.  (A rank per thread, with block-wide counting
+// every 256 ranks, took 2.7 ms where this takes 0.55, D = 8, n = 1e5.)
+__global__ void __launch_bounds__(256) k_bucket_jobs(const uint8_t* __restrict__ lcp, Seg sg, int segs, int i, int d,
+                                                     BucketJob* __restrict__ jobs, uint64_t job_cap,
+                                                     unsigned long long* __restrict__ counts) {
   // grid: x over the positions of a segment, y over the segments
-  __shared__ uint32_t wcnt[32][4];
-  __shared__ unsigned long long bbase[4];
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarp = blockDim.x >> 5;
+  const int lane = threadIdx.x & 31;
   const uint64_t quarter = job_cap / 4;
-  const unsigned lt = (1u << lane) - 1u;
   const uint32_t seg = blockIdx.y;
   const int f = int(seg % uint32_t(sg.D));
   if (f > sg.D - d) return;                        // block-uniform: f cannot be a lowest dim
   const uint8_t* L = lcp + sg.base(int(seg));
-  for (int64_t q0 = blockIdx.x * int64_t(blockDim.x); q0 < sg.M; q0 += int64_t(gridDim.x) * blockDim.x) {
-    const int64_t q = q0 + threadIdx.x;
-    bool emit = false;
-    uint32_t n = 0, p = 0;
-    if (q < sg.M) {
-      p = uint32_t(q);
-      if (int(L[p]) < i && int64_t(p) + 1 < sg.M && int(L[p + 1]) >= i) {
-        // walk to the end of the run, eight prefix lengths at a time where
-        // aligned: every byte of a word is >= i iff byte + 128 - i has its
-        // top bit set (bytes are 0..8, so no carry crosses a byte)
+  const int64_t nw = int64_t(gridDim.x) * (blockDim.x >> 5);
+  for (int64_t w = (blockIdx.x * int64_t(blockDim.x) + threadIdx.x) >> 5; w * 1024 < sg.M; w += nw) {
+    const int64_t p0 = w * 1024 + lane * 32;
+    const uint32_t ge = join_mask(L, p0, sg.M, i);
+    uint32_t next = __shfl_down_sync(0xffffffffu, ge, 1);
+    if (lane == 31) next = p0 + 32 < sg.M && int(L[p0 + 32]) >= i ? 1u : 0u;
+    // (ranks past M are clear in ge and never followed by a set bit)
+    const uint32_t starts = ~ge & ((ge >> 1) | (next << 31));
+    // members of the bucket of a start; the last one may run past the lane's ranks
+    uint32_t n_last = 0;
+    auto members = [&](int b) -> uint32_t {
+      const uint32_t after = b == 31 ? 0u : ~(ge >> (b + 1));          // clear while the bucket goes on
+      const int run = b == 31 ? 0 : __ffs(int(after)) - 1;
+      return b + 1 + run < 32 ? uint32_t(run) + 1u : 0u;               // 0: past the lane's ranks
+    };
+    if (starts) {
+      const int b = 31 - __clz(int(starts));
+      if (members(b) == 0u) {
+        // walk on, eight prefix lengths at a time where aligned: every byte
+        // of a word is >= i iff byte + 128 - i has its top bit set
         const uint64_t add = 0x0101010101010101ull * uint64_t(128 - i);
-        int64_t e = p + 1;
+        int64_t e = p0 + 31;
         while (e + 1 < sg.M) {
           const int64_t q = e + 1;
           if ((reinterpret_cast<uintptr_t>(L + q) & 7) == 0 && q + 8 <= sg.M) {
@@ -445,36 +523,48 @@ __global__ void k_bucket_jobs(const uint8_t* __restrict__ lcp, Seg sg, int segs,
           if (int(L[q]) < i) break;
           ++e;
         }
-        n = uint32_t(e - p + 1);
-        emit = true;
+        n_last = uint32_t(e - (p0 + b) + 1);
       }
     }
-    const int cls = !emit ? -1 : (n > 32u ? 0 : (n > 8u ? 1 : (n > 4u ? 2 : 3)));
-    if (emit && cls == 0) atomicMax(&counts[1], (unsigned long long)n);
-    // room in the four lists: one global atomic per list and block
-    unsigned m[4];
+    // counts per list, 16 bits each (a warp has at most 512 starts)
+    uint64_t cnt = 0;
+    uint32_t big = 0;
+    for (uint32_t m = starts; m; m &= m - 1u) {
+      uint32_t n = members(__ffs(int(m)) - 1);
+      if (!n) n = n_last;
+      const int cls = n > 32u ? 0 : (n > 8u ? 1 : (n > 4u ? 2 : 3));
+      if (cls == 0) big = max(big, n);
+      cnt += 1ull << (16 * cls);
+    }
+    uint64_t incl = cnt;
+    for (int o = 1; o < 32; o <<= 1) {
+      const uint64_t u = __shfl_up_sync(0xffffffffu, incl, o);
+      if (lane >= o) incl += u;
+    }
+    const uint64_t total = __shfl_sync(0xffffffffu, incl, 31);
+    if (!total) continue;                          // warp-uniform
+    big = __reduce_max_sync(0xffffffffu, big);
+    unsigned long long base = 0;
+    if (lane < 4) {
+      const unsigned long long t = (total >> (16 * lane)) & 0xffffull;
+      if (t) base = atomicAdd(&counts[lane == 0 ? 0 : lane + 1], t);
+    }
+    if (lane == 0 && big) atomicMax(&counts[1], (unsigned long long)big);
+    uint64_t at[4];
 #pragma unroll
-    for (int c = 0; c < 4; ++c) {
-      m[c] = __ballot_sync(0xffffffffu, cls == c);
-      if (lane == 0) wcnt[warp][c] = __popc(m[c]);
+    for (int c = 0; c < 4; ++c)
+      at[c] = __shfl_sync(0xffffffffu, base, c) + (((incl - cnt) >> (16 * c)) & 0xffffull);
+    for (uint32_t m = starts; m; m &= m - 1u) {
+      const int b = __ffs(int(m)) - 1;
+      uint32_t n = members(b);
+      if (!n) n = n_last;
+      const int cls = n > 32u ? 0 : (n > 8u ? 1 : (n > 4u ? 2 : 3));
+      uint64_t pos = 0;
+#pragma unroll
+      for (int c = 0; c < 4; ++c)
+        if (c == cls) pos = at[c]++;
+      if (pos < quarter) jobs[cls * quarter + pos] = BucketJob{seg, uint32_t(p0) + uint32_t(b), n, 0u};
     }
-    __syncthreads();
-    if (threadIdx.x < 4) {
-      const int c = threadIdx.x;
-      uint32_t run = 0;
-      for (int ww = 0; ww < nwarp; ++ww) {
-        const uint32_t x = wcnt[ww][c];
-        wcnt[ww][c] = run;
-        run += x;
-      }
-      bbase[c] = run ? atomicAdd(&counts[c == 0 ? 0 : c + 1], (unsigned long long)run) : 0ull;
-    }
-    __syncthreads();
-    if (cls >= 0) {
-      const unsigned long long pos = bbase[cls] + wcnt[warp][cls] + __popc(m[cls] & lt);
-      if (pos < quarter) jobs[cls * quarter + pos] = BucketJob{seg, p, n, 0u};
-    }
-    __syncthreads();                               // wcnt / bbase reused by the next iteration
   }
 }
 
@@ -496,19 +586,13 @@ struct SubArgs {
 // Byte planes 0..NQ-1 of a window's D keys (plane h, word c: byte e =
 // hash value h of dim 8c + e), each key loaded once.
 template <int NQ, int NW>
-__device__ __forceinline__ void key_planes(const uint64_t* kw, int D, int K, uint64_t (&pl)[NQ][NW]) {
+__device__ __forceinline__ void key_planes(const uint64_t* kw, int D, uint64_t (&pl)[NQ][NW]) {
 #pragma unroll
   for (int c = 0; c < NW; ++c) {
-    uint64_t key[8];
+    uint64_t t[NQ];
+    planes8<NQ>(kw, 8 * c, D, t);
 #pragma unroll
-    for (int e = 0; e < 8; ++e) key[e] = 8 * c + e < D ? kw[8 * c + e] : 0ull;
-#pragma unroll
-    for (int h = 0; h < NQ; ++h) {
-      uint64_t a = 0;
-#pragma unroll
-      for (int e = 0; e < 8; ++e) a |= ((key[e] >> (56 - 8 * h)) & 0xFFull) << (8 * e);
-      pl[h][c] = h < K ? a : 0ull;
-    }
+    for (int h = 0; h < NQ; ++h) pl[h][c] = t[h];
   }
 }
 
@@ -555,7 +639,7 @@ __global__ void __launch_bounds__(256) k_subbucket(SubArgs g) {
       const uint32_t wv = O[q];
       widx[q] = wv;
       uint64_t kp[NQ][NW];
-      key_planes<NQ, NW>(Kj + int64_t(wv) * D, D, g.K, kp);
+      key_planes<NQ, NW>(Kj + int64_t(wv) * D, D, kp);
 #pragma unroll
       for (int h = 0; h < NQ; ++h)
 #pragma unroll
@@ -623,9 +707,10 @@ __global__ void __launch_bounds__(256) k_subbucket(SubArgs g) {
           int w0 = 0;
 #pragma unroll
           for (int c = 0; c < NW; ++c) {
-            uint64_t x = valid[c];
+            uint64_t x = 0;
 #pragma unroll
-            for (int h = 0; h < I; ++h) x &= zero_bytes(pu[h][c] ^ pl[(h * NW + c) * cap + v]);
+            for (int h = 0; h < I; ++h) x |= pu[h][c] ^ pl[(h * NW + c) * cap + v];
+            x = valid[c] & zero_bytes(x);
             m[c] = x;
             // f and f2 are the two lowest colliding dims
             lowest = lowest && (x & below[c]) == only_f[c];
@@ -701,7 +786,7 @@ __global__ void __launch_bounds__(256) k_subwarp(SubArgs g, int list) {
       f = seg - (seg / D) * D;
       if (sl < n) {
         wu = g.order[g.sg.base(seg) + job.start + sl];
-        key_planes<NQ, NW>(g.keys + (int64_t(j) * g.sg.M + wu) * D, D, g.K, pu);
+        key_planes<NQ, NW>(g.keys + (int64_t(j) * g.sg.M + wu) * D, D, pu);
       }
     }
     // dims below f must not collide: bytes of dims < f
@@ -714,27 +799,34 @@ __global__ void __launch_bounds__(256) k_subwarp(SubArgs g, int list) {
     int nmax = n;
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) nmax = max(nmax, __shfl_xor_sync(0xffffffffu, nmax, o));
+    checks += sl < n ? uint32_t(sl) : 0u;          // pairs (v, sl), v < sl
     for (int v = 0; v < nmax - 1; ++v) {
-      uint64_t pv[NQ][NW];
-#pragma unroll
-      for (int h = 0; h < NQ; ++h)
-#pragma unroll
-        for (int c = 0; c < NW; ++c) pv[h][c] = __shfl_sync(0xffffffffu, pu[h][c], v, W);
-      const uint32_t wv = __shfl_sync(0xffffffffu, wu, v, W);
+      // the first I planes decide almost every pair; the window and the
+      // plane of the level check follow where some pair of the warp passes
       bool emit = sl > v && sl < n;
-      checks += emit ? 1u : 0u;
-      int w0 = 0, w1 = 0;
+      int w0 = 0;
       bool low = false;
+      uint64_t mm[NW];
 #pragma unroll
       for (int c = 0; c < NW; ++c) {
-        uint64_t x = valid[c];
+        uint64_t x = 0;
 #pragma unroll
-        for (int h = 0; h < I; ++h) x &= zero_bytes(pu[h][c] ^ pv[h][c]);
+        for (int h = 0; h < I; ++h) x |= pu[h][c] ^ __shfl_sync(0xffffffffu, pu[h][c], v, W);
+        x = valid[c] & zero_bytes(x);
+        mm[c] = x;
         low = low || (x & below[c]) != 0;
         w0 += __popcll(x);
-        if (lvl_dup) w1 += __popcll(x & zero_bytes(pu[I][c] ^ pv[I][c]));
       }
-      emit = emit && !low && w0 >= g.d && !(lvl_dup && w1 >= g.d);
+      emit = emit && !low && w0 >= g.d;
+      if (!__any_sync(0xffffffffu, emit)) continue;
+      const uint32_t wv = __shfl_sync(0xffffffffu, wu, v, W);
+      if (lvl_dup) {
+        int w1 = 0;
+#pragma unroll
+        for (int c = 0; c < NW; ++c)
+          w1 += __popcll(mm[c] & zero_bytes(pu[I][c] ^ __shfl_sync(0xffffffffu, pu[I][c], v, W)));
+        emit = emit && w1 < g.d;
+      }
       const uint32_t a = min(wu, wv), b = max(wu, wv);
       emit = emit && int64_t(b) - int64_t(a) > g.excl;
       const uint64_t key = (uint64_t(a) << 32) | b;
@@ -793,7 +885,7 @@ cudaError_t launch_bucket_jobs(const Index& ix, int i, int j0, int j1, int d, Bu
                                uint64_t job_cap, unsigned long long* counts, cudaStream_t s) {
   const int segs = (j1 - j0) * ix.D;
   Seg sg{ix.M, ix.D, j0, int((ix.M + 31) / 32)};
-  int64_t gx = (ix.M + 255) / 256;
+  int64_t gx = (ix.M + 8191) / 8192;               // 8 warps of 1024 ranks
   const int64_t per_seg = std::max<int64_t>(1, (sm_count() * 16 + segs - 1) / segs);
   if (gx > per_seg) gx = per_seg;
   dim3 grid{unsigned(gx), unsigned(segs), 1u};
@@ -857,7 +949,7 @@ cudaError_t launch_collide(const Index& ix, int i, int j0, int j1, int d, const 
   Seg sg{ix.M, ix.D, j0, int(C)};
   const int64_t E = int64_t(segs) * C;
   uint64_t* toff = cs.ntile;
-  MOMENTI_LAUNCH("chunk_agg", s, k_chunk_agg<<<unsigned((E * 32 + 255) / 256), 256, 0, s>>>(ix.lcp, sg, segs, i, d, cs.cagg, toff));
+  MOMENTI_LAUNCH("chunk_agg", s, k_chunk_agg<<<unsigned((E + 255) / 256), 256, 0, s>>>(ix.lcp, sg, segs, i, d, cs.cagg, toff));
   MOMENTI_LAUNCH("chunk_scan", s, k_chunk_scan<<<segs, 1024, 0, s>>>(ix.lcp, sg, i, cs.cagg, cs.cbs, toff));
   const int64_t nb = (E + kScanBlock - 1) / kScanBlock;
   uint64_t* bsum = cs.scan_tmp;

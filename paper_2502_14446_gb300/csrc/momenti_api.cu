@@ -1095,7 +1095,7 @@ static int hash_all_impl(momenti_handle* h, const void* series, int32_t dtype, i
     CK(dalloc(h, &ix.boff, size_t(D) * N));
     CK(dalloc(h, &ix.keys, size_t(L) * M * D));
     CK(dalloc(h, &ix.order, size_t(L) * M * D));
-    CK(dalloc(h, &ix.lcp, size_t(L) * M * D));
+    CK(dalloc(h, &ix.lcp, size_t(L) * M * D + 4));     // read in whole words
     h->draw_a = nullptr;
     h->draw_u = nullptr;
     const int n_fn = tens ? 2 * isqrt(L) : L;          // hash functions per dim
