@@ -395,10 +395,15 @@ k_proj_hash_tc(const __grid_constant__ CUtensorMap tmap, TcArgs g) {
 }
 
 // Canonical FP32 recomputation of flagged values (same arithmetic as the
-// CUDA-core form): patches one byte of the key.
+// CUDA-core form: one FMA chain over t): patches one byte of the key.  One
+// value per thread, its projection vector read along the row of the
+// half-precision copy, which holds the same numbers (8 per load; the float
+// copy's column costs a sector per number: 23 ms for 1e7 values of w = 500
+// against 7.8 here).  Neighbouring flags come from one window tile, so the
+// points are L1 hits.
 __global__ void k_rehash(const float* __restrict__ xh, const float* __restrict__ xl,
                          const float* __restrict__ mh, const float* __restrict__ ml,
-                         const float* __restrict__ isg, const float* __restrict__ a32,
+                         const float* __restrict__ isg, const __half* __restrict__ a16,
                          const float* __restrict__ boff, float inv_r, int64_t n, int64_t M, int D,
                          int w, int Wp, int N, const uint64_t* __restrict__ flags,
                          const uint32_t* __restrict__ count, uint32_t cap,
@@ -413,11 +418,20 @@ __global__ void k_rehash(const float* __restrict__ xh, const float* __restrict__
     const float m0 = mh[o], m1 = ml[o], is = isg[o];
     const float* x = xh + int64_t(f) * n + a;
     const float* l = xl ? xl + int64_t(f) * n + a : nullptr;
-    const float* A = a32 + int64_t(f) * Wp * N + nn;
+    const uint4* A = reinterpret_cast<const uint4*>(a16 + (int64_t(f) * N + nn) * Wp);   // Wp: a multiple of 64
     float acc = 0.f;
-    for (int t = 0; t < w; ++t) {
-      float z = (x[t] - m0) + ((l ? l[t] : 0.f) - m1);
-      acc = fmaf(A[int64_t(t) * N], z, acc);
+    for (int t0 = 0; t0 < w; t0 += 8) {
+      const uint4 v = __ldg(A + (t0 >> 3));
+      const uint32_t hw[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+      for (int u = 0; u < 8; ++u) {
+        const int t = t0 + u;
+        if (t < w) {
+          const float2 c = __half22float2(*reinterpret_cast<const __half2*>(&hw[u >> 1]));
+          const float z = (x[t] - m0) + ((l ? l[t] : 0.f) - m1);
+          acc = fmaf(u & 1 ? c.y : c.x, z, acc);
+        }
+      }
     }
     const float v = acc * is;
     const float qv = (v + boff[int64_t(f) * N + nn]) * inv_r;
@@ -495,7 +509,7 @@ cudaError_t launch_proj_hash_tc(const Index& ix, int j0, int j1, uint64_t* flags
 cudaError_t launch_rehash_fp32(const Index& ix, const uint64_t* flags, const uint32_t* flag_count,
                                uint32_t flag_cap, cudaStream_t s) {
   MOMENTI_LAUNCH("rehash", s, k_rehash<<<sm_count() * 8, 256, 0, s>>>(ix.xs_hi, ix.has_lo ? ix.xs_lo : nullptr, ix.mu_hi, ix.mu_lo,
-                                   ix.inv_sig, ix.a32, ix.boff, ix.inv_r, ix.n, ix.M, ix.D, ix.w,
+                                   ix.inv_sig, ix.a16, ix.boff, ix.inv_r, ix.n, ix.M, ix.D, ix.w,
                                    ix.Wp, ix.L * kRepStride, flags, flag_count, flag_cap,
                                    reinterpret_cast<unsigned long long*>(ix.keys)));
   return cudaGetLastError();
