@@ -1137,16 +1137,6 @@ static int hash_all_impl(momenti_handle* h, const void* series, int32_t dtype, i
     cs.ev_cap = uint64_t(1) << 22;
     h->ev_budget = std::max<uint64_t>(uint64_t(1) << 28, limit / 8);
     CK(dalloc(h, &cs.events, size_t(cs.ev_cap)));
-    if (h->rec_host_cap < new_cap) {
-      if (h->rec_host) {
-        cudaStreamSynchronize(s);
-        cudaFreeHost(h->rec_host);
-        h->rec_host = nullptr;
-      }
-      h->rec_host_cap = 0;
-      CK(cudaMallocHost(&h->rec_host, new_cap * sizeof(PairRec)));
-      h->rec_host_cap = new_cap;
-    }
     if (!h->cnt_host) CK(cudaMallocHost(&h->cnt_host, 8 * sizeof(unsigned long long)));
     if (!h->sort_cnt_host) CK(cudaMallocHost(&h->sort_cnt_host, 64 * sizeof(uint32_t)));
     h->sort.host_cnt = h->sort_cnt_host;
@@ -1398,19 +1388,22 @@ static int search_step_impl(momenti_handle* h, int64_t max_reps, int32_t* ended)
         const uint64_t cap = next_pow2(cnt[1]);
         PairRec* rec = nullptr;
         CK(dalloc(h, &rec, size_t(cap)));
-        if (h->rec_host_cap < cap) {
-          PairRec* rh = nullptr;
-          CK(cudaMallocHost(&rh, cap * sizeof(PairRec)));
-          cudaFreeHost(h->rec_host);
-          h->rec_host = rh;
-          h->rec_host_cap = cap;
-        }
         h->rec_dev = rec;
         h->rec_cap = cap;
         CK(cudaMemsetAsync(h->cs.counters + 1, 0, 7 * sizeof(unsigned long long), s));
       }
       nrec = cnt[1];
       h->set_fill += cnt[2];
+      if (nrec > h->rec_host_cap) {
+        // pinned by need, not by the device buffer's size: pinning 64 MB
+        // took most of a short search with a handle of its own
+        const uint64_t cap = std::max<uint64_t>(uint64_t(1) << 14, next_pow2(nrec));
+        PairRec* rh = nullptr;
+        CK(cudaMallocHost(&rh, cap * sizeof(PairRec)));
+        if (h->rec_host) cudaFreeHost(h->rec_host);
+        h->rec_host = rh;
+        h->rec_host_cap = cap;
+      }
       if (nrec) {
         CK(cudaMemcpyAsync(h->rec_host, h->rec_dev, nrec * sizeof(PairRec), cudaMemcpyDeviceToHost, s));
         CK(cudaStreamSynchronize(s));
