@@ -12,17 +12,22 @@
 // and the key holds byte k at bits 56 - 8k (big-endian: the prefix of
 // length i is the top 8i bits, Section 4's lexicographic order).
 //
-// Tiling: a CTA computes 64 windows x 8 repetitions (64 projections) of one
+// Tiling: a CTA computes 128 windows x 8 repetitions (64 projections) of one
 // dimension; the series segment and the projection vectors of each t-chunk
-// are staged in shared memory.  Thread (tw, tr) owns windows tw and tw+32
-// and repetition tr, i.e. 2 x 8 accumulators.
+// are staged in shared memory.  Thread (tw, tr) owns windows tw, tw+32,
+// tw+64, tw+96 and repetition tr, i.e. 4 x 8 accumulators in pairs: the
+// packed FMA rounds each half as the scalar one, at half the issue slots,
+// and the two shared loads of a step's vectors serve four windows.  Bound
+// by the FP32 lanes (2.8e11 flop at D = 11, w = 200, n = 4e4: 3.5 ms at the
+// peak); two windows with scalar FMAs took 10.4 ms, this 8.3.
 #include "internal.h"
 
 namespace momenti {
 
 namespace {
 
-constexpr int kBM = 64;    // windows per CTA
+constexpr int kWin = 4;    // windows per thread
+constexpr int kBM = 32 * kWin;   // windows per CTA
 constexpr int kBR = 8;     // repetitions per CTA
 constexpr int kBN = kBR * kRepStride;
 constexpr int kTK = 32;    // t-chunk
@@ -57,18 +62,18 @@ k_proj_hash_fp32(const float* __restrict__ xh, const float* __restrict__ xl,
   const float* lf = LO ? xl + int64_t(f) * n : nullptr;
   const float* Af = a32 + int64_t(f) * Wp * N;
 
-  int64_t wa[2] = {a0 + tw, a0 + tw + 32};
-  float m0[2], m1[2];
-  for (int u = 0; u < 2; ++u) {
-    int64_t o = int64_t(f) * M + (wa[u] < M ? wa[u] : 0);
+  int64_t wa[kWin];
+  float m0[kWin], m1[kWin];
+  float2 acc[kWin][kRepStride / 2];
+#pragma unroll
+  for (int u = 0; u < kWin; ++u) {
+    wa[u] = a0 + tw + 32 * u;
+    const int64_t o = int64_t(f) * M + (wa[u] < M ? wa[u] : 0);
     m0[u] = mh[o];
     m1[u] = ml[o];
+#pragma unroll
+    for (int k = 0; k < kRepStride / 2; ++k) acc[u][k] = make_float2(0.f, 0.f);
   }
-  float acc[2][kRepStride];
-#pragma unroll
-  for (int u = 0; u < 2; ++u)
-#pragma unroll
-    for (int k = 0; k < kRepStride; ++k) acc[u][k] = 0.f;
 
   const int nb0 = jb * kRepStride;
   for (int t0 = 0; t0 < w; t0 += kTK) {
@@ -85,16 +90,18 @@ k_proj_hash_fp32(const float* __restrict__ xh, const float* __restrict__ xl,
     }
     __syncthreads();
     const int tmax = min(kTK, w - t0);
+#pragma unroll 4
     for (int tt = 0; tt < tmax; ++tt) {
-      float z0 = (sx[tw + tt] - m0[0]) + ((LO ? sxl[tw + tt] : 0.f) - m1[0]);
-      float z1 = (sx[tw + 32 + tt] - m0[1]) + ((LO ? sxl[tw + 32 + tt] : 0.f) - m1[1]);
       const float4 b0 = *reinterpret_cast<const float4*>(&sb[tt][tr * kRepStride]);
       const float4 b1 = *reinterpret_cast<const float4*>(&sb[tt][tr * kRepStride + 4]);
-      const float bv[8] = {b0.x, b0.y, b0.z, b0.w, b1.x, b1.y, b1.z, b1.w};
+      const float2 bv[4] = {make_float2(b0.x, b0.y), make_float2(b0.z, b0.w), make_float2(b1.x, b1.y),
+                            make_float2(b1.z, b1.w)};
 #pragma unroll
-      for (int k = 0; k < kRepStride; ++k) {
-        acc[0][k] = fmaf(bv[k], z0, acc[0][k]);
-        acc[1][k] = fmaf(bv[k], z1, acc[1][k]);
+      for (int u = 0; u < kWin; ++u) {
+        const float z = (sx[tw + 32 * u + tt] - m0[u]) + ((LO ? sxl[tw + 32 * u + tt] : 0.f) - m1[u]);
+        const float2 zz = make_float2(z, z);
+#pragma unroll
+        for (int k = 0; k < kRepStride / 2; ++k) acc[u][k] = __ffma2_rn(bv[k], zz, acc[u][k]);
       }
     }
   }
@@ -105,13 +112,14 @@ k_proj_hash_fp32(const float* __restrict__ xh, const float* __restrict__ xl,
   float bvals[kRepStride];
 #pragma unroll
   for (int k = 0; k < kRepStride; ++k) bvals[k] = bo[k];
-  for (int u = 0; u < 2; ++u) {
+#pragma unroll
+  for (int u = 0; u < kWin; ++u) {
     if (wa[u] >= M) continue;
     const float is = isg[int64_t(f) * M + wa[u]];
     uint64_t key = 0;
 #pragma unroll
     for (int k = 0; k < kRepStride; ++k) {
-      uint64_t byte = (k < K) ? hash_byte(acc[u][k], is, bvals[k], inv_r) : 0u;
+      uint64_t byte = (k < K) ? hash_byte((k & 1) ? acc[u][k >> 1].y : acc[u][k >> 1].x, is, bvals[k], inv_r) : 0u;
       key |= byte << (56 - 8 * k);
     }
     keys[(int64_t(j) * M + wa[u]) * D + f] = key;
