@@ -425,8 +425,10 @@ __device__ __noinline__ int sw_redo(const SweepJob* jb, const SwVec<P>* rows, Sw
     for (int p = 0; p < P; ++p) o.v[p] = make_float2(__fdividef(1.f, s.v[p].x), __fdividef(1.f, s.v[p].y));
     return o;
   };
-  auto load = [&](int c, int slot) {
-    const SwVec<P>* p0 = tab + sw_off(b + c) * G + L.g;
+  // b is a multiple of 8: its 8 columns, and the next 8, are 8 G apart
+  const SwVec<P>* pb = tab + sw_off(b) * G + L.g;
+  const SwVec<P>* pn = tab + sw_off(b + 8) * G + L.g;
+  auto load = [&](const SwVec<P>* p0, int slot) {
     df[slot] = p0[0];
     dg[slot] = p0[64 * G];
     ib[slot] = inv(p0[128 * G]);
@@ -436,11 +438,11 @@ __device__ __noinline__ int sw_redo(const SweepJob* jb, const SwVec<P>* rows, Sw
     const SwVec<P> c = ck[r * 32 + lane];
 #pragma unroll
     for (int p = 0; p < P; ++p) C[r][p] = c.v[p];
-    load(r, r);
+    load(pb + r * 8 * G, r);
   }
 #pragma unroll 1
   for (int i2 = 0; hot >> i2; i2 += 2) {
-    load(i2 + 8, 8);
+    load(pn + i2 * 8 * G, 8);
 #pragma unroll
     for (int h = 0; h < 2; ++h, rows += 3 * G) {
       const int i = i2 + h;
@@ -521,7 +523,7 @@ __device__ __noinline__ int sw_redo(const SweepJob* jb, const SwVec<P>* rows, Sw
       dg[r] = dg[r + 2];
       ib[r] = ib[r + 2];
     }
-    load(i2 + 9, 7);
+    load(pn + (i2 + 1) * 8 * G, 7);
   }
   return qn;
 }
