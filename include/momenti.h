@@ -455,7 +455,7 @@ uint64_t momenti_launch_count(void);
  * Kernel names: split_f32, split_f64, point_major, window_stats,
  * stats_pm, mean16, r_sample, draw, layout_hash, layout_boff,
  * proj_hash_fp32, proj_hash_tc, rehash, sort_init, sort_hist, sort_scan,
- * sort_scatter, sort_local, tensor_keys, chunk_agg, chunk_scan, scan_local, scan_top,
+ * sort_scatter, sort_local, tensor_keys, chunk_scan, scan_top,
  * scan_add, collide, bucket_jobs, subbucket, subwarp, hs_clear,
  * verify_events, verify_pairs, sweep_table, allpairs, allpairs_sample,
  * allpairs_batch, select_pairs. */

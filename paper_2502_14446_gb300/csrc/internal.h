@@ -211,10 +211,9 @@ struct Event {
   uint32_t pad;
 };
 struct CollideScratch {
-  int32_t* cagg = nullptr;     // [segs][chunks] last bucket start in chunk, or -1
   int32_t* cbs = nullptr;      // [segs][chunks] bucket start of the chunk's first rank
   uint64_t* ntile = nullptr;   // [segs*chunks + 1] tiles per chunk, then exclusive scan
-  uint64_t* scan_tmp = nullptr;   // [segs*chunks / 1024 + 2]
+  uint64_t* scan_tmp = nullptr;   // [segs + 1] tiles per segment, then exclusive scan
   Event* events = nullptr;
   uint64_t ev_cap = 0;
   // [0] events (or plain pairs), [1] close records, [2] set inserts,

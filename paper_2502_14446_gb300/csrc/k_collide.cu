@@ -64,104 +64,88 @@ __device__ __forceinline__ uint32_t join_mask(const uint8_t* L, int64_t p0, int6
   return left >= 32 ? m : m & ((1u << left) - 1u);
 }
 
-// One thread per (segment, chunk): the last bucket start in the chunk (or
-// -1) and whether any rank of the chunk continues the bucket of its
-// predecessor.
-__global__ void k_chunk_agg(const uint8_t* __restrict__ lcp, Seg sg, int segs, int i, int d,
-                            int32_t* __restrict__ cagg, uint64_t* __restrict__ ntile) {
-  const int64_t q = blockIdx.x * int64_t(blockDim.x) + threadIdx.x;
-  if (q >= int64_t(segs) * sg.C) return;
-  const int seg = int(q / sg.C);
-  const int64_t c = q - int64_t(seg) * sg.C;
-  const uint32_t ge = join_mask(lcp + sg.base(seg), c * 32, sg.M, i);
-  const int64_t left = sg.M - c * 32;
-  const uint32_t st = ~ge & (left >= 32 ? ~0u : (1u << left) - 1u);
-  // a pair handled from dim f needs d - 1 more colliding dims above f
-  const int f = seg - (seg / sg.D) * sg.D;
-  cagg[q] = st ? int32_t(c * 32 + 31 - __clz(int(st))) : -1;
-  ntile[q] = ge && f <= sg.D - d ? 1u : 0u;
-}
-
-// One block per segment: bucket start of each chunk's first rank (exclusive
-// max-scan of the chunk aggregates) and the number of tiles whose column
-// chunk is this chunk: row chunks from the bucket start's chunk up to itself.
+// One block per segment, a thread per chunk of 32 ranks: the bucket start of
+// each chunk's first rank (an exclusive max-scan of the chunks' last bucket
+// starts), and the tiles whose column chunk is this chunk: row chunks from
+// the bucket start's chunk up to itself, where some rank of the chunk
+// continues the bucket of its predecessor.  ntile gets the tiles before the
+// chunk in its segment, segsum the segment's.  (Chunk values, their scan and
+// the scan of all tiles were four kernels: on short series, where a level
+// is a handful of short launches, they took a quarter of the traversal.)
 __global__ void __launch_bounds__(1024)
-k_chunk_scan(const uint8_t* __restrict__ lcp, Seg sg, int i, const int32_t* __restrict__ cagg,
-             int32_t* __restrict__ cbs, uint64_t* __restrict__ ntile) {
-  __shared__ int32_t wtot[32];
+k_chunk_scan(const uint8_t* __restrict__ lcp, Seg sg, int i, int d, int32_t* __restrict__ cbs,
+             uint64_t* __restrict__ ntile, uint64_t* __restrict__ segsum) {
+  __shared__ int32_t wmax[32];
+  __shared__ uint64_t wsum[32];
   __shared__ int32_t carry_s;
+  __shared__ uint64_t sum_s;
   const int seg = blockIdx.x;
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nwarp = blockDim.x >> 5;
   const uint8_t* L = lcp + sg.base(seg);
   const int64_t off = int64_t(seg) * sg.C;
-  if (threadIdx.x == 0) carry_s = -1;
+  // a pair handled from dim f needs d - 1 more colliding dims above f
+  const bool useful = seg - (seg / sg.D) * sg.D <= sg.D - d;
+  if (threadIdx.x == 0) {
+    carry_s = -1;
+    sum_s = 0;
+  }
   __syncthreads();
   for (int64_t b0 = 0; b0 < sg.C; b0 += blockDim.x) {
-    const int64_t c = b0 + threadIdx.x;
-    int32_t v = c < sg.C ? cagg[off + c] : -1;
-    int32_t incl = v;
+    const int64_t c = b0 + threadIdx.x, p0 = c * 32;
+    const uint32_t ge = c < sg.C ? join_mask(L, p0, sg.M, i) : 0u;
+    const int64_t left = sg.M - p0;
+    const uint32_t st = c < sg.C ? ~ge & (left >= 32 ? ~0u : (1u << left) - 1u) : 0u;
+    int32_t incl = st ? int32_t(p0 + 31 - __clz(int(st))) : -1;
     for (int o = 1; o < 32; o <<= 1) {
-      int32_t u = __shfl_up_sync(0xffffffffu, incl, o);
+      const int32_t u = __shfl_up_sync(0xffffffffu, incl, o);
       if (lane >= o) incl = max(incl, u);
     }
-    if (lane == 31) wtot[wid] = incl;
+    if (lane == 31) wmax[wid] = incl;
     __syncthreads();
-    if (wid == 0) {
-      int32_t t = wtot[lane];
-      for (int o = 1; o < 32; o <<= 1) {
-        int32_t u = __shfl_up_sync(0xffffffffu, t, o);
-        if (lane >= o) t = max(t, u);
-      }
-      wtot[lane] = t;
-    }
-    __syncthreads();
-    const int32_t carry = carry_s;
-    int32_t before = wid ? wtot[wid - 1] : -1;
     int32_t excl = __shfl_up_sync(0xffffffffu, incl, 1);
     if (lane == 0) excl = -1;
-    excl = max(max(excl, before), carry);
-    if (c < sg.C) {
-      const int64_t p0 = c * 32;
-      const int32_t bs = (int(L[p0]) < i) ? int32_t(p0) : excl;
-      cbs[off + c] = bs;
-      const uint64_t has = ntile[off + c];
-      ntile[off + c] = has ? uint64_t(c - bs / 32 + 1) : 0u;
-    }
-    __syncthreads();
-    if (threadIdx.x == 0) carry_s = max(carry, wtot[31]);
-    __syncthreads();
-  }
-}
-
-// Device-wide exclusive scan of n uint64 values in place; v[n] = total.
-constexpr int kScanBlock = 1024;
-__global__ void __launch_bounds__(kScanBlock)
-k_scan_local(uint64_t* __restrict__ v, int64_t n, uint64_t* __restrict__ bsum) {
-  __shared__ uint64_t wt[32];
-  const int64_t q = blockIdx.x * int64_t(kScanBlock) + threadIdx.x;
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  uint64_t x = q < n ? v[q] : 0;
-  uint64_t incl = x;
-  for (int o = 1; o < 32; o <<= 1) {
-    uint64_t u = __shfl_up_sync(0xffffffffu, incl, o);
-    if (lane >= o) incl += u;
-  }
-  if (lane == 31) wt[wid] = incl;
-  __syncthreads();
-  if (wid == 0) {
-    uint64_t t = wt[lane];
+    int32_t wm = lane < nwarp ? wmax[lane] : -1;                 // every warp scans the warps' values
     for (int o = 1; o < 32; o <<= 1) {
-      uint64_t u = __shfl_up_sync(0xffffffffu, t, o);
-      if (lane >= o) t += u;
+      const int32_t u = __shfl_up_sync(0xffffffffu, wm, o);
+      if (lane >= o) wm = max(wm, u);
     }
-    wt[lane] = t;
+    const int32_t carry = carry_s;
+    const int32_t warps_before = __shfl_sync(0xffffffffu, wm, wid ? wid - 1 : 0);
+    if (wid) excl = max(excl, warps_before);
+    excl = max(excl, carry);
+    const int32_t last = max(carry, __shfl_sync(0xffffffffu, wm, 31));
+    const int32_t bs = (st & 1u) ? int32_t(p0) : excl;
+    const uint64_t mine = ge && useful ? uint64_t(c - bs / 32 + 1) : 0u;
+    uint64_t run = mine;
+    for (int o = 1; o < 32; o <<= 1) {
+      const uint64_t u = __shfl_up_sync(0xffffffffu, run, o);
+      if (lane >= o) run += u;
+    }
+    if (lane == 31) wsum[wid] = run;
+    __syncthreads();
+    uint64_t ws = lane < nwarp ? wsum[lane] : 0u;
+    for (int o = 1; o < 32; o <<= 1) {
+      const uint64_t u = __shfl_up_sync(0xffffffffu, ws, o);
+      if (lane >= o) ws += u;
+    }
+    const uint64_t prev = __shfl_sync(0xffffffffu, ws, wid ? wid - 1 : 0);
+    const uint64_t before = sum_s + (wid ? prev : 0u), total = sum_s + __shfl_sync(0xffffffffu, ws, 31);
+    if (c < sg.C) {
+      cbs[off + c] = bs;
+      ntile[off + c] = before + run - mine;
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+      carry_s = last;
+      sum_s = total;
+    }
+    __syncthreads();
   }
-  __syncthreads();
-  uint64_t before = wid ? wt[wid - 1] : 0;
-  if (q < n) v[q] = before + incl - x;
-  if (threadIdx.x == kScanBlock - 1) bsum[blockIdx.x] = before + incl;
+  if (threadIdx.x == 0) segsum[seg] = sum_s;
 }
 
+// Exclusive scan of the segments' totals in place; *total_out = their sum.
+constexpr int kScanBlock = 1024;
 __global__ void __launch_bounds__(kScanBlock)
 k_scan_top(uint64_t* __restrict__ bsum, int64_t nb, uint64_t* __restrict__ total_out) {
   __shared__ uint64_t wt[32];
@@ -198,9 +182,11 @@ k_scan_top(uint64_t* __restrict__ bsum, int64_t nb, uint64_t* __restrict__ total
   if (threadIdx.x == 0) *total_out = carry_s;
 }
 
-__global__ void k_scan_add(uint64_t* __restrict__ v, int64_t n, const uint64_t* __restrict__ bsum) {
-  const int64_t q = blockIdx.x * int64_t(kScanBlock) + threadIdx.x;
-  if (q < n) v[q] += bsum[blockIdx.x];
+// The segments' offsets added to their chunks'.
+__global__ void k_scan_add(uint64_t* __restrict__ v, int C, const uint64_t* __restrict__ segsum) {
+  const uint64_t base = segsum[blockIdx.y];
+  uint64_t* row = v + int64_t(blockIdx.y) * C;
+  for (int q = blockIdx.x * blockDim.x + threadIdx.x; q < C; q += gridDim.x * blockDim.x) row[q] += base;
 }
 
 struct CollideArgs {
@@ -949,13 +935,12 @@ cudaError_t launch_collide(const Index& ix, int i, int j0, int j1, int d, const 
   Seg sg{ix.M, ix.D, j0, int(C)};
   const int64_t E = int64_t(segs) * C;
   uint64_t* toff = cs.ntile;
-  MOMENTI_LAUNCH("chunk_agg", s, k_chunk_agg<<<unsigned((E + 255) / 256), 256, 0, s>>>(ix.lcp, sg, segs, i, d, cs.cagg, toff));
-  MOMENTI_LAUNCH("chunk_scan", s, k_chunk_scan<<<segs, 1024, 0, s>>>(ix.lcp, sg, i, cs.cagg, cs.cbs, toff));
-  const int64_t nb = (E + kScanBlock - 1) / kScanBlock;
-  uint64_t* bsum = cs.scan_tmp;
-  MOMENTI_LAUNCH("scan_local", s, k_scan_local<<<unsigned(nb), kScanBlock, 0, s>>>(toff, E, bsum));
-  MOMENTI_LAUNCH("scan_top", s, k_scan_top<<<1, kScanBlock, 0, s>>>(bsum, nb, toff + E));
-  MOMENTI_LAUNCH("scan_add", s, k_scan_add<<<unsigned(nb), kScanBlock, 0, s>>>(toff, E, bsum));
+  uint64_t* segsum = cs.scan_tmp;
+  const unsigned bt = unsigned(std::min<int64_t>(1024, (C + 31) / 32 * 32));
+  MOMENTI_LAUNCH("chunk_scan", s, k_chunk_scan<<<segs, bt, 0, s>>>(ix.lcp, sg, i, d, cs.cbs, toff, segsum));
+  MOMENTI_LAUNCH("scan_top", s, k_scan_top<<<1, kScanBlock, 0, s>>>(segsum, segs, toff + E));
+  dim3 ga{unsigned(std::min<int64_t>((C + 255) / 256, 64)), unsigned(segs), 1u};
+  MOMENTI_LAUNCH("scan_add", s, k_scan_add<<<ga, 256, 0, s>>>(toff, int(C), segsum));
   CollideArgs g{ix.order, ix.lcp, ix.keys, sg, segs, i, ix.K, d, ix.excl, cs.cbs, toff, hs,
                 cs.events, cs.ev_cap, cs.counters, out_pairs, out_cap};
   const int G = (ix.D + 7) / 8;

@@ -1119,10 +1119,9 @@ static int hash_all_impl(momenti_handle* h, const void* series, int32_t dtype, i
     cs.seg_cap = int64_t(chunk) * D;
     cs.chunk_cap = C;
     const int64_t E = cs.seg_cap * C;
-    CK(dalloc(h, &cs.cagg, size_t(E)));
     CK(dalloc(h, &cs.cbs, size_t(E)));
     CK(dalloc(h, &cs.ntile, size_t(E + 1)));
-    CK(dalloc(h, &cs.scan_tmp, size_t(E / 1024 + 2)));
+    CK(dalloc(h, &cs.scan_tmp, size_t(cs.seg_cap + 1)));
     CK(dalloc(h, &cs.counters, 8));
     h->rec_cap = new_cap;
     CK(dalloc(h, &h->rec_dev, size_t(new_cap)));
