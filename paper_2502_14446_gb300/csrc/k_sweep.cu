@@ -780,21 +780,23 @@ int64_t sw_gy(const SweepView& v) {
 }
 
 // Rows per block.  A block pays a direct start of w points (about 22
-// issue slots each) before its rows (about 78 each); a launch runs about
-// three blocks per SM at a time.  Long blocks where there are many of
-// them, shorter ones where a wave would not be filled.
+// issue slots each) before its rows (about 78 each); a launch runs two or
+// three blocks per SM at a time.  Long blocks where there are many of them
+// (8192 rows at n = 2e5, D = 32, w = 500: 128 ms against 140 with 2048; the
+// error of C grows with the root of the rows, 1e-5 in the correlation there),
+// shorter ones where waves would be partly empty.
 int sw_seg(const SweepView& v) {
   const int64_t slots = int64_t(sm_count()) * (v.P == 2 ? kSwBlocks<2> : kSwBlocks<1>), nd = sw_diags(v.G), gy = sw_gy(v);
   int best = 2048;
   double best_cost = 1e300;
-  for (int seg = 2048; seg >= 32; seg >>= 1) {
+  for (int seg = 8192; seg >= 32; seg >>= 1) {
     int64_t blocks = 0;
     for (int64_t by = 0; by < gy; ++by) {
       const int64_t d0 = ((int64_t(v.excl) + 1) & ~int64_t(7)) + by * nd;
       blocks += std::max<int64_t>(0, (v.M - d0 + seg - 1) / seg);
     }
     const double waves = std::max(1.0, double(blocks) / double(slots));
-    const double cost = (waves > 4.0 ? waves : std::ceil(waves)) * (22.0 * v.w + 78.0 * seg);
+    const double cost = (waves > 16.0 ? waves : std::ceil(waves)) * (22.0 * v.w + 78.0 * seg);
     if (cost < best_cost) {
       best_cost = cost;
       best = seg;
