@@ -734,12 +734,13 @@ int exact_path(momenti_handle* h, int d, double tau0, momenti_motif* out, int32_
   // sample: first about 2^20 pairs of all distances, then, where `want`
   // pairs are fewer than that sample resolves, a fraction holding about 24
   // of them, swept below the first sample's edge (small blocks: close pairs
-  // come in clusters).  Where even that edge
-  // sends four groups of rows out of five through the slow branch (many
-  // dimensions, or a d whose background distances are close), a sweep at 5%
-  // of the largest possible distance costs a quarter of one at the edge and
-  // holds the motifs whenever they stand out, so it goes first (the wide
-  // workload: 149 ms against 570).  Any edge gives the same result; one that
+  // come in clusters).  A sweep at 5% of the largest possible distance takes
+  // no slow branch and holds the motifs whenever they stand out, so it goes
+  // first where the background lies far above it (without TOP's k-th: where
+  // the first sample's edge is 2.5 times as far, and the fine sample waits
+  // until it is needed), or where even the sampled edge sends four groups
+  // of rows out of five through the slow branch (the wide workload: 149 ms
+  // against 570).  Any edge gives the same result; one that
   // holds fewer than k motifs is followed by the next.
   const double n_pairs = 0.5 * double(ix.M - ix.excl) * double(ix.M - ix.excl - 1);
   const double want = 2048.0 + double(k) * std::max(64.0, double(ix.w) * double(ix.w) / 256.0);
@@ -779,6 +780,15 @@ int exact_path(momenti_handle* h, int d, double tau0, momenti_motif* out, int32_
     }
     return MOMENTI_OK;
   };
+  const float far = float(2.0 * std::sqrt(double(ix.w)) * d), low = 0.05f * far;
+  float fine_edge = 0.f;                           // the fine sample's edge, still to be run
+  auto fine_sample = [&](float edge) -> int {
+    float ea = 0.f, eb = 0.f;
+    const int r = sample(edge, std::min(1.0 / 32.0, 24.0 / want), 32, want, 16.0 * want, &ea, &eb);
+    hi = std::min(edge, ea);
+    hi_next = std::min(edge, eb);
+    return r;
+  };
   const double kSample = double(1 << 20), sweep_work = n_pairs * double(ix.D);
   if (n_pairs > 0.25 * kSample && (!(tau0 > 0) || sweep_work > 2e8)) {
     float edge = hi_top;
@@ -793,17 +803,18 @@ int exact_path(momenti_handle* h, int d, double tau0, momenti_motif* out, int32_
         hi = edge;
         hi_next = std::min(hi_top, eb);
       }
+      groups[0] = groups[1] = 0;                   // of no edge that a sweep would take
     }
-    if (fine) {
-      float ea = 0.f, eb = 0.f;
-      const int r = sample(edge, std::min(1.0 / 32.0, 24.0 / want), 32, want, 16.0 * want, &ea, &eb);
+    if (fine && !(tau0 > 0) && edge > 2.5f * low) {
+      hi = low;                                    // first, and the fine sample only if it holds too few
+      fine_edge = edge;
+    } else if (fine) {
+      const int r = fine_sample(edge);
       if (r != MOMENTI_OK) return r;
-      hi = std::min(edge, ea);
-      hi_next = std::min(edge, eb);
     }
   }
-  const float far = float(2.0 * std::sqrt(double(ix.w)) * d), low = 0.05f * far;
-  if (groups[1] * 5 > groups[0] * 4 && hi > 2.f * low && (!(tau0 > 0) || float(tau0) > 0.25f * far)) {
+  if (groups[1] * 5 > groups[0] * 4 && fine_edge == 0.f && hi > 2.f * low &&
+      (!(tau0 > 0) || float(tau0) > 0.25f * far)) {
     hi_next = hi;
     hi = low;
   }
@@ -887,6 +898,14 @@ int exact_path(momenti_handle* h, int d, double tau0, momenti_motif* out, int32_
       break;
     }
     lo = hi;
+    if (fine_edge > 0.f) {                         // the low start held too few
+      const int r = fine_sample(fine_edge);
+      if (r != MOMENTI_OK) return r;
+      fine_edge = 0.f;
+      hi_next = std::max(hi, hi_next);
+      if (hi > lo * 1.01f) continue;
+      hi = lo;
+    }
     // the next sample edge, TOP's k-th (which holds all k), then twice as far
     if (hi_next > hi * 1.01f) hi = hi_next;
     else if (hi_top > hi && tau0 > 0) hi = hi_top;
