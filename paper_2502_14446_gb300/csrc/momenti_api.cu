@@ -299,6 +299,9 @@ class SweepBatcher {
       for (Req* q : batch)
         if (e == cudaSuccess) e = cudaStreamWaitEvent(q->s, ev, 0);
       if (e == cudaSuccess) e = cudaStreamSynchronize(stream_);
+      // a failed batch may have started a launch: it ends before the
+      // requesters give their tables and record buffers back
+      else if (stream_) cudaStreamSynchronize(stream_);
     } catch (...) {
       if (stream_) cudaStreamSynchronize(stream_);
       e = cudaErrorMemoryAllocation;
