@@ -283,10 +283,10 @@ struct ApRec {
 
 // ---- k_sweep.cu ---------------------------------------------------------
 // The sweep's view of an index: its table (k_sweep.cu: df, dg and sigma per
-// window, in planes of transposed 64-window blocks), the series' points in the same
+// window, in planes of transposed 64-window blocks, then 1/sigma), the series' points in the same
 // order, and the window means.
 struct SweepView {
-  const void* tab = nullptr;     // [Mpad / 64][3][64][G] vectors of 2 P dims
+  const void* tab = nullptr;     // [Mpad / 64][3][64][G] vectors of 2 P dims, then [Mpad][G]
   const void* xp = nullptr;      // [npad][G]
   const void* xl = nullptr;      // [npad][G] low parts, float64 input only
   const double* mu = nullptr;    // [D][M]

@@ -82,7 +82,9 @@ __host__ __device__ __forceinline__ int64_t sw_pos(int64_t b) {
 // Offset of window b in the table, in units of G vectors: blocks of 64
 // windows with their df, dg and sigma planes (64 units each) one after
 // another, so that a warp's load of one kind touches whole cache lines (12
-// lines a load when the three lay together: L1 was the limit).
+// lines a load when the three lay together: L1 was the limit).  1/sigma, which
+// only the queued pairs need, follows in an array of its own, ordered by
+// sw_pos.
 __host__ __device__ __forceinline__ int64_t sw_off(int64_t b) {
   return (b >> 6) * 192 + ((b & 7) << 3) + ((b >> 3) & 7);
 }
@@ -111,8 +113,9 @@ size_t sw_smem(int G) {
 }
 size_t sw_smem(const SweepView& v) { return v.P == 2 ? sw_smem<2>(v.G) : sw_smem<1>(v.G); }
 
-// Table of an index: per window and group of 4 dims {df x4, dg x4, sigma x4};
-// per point the 4 values (and their low parts for float64 input).  A block
+// Table of an index: per window and group of 2 P dims {df, dg, sigma,
+// 1/sigma}, each computed in float64 and rounded once; per point the values
+// (and their low parts for float64 input).  A block
 // builds 64 windows and points: first the marks (one warp per dim, the
 // level change bounded by the range of the means before the exact scan of
 // the 256 windows before it), then the records.
@@ -160,13 +163,13 @@ __global__ void __launch_bounds__(256) k_sweep_table(Index ix, SweepView v, SwVe
     const int c = q & 63, g = q >> 6;
     const int64_t b = B + c;
     const bool in = b < M;
-    SwVec<P> df, dg, sg, xh, xlo;
+    SwVec<P> df, dg, sg, is, xh, xlo;
 #pragma unroll
     for (int e = 0; e < 2 * P; ++e) {
       const int f = 2 * P * g + e;
       float vdf = 0.f, vdg = 0.f, vx = 0.f, vl = 0.f;
       // past the last window: a sigma no correlation reaches; no such dim: 0
-      float vs = f < ix.D ? 1e30f : 0.f;
+      float vs = f < ix.D ? 1e30f : 0.f, vi = f < ix.D ? 1e-30f : INFINITY;
       if (f < ix.D) {
         const float* h = ix.xs_hi + int64_t(f) * n;
         const float* l = ix.has_lo ? ix.xs_lo + int64_t(f) * n : nullptr;
@@ -177,17 +180,19 @@ __global__ void __launch_bounds__(256) k_sweep_table(Index ix, SweepView v, SwVe
             vdf = float(0.5 * (xi - xo));
             vdg = float((xi - ix.mu[int64_t(f) * M + b]) + (xo - ix.mu[int64_t(f) * M + b - 1]));
           }
-          vs = mark[c] ? __int_as_float(0x7fc00000) : float(ix.sig[int64_t(f) * M + b]);
+          const double sd = ix.sig[int64_t(f) * M + b];
+          vs = mark[c] ? __int_as_float(0x7fc00000) : float(sd);
+          vi = mark[c] ? vs : float(1.0 / sd);
         }
         if (b < n) {
           vx = h[b];
           if (l) vl = l[b];
         }
       }
-      float2* o[5] = {&df.v[e / 2], &dg.v[e / 2], &sg.v[e / 2], &xh.v[e / 2], &xlo.v[e / 2]};
-      const float val[5] = {vdf, vdg, vs, vx, vl};
+      float2* o[6] = {&df.v[e / 2], &dg.v[e / 2], &sg.v[e / 2], &is.v[e / 2], &xh.v[e / 2], &xlo.v[e / 2]};
+      const float val[6] = {vdf, vdg, vs, vi, vx, vl};
 #pragma unroll
-      for (int k = 0; k < 5; ++k) {
+      for (int k = 0; k < 6; ++k) {
         if (e & 1) o[k]->y = val[k];
         else o[k]->x = val[k];
       }
@@ -198,6 +203,7 @@ __global__ void __launch_bounds__(256) k_sweep_table(Index ix, SweepView v, SwVe
       t[0] = df;
       t[64 * G] = dg;
       t[128 * G] = sg;
+      tab[3 * v.Mpad * G + p] = is;
     }
     if (b < v.npad) {
       xp[p] = xh;
@@ -246,13 +252,13 @@ __device__ __forceinline__ void sort_desc(float (&c)[N]) {
       }
 }
 
-// dist_d of one hit from its correlations (less yl): the sum of the
-// distances of the d largest.  N >= D values in registers.
+// dist_d of one hit from its correlations: the sum of the distances of the d
+// largest.  N >= D values in registers.
 template <int N>
-__device__ __forceinline__ float sw_dist(const float* e, int D, int d, float yl, float wf) {
+__device__ __forceinline__ float sw_dist(const float* e, int D, int d, float wf) {
   float c[N];
 #pragma unroll
-  for (int f = 0; f < N; ++f) c[f] = f < D ? e[f] + yl : -INFINITY;
+  for (int f = 0; f < N; ++f) c[f] = f < D ? e[f] : -INFINITY;
   sort_desc<N>(c);
   float sm = 0.f;
 #pragma unroll
@@ -270,6 +276,13 @@ __device__ __forceinline__ float sw_dist(const float* e, int D, int d, float yl,
 // At q = 1.5 this passes a tenth of the pairs that have one dimension
 // within thr / d on the sensor workload (0.3 % against 3.3 %); for d = 1,
 // where the one-dimension test is the exact one, q is near 1.
+//
+// Both tests are necessary conditions of the distance that is recorded: they
+// give way by more than that distance's rounding (kSwSlack in the
+// correlation: a few units in the last place of values up to 2, from the
+// product, the square root and the sum), so that what a sweep records
+// depends on the distance alone and consecutive slices leave no pair out.
+constexpr float kSwSlack = 2e-6f;
 struct SwJoint {
   float yl, need;
 };
@@ -278,7 +291,7 @@ __device__ __forceinline__ SwJoint sw_joint(const SweepJob* jb) {
   const float lam = q * jb->thr / float(jb->d);
   SwJoint j;
   j.yl = 1.f - lam * lam / (2.f * float(jb->v.w));
-  j.need = (float(jb->d) * (1.f - 1.f / q) - 1e-3f) * (1.f - j.yl);
+  j.need = (float(jb->d) * (1.f - 1.f / q) - 1e-3f) * (1.f - j.yl) - kSwSlack * float(jb->v.D);
   return j;
 }
 
@@ -291,7 +304,7 @@ __device__ __noinline__ int sw_drain(const SweepJob* jb, float* queue, int qn, b
   const SweepView& v = jb->v;
   const int lane = threadIdx.x & 31;
   const int D = v.D, d = jb->d, QS = sw_entry<P>(v.G);
-  const float thr = jb->thr, wf = float(v.w), yl = sw_joint(jb).yl;
+  const float thr = jb->thr, wf = float(v.w);
   __syncwarp();
   while (qn >= 32 || (all && qn > 0)) {
     const int n = min(32, qn);
@@ -302,8 +315,8 @@ __device__ __noinline__ int sw_drain(const SweepJob* jb, float* queue, int qn, b
       if (int64_t(b) < v.M && int64_t(b) - int64_t(a) > int64_t(v.excl)) {
         float sm = 0.f;
         if (!isnan(e[0])) {
-          if (D <= 8) sm = sw_dist<8>(e, D, d, yl, wf);
-          else if (D <= 16) sm = sw_dist<16>(e, D, d, yl, wf);
+          if (D <= 8) sm = sw_dist<8>(e, D, d, wf);
+          else if (D <= 16) sm = sw_dist<16>(e, D, d, wf);
           else {
             for (int q = 0; q < d && sm <= thr; ++q) {
               float best = -INFINITY;
@@ -316,7 +329,7 @@ __device__ __noinline__ int sw_drain(const SweepJob* jb, float* queue, int qn, b
                 }
               }
               e[at] = -INFINITY;
-              sm += sqrtf(fmaxf(2.f * wf * (1.f - (best + yl)), 0.f));
+              sm += sqrtf(fmaxf(2.f * wf * (1.f - best), 0.f));
             }
           }
         }
@@ -401,7 +414,8 @@ __device__ __forceinline__ void sw_cols(const SwVec<P>* tab, int64_t b0, int G, 
 // again from its start (the cross products in ck), up to its last hot row
 // (bits of hot), with the joint test in the hot rows: the correlations of
 // the lane's dims, their part of the sum, the sum over the
-// diagonal's lanes.  Passing pairs go to the queue, one entry per pair.
+// diagonal's lanes.  Passing pairs go to the queue, one entry per pair, with
+// their correlations (which depend on no threshold).
 // Returns the queue's length.  Two rows per turn, with the columns moved
 // along in registers: unrolled over all 8 rows, the code fell out of the
 // instruction cache (a sweep of n = 2e4 at a
@@ -412,14 +426,16 @@ __device__ __noinline__ int sw_redo(const SweepJob* jb, const SwVec<P>* rows, Sw
   const int G = GT ? GT : jb->v.G, QS = sw_entry<P>(G), lane = threadIdx.x & 31;
   const SwLane L = sw_lane(G);
   const SwVec<P>* tab = static_cast<const SwVec<P>*>(jb->v.tab);
-  const float wf = float(jb->v.w);
+  const SwVec<P>* inv = tab + 3 * jb->v.Mpad * G + L.g;          // 1 / sigma
+  const float wf = float(jb->v.w), iw = 1.f / wf;
   const SwJoint J = sw_joint(jb);
   const float2 nyl = make_float2(-J.yl, -J.yl);
   int top = 0;                                                   // the largest power of two below G
   for (int o = 1; o < G; o <<= 1) top = o;
   float2 C[kSwR][P];
   SwVec<P> df[kSwR + 1], dg[kSwR + 1], ib[kSwR + 1];             // columns b + i .. b + i + 8; ib: 1 / sigma
-  auto inv = [](const SwVec<P>& s) {
+  // the test's own quotients, to two units in the last place
+  auto quot = [](const SwVec<P>& s) {
     SwVec<P> o;
 #pragma unroll
     for (int p = 0; p < P; ++p) o.v[p] = make_float2(__fdividef(1.f, s.v[p].x), __fdividef(1.f, s.v[p].y));
@@ -431,7 +447,7 @@ __device__ __noinline__ int sw_redo(const SweepJob* jb, const SwVec<P>* rows, Sw
   auto load = [&](const SwVec<P>* p0, int slot) {
     df[slot] = p0[0];
     dg[slot] = p0[64 * G];
-    ib[slot] = inv(p0[128 * G]);
+    ib[slot] = quot(p0[128 * G]);
   };
 #pragma unroll
   for (int r = 0; r < kSwR; ++r) {
@@ -458,19 +474,18 @@ __device__ __noinline__ int sw_redo(const SweepJob* jb, const SwVec<P>* rows, Sw
       SwVec<P> ws = rows[2 * G];
 #pragma unroll
       for (int p = 0; p < P; ++p) ws.v[p] = make_float2(wf * ws.v[p].x, wf * ws.v[p].y);
-      const SwVec<P> ia = inv(ws);                               // 1 / (w sigma_a)
-      float2 y[kSwR][P];
+      const SwVec<P> ia = quot(ws);                              // 1 / (w sigma_a)
       float sum[kSwR];
       uint32_t hit = 0;
 #pragma unroll
       for (int r = 0; r < kSwR; ++r) {
-        float2 part = make_float2(0.f, 0.f);
+        float2 part = make_float2(0.f, 0.f), y[P];
 #pragma unroll
         for (int p = 0; p < P; ++p) {
-          y[r][p] = __ffma2_rn(__fmul2_rn(C[r][p], ib[h + r].v[p]), ia.v[p], nyl);
-          part = __fadd2_rn(part, make_float2(fmaxf(y[r][p].x, 0.f), fmaxf(y[r][p].y, 0.f)));
+          y[p] = __ffma2_rn(__fmul2_rn(C[r][p], ib[h + r].v[p]), ia.v[p], nyl);
+          part = __fadd2_rn(part, make_float2(fmaxf(y[p].x, 0.f), fmaxf(y[p].y, 0.f)));
         }
-        sum[r] = fmaf(0.f, y[r][0].x, part.x + part.y);          // NaN (an unresolvable window) stays NaN
+        sum[r] = fmaf(0.f, y[0].x, part.x + part.y);             // NaN (an unresolvable window) stays NaN
       }
       if (G == 2) {                                              // over the diagonal's lanes
 #pragma unroll
@@ -493,11 +508,13 @@ __device__ __noinline__ int sw_redo(const SweepJob* jb, const SwVec<P>* rows, Sw
       uint32_t rmask = __reduce_or_sync(0xffffffffu, hit);
       if (!rmask) continue;
       __syncwarp();
+      const SwVec<P> sa = inv[sw_pos(a + i) * G];
 #pragma unroll
-      for (int r = 0; r < kSwR; ++r) {                           // the checkpoint has been read: room for y
-        SwVec<P> c;
+      for (int r = 0; r < kSwR; ++r) {                           // the checkpoint has been read: room for the correlations
+        SwVec<P> c = inv[sw_pos(b + i + r) * G];
 #pragma unroll
-        for (int p = 0; p < P; ++p) c.v[p] = y[r][p];
+        for (int p = 0; p < P; ++p)
+          c.v[p] = __fmul2_rn(__fmul2_rn(C[r][p], c.v[p]), __fmul2_rn(sa.v[p], make_float2(iw, iw)));
         ck[r * 32 + lane] = c;
       }
 #pragma unroll 1
@@ -656,7 +673,7 @@ __device__ __forceinline__ void sw_block(const SweepJob* jb, int64_t bx, int64_t
     ck[r * 32 + lane] = c;
   }
   const float t1 = jb->thr / float(jb->d);
-  const float nk = -(1.f - t1 * t1 / (2.f * float(w))) * float(w);
+  const float nk = -(1.f - t1 * t1 / (2.f * float(w)) - kSwSlack) * float(w);
   const float2 nk2 = make_float2(nk, nk);
   int qn = 0, cb = 0, redone = 0;   // queued hits, this group's checkpoint, groups run twice
   const int nstage = (nrow + RS - 1) / RS;
@@ -810,13 +827,13 @@ int sw_seg(const SweepView& v) {
 size_t sweep_table_bytes(const Index& ix) {
   const int P = sw_pairs(ix.D);
   const size_t G = size_t((ix.D + 2 * P - 1) / (2 * P));
-  return (size_t(sw_round(ix.M)) * 3 + size_t(sw_round(ix.n)) * (ix.has_lo ? 2 : 1)) * G * (8 * size_t(P));
+  return (size_t(sw_round(ix.M)) * 4 + size_t(sw_round(ix.n)) * (ix.has_lo ? 2 : 1)) * G * (8 * size_t(P));
 }
 
 template <int P>
 static cudaError_t sweep_table(const Index& ix, SweepView& v, void* buf, cudaStream_t s) {
   SwVec<P>* tab = static_cast<SwVec<P>*>(buf);
-  SwVec<P>* xp = tab + v.Mpad * v.G * 3;
+  SwVec<P>* xp = tab + v.Mpad * v.G * 4;
   SwVec<P>* xl = ix.has_lo ? xp + v.npad * v.G : nullptr;
   v.tab = tab;
   v.xp = xp;
