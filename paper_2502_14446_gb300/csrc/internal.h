@@ -267,7 +267,7 @@ cudaError_t launch_verify_pairs(const Index& ix, int d, const uint64_t* pairs, i
                                 int fp64, double* per_dim, double* dist_d, uint64_t* dims,
                                 cudaStream_t s);
 // Output of an all-pairs sweep: pairs whose approximate dist_d (float32
-// Pearson form, within 1% + 0.01 of the exact value) lies in (lo, thr]
+// Pearson form, at most 1% + 0.01 above the exact value) lies in (lo, thr]
 // go to out / out_d while count < cap; count counts them all and hist
 // (kApBins bins over (lo, thr], may be NULL) their distribution.
 constexpr int kApBins = 4096;
@@ -284,12 +284,14 @@ struct ApRec {
 // ---- k_sweep.cu ---------------------------------------------------------
 // The sweep's view of an index: its table (k_sweep.cu: df, dg and sigma per
 // window, in planes of transposed 64-window blocks, then 1/sigma), the series' points in the same
-// order, and the window means.
+// order, the cuts, and the window means and deviations.
 struct SweepView {
   const void* tab = nullptr;     // [Mpad / 64][3][64][G] vectors of 2 P dims, then [Mpad][G]
   const void* xp = nullptr;      // [npad][G]
   const void* xl = nullptr;      // [npad][G] low parts, float64 input only
+  const uint8_t* cut = nullptr;  // [Mpad] nonzero: at a cut, C of the recurrence starts anew after it
   const double* mu = nullptr;    // [D][M]
+  const double* sig = nullptr;   // [D][M]
   int64_t M = 0, Mpad = 0, npad = 0;
   int D = 0, P = 0, G = 0;       // dims, pairs of dims per lane, lanes per diagonal
   int w = 0, excl = 0;

@@ -17,7 +17,7 @@
 // rounded (k_sweep_table), so a pair and dimension costs two FMA for the
 // recurrence and one for the threshold test, and nothing of the state
 // depends on the series' level: it is C itself, in float32, restarted
-// directly every `seg` rows.  Its error per step is one rounding of C and
+// directly every `seg` rows and after every cut.  Its error per step is one rounding of C and
 // of the two products; a form that slides products centred on a constant
 // carries those and the centring offset's on top.
 //
@@ -40,15 +40,15 @@
 // of 64 windows transposed (8 x 8), so that they are consecutive.
 //
 // What bounds it (D = 8, w = 300, 5e9 pairs, edge below the background):
-// 7.3 ms, 5.5 pair-dimensions per cycle and scheduler of the 10.7 that three
+// 7.6 ms, 5.2 pair-dimensions per cycle and scheduler of the 10.7 that three
 // FMA on the FP32 lanes allow; 8 warps per SM, fixed-latency dependencies
 // first.  The form before, one diagonal per lane sliding centred products,
 // took 35.6 ms; at D = 32, w = 500, n = 2e5, 145 against 848 ms.
 //
-// Windows that the float32 test cannot resolve (flat, or with a level
-// change of more than about 100 sigma within the last 256 windows) have
-// sigma = NaN in the table: their tests give NaN, whose sign bit is clear,
-// so they always reach the slow branch, which takes them as candidates.
+// Windows that C cannot resolve (flat ones, and the 7 where the series falls
+// quiet: k_sweep_cuts) have sigma = NaN in the table: their tests give NaN,
+// whose sign bit is clear, so they always reach the slow branch, which
+// computes their pairs directly and starts C again after a cut.
 #include "internal.h"
 
 #include <algorithm>
@@ -62,7 +62,7 @@ constexpr int kSwThreads = 128;
 constexpr int kSwWarps = kSwThreads / 32;
 constexpr int kSwR = 8;                 // diagonals per lane
 constexpr int kSwPad = 2048;            // records after the last window / point
-constexpr int kSwFlagBack = 256;        // windows looked back at for the level-change mark
+constexpr int kSwSegMax = 2048;         // most rows between direct starts
 
 // P pairs of dims: 2 P floats of one kind, loaded with one instruction.
 template <int P>
@@ -113,52 +113,98 @@ size_t sw_smem(int G) {
 }
 size_t sw_smem(const SweepView& v) { return v.P == 2 ? sw_smem<2>(v.G) : sw_smem<1>(v.G); }
 
+// Error of the recurrence.  C is a float32 running sum: what is rounded away
+// in a loud stretch stays when both windows have become quiet.  Between a
+// direct start and window x the rounding of C, relative to w sigma_a sigma_b,
+// stays below kSwErr e_a e_b with
+//   e_x^4 = sum of sigma^4 over the windows since the start / sigma_x^4
+// (a rounding step is at most 2^-24 of |C| <= w sigma_a sigma_b; steps add in
+// squares, and Cauchy-Schwarz parts the two windows; emulated in float32 on
+// walks, noise, sinusoids, spikes and repeated stretches at w = 50 to 1000:
+// at most 2.7 2^-24 e_a e_b).  Three things keep it harmless, all decided per
+// window here, so that they depend on no pass and no block:
+//   - sigma is stored less kappa = kSwErr (e^2 + sqrt w) of itself (the root:
+//     the direct start's own error), so that a pair's correlation, and with it
+//     its recorded distance, errs to the near side;
+//   - where e would exceed kSwLoud (sum over at least the 2047 windows back),
+//     the sum starts anew and the window is a cut: the sweep starts C again
+//     after the 8-row group in which a cut falls (walks reach e = 47, even
+//     noise 8: no cuts there);
+//   - the rest of such a group still has the old C, so a cut and the 6 windows
+//     after it have sigma = NaN and their pairs are computed directly.
+// One warp per dimension and 256 windows (a warp's scan is serial: 2048 took
+// 90 us); the sum starts with that of the 2048 windows before, whatever cuts
+// lie there.  kappa goes where 1/sigma will lie.  With the table 0.12 ms at
+// D = 8, n = 1e5 (0.05 without).
+constexpr float kSwErr = 4.f / 16777216.f;
+constexpr double kSwLoud = 64.0;
+constexpr int kSwCutRun = 256;
+template <int P>
+__global__ void __launch_bounds__(128) k_sweep_cuts(Index ix, SweepView v, float* __restrict__ kap,
+                                                    uint8_t* __restrict__ cut) {
+  const int lane = threadIdx.x & 31, f = blockIdx.y;
+  const int64_t M = ix.M, x0 = (blockIdx.x * int64_t(4) + (threadIdx.x >> 5)) * kSwCutRun;
+  if (x0 >= M) return;                           // warp-uniform
+  const double* sig = ix.sig + int64_t(f) * M;
+  const float* isg = ix.inv_sig + int64_t(f) * M;
+  auto fourth = [&](int64_t x) {                 // flat windows have no part in this: they are always computed directly
+    const double s2 = isg[x] == 0.f ? 0.0 : sig[x] * sig[x];
+    return s2 * s2;
+  };
+  double S = 0.0;                                // since the last cut
+  #pragma unroll 8
+  for (int64_t x = max(int64_t(0), x0 - kSwSegMax) + lane; x < x0; x += 32) S += fourth(x);
+  for (int o = 16; o > 0; o >>= 1) S += __shfl_xor_sync(0xffffffffu, S, o);
+  const double limit = kSwLoud * kSwLoud * kSwLoud * kSwLoud;
+  const int64_t x1 = min(M, x0 + kSwCutRun);
+  for (int64_t xb = x0; xb < x1; xb += 32) {
+    const int64_t x = xb + lane;
+    const double q = x < x1 ? fourth(x) : 0.0;
+    double part = q, run = 0.0;                  // lanes before the last cut: 0
+    int from = 0;
+    for (;;) {
+      double p = part;
+      for (int o = 1; o < 32; o <<= 1) {
+        const double u = __shfl_up_sync(0xffffffffu, p, o);
+        if (lane >= o) p += u;
+      }
+      if (lane >= from) run = S + p;
+      const uint32_t loud = __ballot_sync(0xffffffffu, lane >= from && q > 0.0 && run > limit * q);
+      if (!loud) break;
+      const int c = __ffs(int(loud)) - 1;
+      if (lane < 7 && xb + c + lane < M) cut[xb + c + lane] = 1;
+      S = 0.0;                                   // the sum starts anew with window c
+      from = c;
+      if (lane < c) part = 0.0;
+    }
+    if (q > 0.0)
+      kap[(sw_pos(x) * v.G + f / (2 * P)) * (2 * P) + f % (2 * P)] =
+          kSwErr * (sqrtf(float(run / q)) + sqrtf(float(ix.w)));
+    S = __shfl_sync(0xffffffffu, run, 31);
+  }
+}
+
 // Table of an index: per window and group of 2 P dims {df, dg, sigma,
 // 1/sigma}, each computed in float64 and rounded once; per point the values
 // (and their low parts for float64 input).  A block
-// builds 64 windows and points: first the marks (one warp per dim, the
-// level change bounded by the range of the means before the exact scan of
-// the 256 windows before it), then the records.
+// builds 64 windows and points: first the marks (flat in some dim, or at a
+// cut), then the records.
 template <int P>
-__global__ void __launch_bounds__(256) k_sweep_table(Index ix, SweepView v, SwVec<P>* __restrict__ tab,
+__global__ void __launch_bounds__(256) k_sweep_table(Index ix, SweepView v, SwVec<P>* tab,
                                                      SwVec<P>* __restrict__ xp, SwVec<P>* __restrict__ xl) {
   __shared__ int mark[64];
   const int64_t B = int64_t(blockIdx.x) * 64;
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int64_t M = ix.M, n = ix.n;
   if (threadIdx.x < 64) mark[threadIdx.x] = 0;
   __syncthreads();
-  if (B < M) {
-    const int64_t q0 = B > kSwFlagBack ? B - kSwFlagBack : 0, q1 = min(M, B + 64);
-    for (int f = warp; f < ix.D; f += 8) {
-      const float* mh = ix.mu_hi + int64_t(f) * M;
-      float lo = INFINITY, hi = -INFINITY;
-      for (int64_t q = q0 + lane; q < q1; q += 32) {
-        lo = fminf(lo, mh[q]);
-        hi = fmaxf(hi, mh[q]);
-      }
-      for (int o = 16; o > 0; o >>= 1) {
-        lo = fminf(lo, __shfl_xor_sync(0xffffffffu, lo, o));
-        hi = fmaxf(hi, __shfl_xor_sync(0xffffffffu, hi, o));
-      }
-      const double range = double(hi) - double(lo);
-      for (int64_t b = B + lane; b < q1; b += 32) {
-        const double sg = ix.sig[int64_t(f) * M + b], var = sg * sg;
-        bool bad = ix.inv_sig[int64_t(f) * M + b] == 0.f;
-        if (!bad && !(var > 1e-4 * (var + range * range))) {
-          const float mb = mh[b];
-          float dmax = 0.f;
-          for (int64_t q = b > kSwFlagBack ? b - kSwFlagBack : 0; q <= b; ++q)
-            dmax = fmaxf(dmax, fabsf(mh[q] - mb));
-          const double dm = double(dmax);
-          bad = !(var > 1e-4 * (var + dm * dm));
-        }
-        if (bad) atomicOr(&mark[int(b - B)], 1);
-      }
-    }
+  for (int q = threadIdx.x; q < 64 * (ix.D + 1); q += 256) {
+    const int c = q & 63, f = q >> 6;
+    if (B + c >= M) continue;
+    if (f == ix.D ? v.cut[B + c] != 0 : ix.inv_sig[int64_t(f) * M + B + c] == 0.f) atomicOr(&mark[c], 1);
   }
   __syncthreads();
   const int G = v.G;
+  const float* kap = reinterpret_cast<const float*>(tab + 3 * v.Mpad * G);   // replaced by 1/sigma below
   for (int q = threadIdx.x; q < 64 * G; q += 256) {
     const int c = q & 63, g = q >> 6;
     const int64_t b = B + c;
@@ -180,7 +226,8 @@ __global__ void __launch_bounds__(256) k_sweep_table(Index ix, SweepView v, SwVe
             vdf = float(0.5 * (xi - xo));
             vdg = float((xi - ix.mu[int64_t(f) * M + b]) + (xo - ix.mu[int64_t(f) * M + b - 1]));
           }
-          const double sd = ix.sig[int64_t(f) * M + b];
+          const double kappa = mark[c] ? 0.0 : double(kap[(sw_pos(b) * G + g) * (2 * P) + e]);
+          const double sd = ix.sig[int64_t(f) * M + b] * (1.0 - kappa);
           vs = mark[c] ? __int_as_float(0x7fc00000) : float(sd);
           vi = mark[c] ? vs : float(1.0 / sd);
         }
@@ -295,10 +342,44 @@ __device__ __forceinline__ SwJoint sw_joint(const SweepJob* jb) {
   return j;
 }
 
+// The correlations of pair (a, b), computed directly by the warp into e:
+// z-normalised windows point by point, as the verification does.  They err
+// to the near side by two units in the last place of 1.
+template <int P>
+__device__ __forceinline__ void sw_direct_pair(const SweepView& v, uint32_t a, uint32_t b, float* e) {
+  const int lane = threadIdx.x & 31, w = v.w, stride = v.G * 2 * P;
+  const float* px = static_cast<const float*>(v.xp);
+  const float* pl = static_cast<const float*>(v.xl);
+#pragma unroll 1
+  for (int f = 0; f < v.D; ++f) {
+    const int64_t oa = int64_t(f) * v.M + a, ob = int64_t(f) * v.M + b;
+    const double ma = v.mu[oa], sa = v.sig[oa], mb = v.mu[ob], sb = v.sig[ob];
+    const float ha = float(ma), la = float(ma - double(ha)), hb = float(mb), lb = float(mb - double(hb));
+    const float ia = sa <= kFlatRel * (1.0 + fabs(ma)) ? 0.f : float(1.0 / sa);   // flat: the zero vector
+    const float ib = sb <= kFlatRel * (1.0 + fabs(mb)) ? 0.f : float(1.0 / sb);
+    float acc = 0.f;
+#pragma unroll 1
+    for (int t = lane; t < w; t += 32) {
+      const int64_t pa = sw_pos(int64_t(a) + t) * stride + f, pb = sw_pos(int64_t(b) + t) * stride + f;
+      float ua = -la, ub = -lb;
+      if (pl) {
+        ua += pl[pa];
+        ub += pl[pb];
+      }
+      const float dd = ((px[pa] - ha) + ua) * ia - ((px[pb] - hb) + ub) * ib;
+      acc = fmaf(dd, dd, acc);
+    }
+    for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+    if (lane == 0) e[f] = 1.f - acc / (2.f * float(w)) + 1.2e-7f;
+  }
+}
+
 // The queued hits of a warp, the last 32 at a time (all of them when
 // `all`), one per lane: pairs that exist and are not trivial get their
-// distance; pairs with an unresolvable window (NaN) distance 0.  Returns
-// the number left.
+// distance; the correlations of pairs with a window that has sigma = NaN are
+// computed directly first (7 windows per cut, and flat ones; taken as
+// candidates at distance 0, as they were, a quiet stretch's thousands of
+// pairs per window all went through the host).  Returns the number left.
 template <int P>
 __device__ __noinline__ int sw_drain(const SweepJob* jb, float* queue, int qn, bool all) {
   const SweepView& v = jb->v;
@@ -309,32 +390,41 @@ __device__ __noinline__ int sw_drain(const SweepJob* jb, float* queue, int qn, b
   while (qn >= 32 || (all && qn > 0)) {
     const int n = min(32, qn);
     qn -= n;
+    float* e = queue + (qn + lane) * QS;
+    uint32_t a = 0, b = 0;
+    bool pair = false;
     if (lane < n) {
-      float* e = queue + (qn + lane) * QS;
-      const uint32_t a = __float_as_uint(e[QS - 2]), b = __float_as_uint(e[QS - 1]);
-      if (int64_t(b) < v.M && int64_t(b) - int64_t(a) > int64_t(v.excl)) {
-        float sm = 0.f;
-        if (!isnan(e[0])) {
-          if (D <= 8) sm = sw_dist<8>(e, D, d, wf);
-          else if (D <= 16) sm = sw_dist<16>(e, D, d, wf);
-          else {
-            for (int q = 0; q < d && sm <= thr; ++q) {
-              float best = -INFINITY;
-              int at = 0;
-              for (int f = 0; f < D; ++f) {
-                const float c = e[f];
-                if (c > best) {
-                  best = c;
-                  at = f;
-                }
-              }
-              e[at] = -INFINITY;
-              sm += sqrtf(fmaxf(2.f * wf * (1.f - best), 0.f));
+      a = __float_as_uint(e[QS - 2]);
+      b = __float_as_uint(e[QS - 1]);
+      pair = int64_t(b) < v.M && int64_t(b) - int64_t(a) > int64_t(v.excl);
+    }
+    uint32_t direct = __ballot_sync(0xffffffffu, pair && isnan(e[0]));
+    while (direct) {
+      const int q = __ffs(int(direct)) - 1;
+      direct &= direct - 1u;
+      sw_direct_pair<P>(v, __shfl_sync(0xffffffffu, a, q), __shfl_sync(0xffffffffu, b, q), queue + (qn + q) * QS);
+    }
+    __syncwarp();
+    if (pair) {
+      float sm = 0.f;
+      if (D <= 8) sm = sw_dist<8>(e, D, d, wf);
+      else if (D <= 16) sm = sw_dist<16>(e, D, d, wf);
+      else {
+        for (int q = 0; q < d && sm <= thr; ++q) {
+          float best = -INFINITY;
+          int at = 0;
+          for (int f = 0; f < D; ++f) {
+            const float c = e[f];
+            if (c > best) {
+              best = c;
+              at = f;
             }
           }
+          e[at] = -INFINITY;
+          sm += sqrtf(fmaxf(2.f * wf * (1.f - best), 0.f));
         }
-        if (sm <= thr && sm > jb->rc.lo) sw_record(jb->rc, a, b, sm);
       }
+      if (sm <= thr && sm > jb->rc.lo) sw_record(jb->rc, a, b, sm);
     }
     __syncwarp();
   }
@@ -410,16 +500,97 @@ __device__ __forceinline__ void sw_cols(const SwVec<P>* tab, int64_t b0, int G, 
   }
 }
 
+// Direct start: C(a, b + r) of the lane's 8 columns (a, b multiples of 8) into
+// C.  The columns are centred on the first one's mean c and corrected by
+// (c - mu_b) sum_t u_t, u_t = x_{a+t} - mu_a (a sum that is zero but for
+// rounding).
+template <int P>
+__device__ __forceinline__ void sw_start(const SweepView& v, int G, int g, int64_t a, int64_t b, float2 (&C)[kSwR][P]) {
+  const int D = v.D, w = v.w;
+  const int64_t M = v.M;
+  SwVec<P> mah, mal, cc;
+#pragma unroll
+  for (int e = 0; e < (2 * P); ++e) {
+    const int f = (2 * P) * g + e;
+    const bool in = f < D;
+    const double ma = in ? v.mu[int64_t(f) * M + a] : 0.0;
+    const float hi = float(ma), lo = float(ma - double(hi));
+    const float c = in ? float(v.mu[int64_t(f) * M + min(b, M - 1)]) : 0.f;
+    if (e & 1) { mah.v[e / 2].y = hi; mal.v[e / 2].y = lo; cc.v[e / 2].y = c; }
+    else { mah.v[e / 2].x = hi; mal.v[e / 2].x = lo; cc.v[e / 2].x = c; }
+  }
+  const SwVec<P>* px = static_cast<const SwVec<P>*>(v.xp) + g;
+  const SwVec<P>* pl = v.xl ? static_cast<const SwVec<P>*>(v.xl) + g : nullptr;
+  auto value = [&](int64_t pos, const SwVec<P>& m) {
+    SwVec<P> x = px[pos * G];
+#pragma unroll
+    for (int p = 0; p < P; ++p) x.v[p] = __fadd2_rn(x.v[p], make_float2(-m.v[p].x, -m.v[p].y));
+    if (pl) {
+      const SwVec<P> l = pl[pos * G];
+#pragma unroll
+      for (int p = 0; p < P; ++p) x.v[p] = __fadd2_rn(x.v[p], l.v[p]);
+    }
+    return x;
+  };
+  SwVec<P> col[kSwR];
+  float2 su[P];
+#pragma unroll
+  for (int p = 0; p < P; ++p) su[p] = make_float2(0.f, 0.f);
+#pragma unroll
+  for (int r = 0; r < kSwR; ++r) {
+#pragma unroll
+    for (int p = 0; p < P; ++p) C[r][p] = make_float2(0.f, 0.f);
+    col[r] = value(sw_pos(b + r), cc);
+  }
+  for (int t = 0; t < w; t += 8) {
+    const int64_t pr = sw_pos(a + t), pc = sw_pos(b + t + 8);
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+      SwVec<P> u = value(pr + 8 * i, mah);
+#pragma unroll
+      for (int p = 0; p < P; ++p) {
+        u.v[p] = __fadd2_rn(u.v[p], make_float2(-mal.v[p].x, -mal.v[p].y));
+        if (t + i >= w) u.v[p] = make_float2(0.f, 0.f);
+        su[p] = __fadd2_rn(su[p], u.v[p]);
+      }
+#pragma unroll
+      for (int r = 0; r < kSwR; ++r)
+#pragma unroll
+        for (int p = 0; p < P; ++p) C[r][p] = __ffma2_rn(u.v[p], col[(i + r) & 7].v[p], C[r][p]);
+      col[i] = value(pc + 8 * i, cc);
+    }
+  }
+#pragma unroll
+  for (int r = 0; r < kSwR; ++r) {
+#pragma unroll
+    for (int p = 0; p < P; ++p) {
+      float dm[2];
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        const int f = (2 * P) * g + 2 * p + h;
+        const float c = h ? cc.v[p].y : cc.v[p].x;
+        dm[h] = f < D ? float(double(c) - v.mu[int64_t(f) * M + min(b + r, M - 1)]) : 0.f;
+      }
+      C[r][p] = __ffma2_rn(make_float2(dm[0], dm[1]), su[p], C[r][p]);
+      // a dim that does not exist: negative, against sigma 0
+      if ((2 * P) * g + 2 * p >= D) C[r][p].x = -1.f;
+      if ((2 * P) * g + 2 * p + 1 >= D) C[r][p].y = -1.f;
+    }
+  }
+}
+
 // An 8-row group in which some dim of some pair passed the first test,
 // again from its start (the cross products in ck), up to its last hot row
 // (bits of hot), with the joint test in the hot rows: the correlations of
 // the lane's dims, their part of the sum, the sum over the
 // diagonal's lanes.  Passing pairs go to the queue, one entry per pair, with
 // their correlations (which depend on no threshold).
-// Returns the queue's length.  Two rows per turn, with the columns moved
+// Returns the queue's length, with kSwCut where a row or column of the group
+// is at a cut.  Two rows per turn, with the columns moved
 // along in registers: unrolled over all 8 rows, the code fell out of the
 // instruction cache (a sweep of n = 2e4 at a
 // loose threshold took 7.3 ms against 3.4).
+constexpr int kSwCut = 1 << 30;
 template <int P, int GT>
 __device__ __noinline__ int sw_redo(const SweepJob* jb, const SwVec<P>* rows, SwVec<P>* ck, float* queue,
                                     int64_t a, int64_t b, uint32_t hot, int qn) {
@@ -542,6 +713,8 @@ __device__ __noinline__ int sw_redo(const SweepJob* jb, const SwVec<P>* rows, Sw
     }
     load(pn + (i2 + 1) * 8 * G, 7);
   }
+  const unsigned long long* cuts = reinterpret_cast<const unsigned long long*>(jb->v.cut);
+  if (__any_sync(0xffffffffu, (cuts[a >> 3] | cuts[b >> 3] | cuts[(b >> 3) + 1]) != 0ull)) qn |= kSwCut;
   return qn;
 }
 
@@ -552,7 +725,7 @@ template <int P, int GT>
 __device__ __forceinline__ void sw_block(const SweepJob* jb, int64_t bx, int64_t by) {
   extern __shared__ __align__(16) unsigned char sw_mem[];
   const SweepView& v = jb->v;
-  const int G = GT ? GT : v.G, D = v.D, w = v.w;
+  const int G = GT ? GT : v.G, w = v.w;
   const int64_t M = v.M;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int LPW = 32 / G;
@@ -584,94 +757,37 @@ __device__ __forceinline__ void sw_block(const SweepJob* jb, int64_t bx, int64_t
   __syncthreads();                  // a previous block of this CTA is done with the row buffers
   stage(0);
 
-  // ---- direct start: C(a0, b) of the lane's 8 columns.  The columns are
-  // centred on the first one's mean c and corrected by
-  // (c - mu_b) sum_t u_t, u_t = x_{a0+t} - mu_a0 (a sum that is zero but
-  // for rounding)
+  // ---- the state: C, the columns in flight
   float2 C[kSwR][P];
-  {
-    SwVec<P> mah, mal, cc;
-#pragma unroll
-    for (int e = 0; e < (2 * P); ++e) {
-      const int f = (2 * P) * g + e;
-      const bool in = f < D;
-      const double ma = in ? v.mu[int64_t(f) * M + a0] : 0.0;
-      const float hi = float(ma), lo = float(ma - double(hi));
-      const float c = in ? float(v.mu[int64_t(f) * M + min(b0, M - 1)]) : 0.f;
-      if (e & 1) { mah.v[e / 2].y = hi; mal.v[e / 2].y = lo; cc.v[e / 2].y = c; }
-      else { mah.v[e / 2].x = hi; mal.v[e / 2].x = lo; cc.v[e / 2].x = c; }
-    }
-    const SwVec<P>* px = static_cast<const SwVec<P>*>(v.xp) + g;
-    const SwVec<P>* pl = v.xl ? static_cast<const SwVec<P>*>(v.xl) + g : nullptr;
-    auto value = [&](int64_t pos, const SwVec<P>& m) {
-      SwVec<P> x = px[pos * G];
-#pragma unroll
-      for (int p = 0; p < P; ++p) x.v[p] = __fadd2_rn(x.v[p], make_float2(-m.v[p].x, -m.v[p].y));
-      if (pl) {
-        const SwVec<P> l = pl[pos * G];
-#pragma unroll
-        for (int p = 0; p < P; ++p) x.v[p] = __fadd2_rn(x.v[p], l.v[p]);
-      }
-      return x;
-    };
-    SwVec<P> col[kSwR];
-    float2 su[P];
-#pragma unroll
-    for (int p = 0; p < P; ++p) su[p] = make_float2(0.f, 0.f);
-#pragma unroll
-    for (int r = 0; r < kSwR; ++r) {
-#pragma unroll
-      for (int p = 0; p < P; ++p) C[r][p] = make_float2(0.f, 0.f);
-      col[r] = value(sw_pos(b0 + r), cc);
-    }
-    for (int t = 0; t < w; t += 8) {
-      const int64_t pr = sw_pos(a0 + t), pc = sw_pos(b0 + t + 8);
-#pragma unroll
-      for (int i = 0; i < 8; ++i) {
-        SwVec<P> u = value(pr + 8 * i, mah);
-#pragma unroll
-        for (int p = 0; p < P; ++p) {
-          u.v[p] = __fadd2_rn(u.v[p], make_float2(-mal.v[p].x, -mal.v[p].y));
-          if (t + i >= w) u.v[p] = make_float2(0.f, 0.f);
-          su[p] = __fadd2_rn(su[p], u.v[p]);
-        }
-#pragma unroll
-        for (int r = 0; r < kSwR; ++r)
-#pragma unroll
-          for (int p = 0; p < P; ++p) C[r][p] = __ffma2_rn(u.v[p], col[(i + r) & 7].v[p], C[r][p]);
-        col[i] = value(pc + 8 * i, cc);
-      }
-    }
-#pragma unroll
-    for (int r = 0; r < kSwR; ++r) {
-#pragma unroll
-      for (int p = 0; p < P; ++p) {
-        float dm[2];
-#pragma unroll
-        for (int h = 0; h < 2; ++h) {
-          const int f = (2 * P) * g + 2 * p + h;
-          const float c = h ? cc.v[p].y : cc.v[p].x;
-          dm[h] = f < D ? float(double(c) - v.mu[int64_t(f) * M + min(b0 + r, M - 1)]) : 0.f;
-        }
-        C[r][p] = __ffma2_rn(make_float2(dm[0], dm[1]), su[p], C[r][p]);
-        // a dim that does not exist: negative, against sigma 0
-        if ((2 * P) * g + 2 * p >= D) C[r][p].x = -1.f;
-        if ((2 * P) * g + 2 * p + 1 >= D) C[r][p].y = -1.f;
-      }
-    }
-  }
-
-  // ---- the columns in flight and the row factor of the test
   const int cstep = 8 * G;                                       // vectors between the columns of an 8-row group
   SwVec<P> df[kSwR], dg[kSwR], sg[kSwR];
-  sw_cols<P>(tab, b0, G, g, df, dg, sg);
+  // C started anew for the group at row ro (df and dg of that row in rf, rg),
+  // and its columns: back by one row from the direct value, which the group's
+  // first row then takes again; into the group's checkpoint
+  auto restart = [&](int64_t ro, SwVec<P>* to, const SwVec<P>& rf, const SwVec<P>& rg) {
+    sw_start<P>(v, G, g, a0 + ro, b0 + ro, C);
+    sw_cols<P>(tab, b0 + ro, G, g, df, dg, sg);
 #pragma unroll
-  for (int r = 0; r < kSwR; ++r) {
-    SwVec<P> c;
+    for (int r = 0; r < kSwR; ++r) {
+      SwVec<P> c;
 #pragma unroll
-    for (int p = 0; p < P; ++p) c.v[p] = C[r][p];
-    ck[r * 32 + lane] = c;
-  }
+      for (int p = 0; p < P; ++p) {
+        C[r][p] = __ffma2_rn(make_float2(-rg.v[p].x, -rg.v[p].y), df[r].v[p], C[r][p]);
+        C[r][p] = __ffma2_rn(make_float2(-rf.v[p].x, -rf.v[p].y), dg[r].v[p], C[r][p]);
+        c.v[p] = C[r][p];
+      }
+      to[r * 32 + lane] = c;
+    }
+  };
+  // One place for it, at the head of a group, costs no registers with a
+  // constant G; the runtime form spills less with a second one in the slow
+  // branch (D = 27, n = 6e4: 12.3 ms against 15.4; D = 32, n = 1e5: 33.9 against 32.2)
+  bool fresh = GT != 0;                                          // the next group begins with a direct start
+  auto restart0 = [&](int64_t ro, SwVec<P>* to) {
+    const SwVec<P>* ra = tab + sw_off(a0 + ro) * G + g;
+    restart(ro, to, ra[0], ra[64 * G]);
+  };
+  if (GT == 0) restart0(0, ck);
   const float t1 = jb->thr / float(jb->d);
   const float nk = -(1.f - t1 * t1 / (2.f * float(w)) - kSwSlack) * float(w);
   const float2 nk2 = make_float2(nk, nk);
@@ -680,13 +796,6 @@ __device__ __forceinline__ void sw_block(const SweepJob* jb, int64_t bx, int64_t
   for (int s = 0; s < nstage; ++s) {
     asm volatile("cp.async.wait_group 0;" ::: "memory");
     __syncthreads();                // this stage's rows are here, the other buffer is free
-    if (s == 0) {                   // the first row takes no update
-      for (int q = threadIdx.x; q < G * 2; q += kSwThreads) {
-#pragma unroll
-        for (int p = 0; p < P; ++p) rows[q].v[p] = make_float2(0.f, 0.f);
-      }
-      __syncthreads();
-    }
     if (s + 1 < nstage) stage(s + 1);
     const int rn = min(RS, ((nrow + 7) & ~7) - s * RS);
     const SwVec<P>* rp = rows + (s & 1) * RS * G * 3 + g;
@@ -697,6 +806,10 @@ __device__ __forceinline__ void sw_block(const SweepJob* jb, int64_t bx, int64_t
     // overlapping, took 185 ms on the wide workload against 145)
     for (int r0 = 0; r0 < rn; r0 += 8) {
       const int64_t ro = int64_t(s) * RS + r0;
+      if (GT != 0 && fresh) {                                    // warp-uniform
+        fresh = false;
+        restart(ro, ck + cb, nf, ng);
+      }
       const SwVec<P>* pc = tab + sw_off(b0 + ro + 8) * G + g;
       const SwVec<P>* r8 = rp;
       uint32_t quiet = ~0u;                                      // bit 7 - i: no dim of row i's pairs passed
@@ -728,6 +841,11 @@ __device__ __forceinline__ void sw_block(const SweepJob* jb, int64_t bx, int64_t
         ++redone;
         const uint32_t hot = __brev(__reduce_or_sync(0xffffffffu, ~quiet)) >> 24;   // bit i: row i
         qn = sw_redo<P, GT>(jb, r8, ck + (cb ^ (kSwR * 32)), queue, a0 + ro, b0 + ro, hot, qn);
+        if (qn >= kSwCut) {                                      // a cut in the group
+          qn &= kSwCut - 1;
+          if (GT != 0) fresh = true;
+          else if (ro + 8 < nrow) restart0(ro + 8, ck + cb);
+        }
         // the state again from memory, so that none of it lives across the call
 #pragma unroll
         for (int r = 0; r < kSwR; ++r) {
@@ -798,15 +916,15 @@ int64_t sw_gy(const SweepView& v) {
 
 // Rows per block.  A block pays a direct start of w points (about 22
 // issue slots each) before its rows (about 78 each); a launch runs two or
-// three blocks per SM at a time.  Long blocks where there are many of them
-// (8192 rows at n = 2e5, D = 32, w = 500: 128 ms against 140 with 2048; the
-// error of C grows with the root of the rows, 1e-5 in the correlation there),
-// shorter ones where waves would be partly empty.
+// three blocks per SM at a time.  Long blocks where there are many of them,
+// shorter ones where waves would be partly empty.  At most 2048: the error of
+// C grows with the root of the rows (8192 took 128 ms where this takes 140,
+// n = 2e5, D = 32, w = 500, at twice the error).
 int sw_seg(const SweepView& v) {
   const int64_t slots = int64_t(sm_count()) * (v.P == 2 ? kSwBlocks<2> : kSwBlocks<1>), nd = sw_diags(v.G), gy = sw_gy(v);
-  int best = 2048;
+  int best = kSwSegMax;
   double best_cost = 1e300;
-  for (int seg = 8192; seg >= 32; seg >>= 1) {
+  for (int seg = kSwSegMax; seg >= 32; seg >>= 1) {
     int64_t blocks = 0;
     for (int64_t by = 0; by < gy; ++by) {
       const int64_t d0 = ((int64_t(v.excl) + 1) & ~int64_t(7)) + by * nd;
@@ -827,7 +945,8 @@ int sw_seg(const SweepView& v) {
 size_t sweep_table_bytes(const Index& ix) {
   const int P = sw_pairs(ix.D);
   const size_t G = size_t((ix.D + 2 * P - 1) / (2 * P));
-  return (size_t(sw_round(ix.M)) * 4 + size_t(sw_round(ix.n)) * (ix.has_lo ? 2 : 1)) * G * (8 * size_t(P));
+  return (size_t(sw_round(ix.M)) * 4 + size_t(sw_round(ix.n)) * (ix.has_lo ? 2 : 1)) * G * (8 * size_t(P)) +
+         size_t(sw_round(ix.M));
 }
 
 template <int P>
@@ -838,6 +957,12 @@ static cudaError_t sweep_table(const Index& ix, SweepView& v, void* buf, cudaStr
   v.tab = tab;
   v.xp = xp;
   v.xl = xl;
+  uint8_t* cut = reinterpret_cast<uint8_t*>(xp + v.npad * v.G * (ix.has_lo ? 2 : 1));
+  v.cut = cut;
+  const cudaError_t e = cudaMemsetAsync(cut, 0, size_t(v.Mpad), s);
+  if (e != cudaSuccess) return e;
+  const dim3 gc{unsigned((ix.M + 4 * kSwCutRun - 1) / (4 * kSwCutRun)), unsigned(ix.D), 1u};
+  MOMENTI_LAUNCH("sweep_cuts", s, k_sweep_cuts<P><<<gc, 128, 0, s>>>(ix, v, reinterpret_cast<float*>(tab + v.Mpad * v.G * 3), cut));
   MOMENTI_LAUNCH("sweep_table", s, k_sweep_table<P><<<unsigned(v.npad / 64), 256, 0, s>>>(ix, v, tab, xp, xl));
   return cudaGetLastError();
 }
@@ -853,6 +978,7 @@ cudaError_t launch_sweep_table(const Index& ix, void* buf, SweepView* out, cudaS
   v.w = ix.w;
   v.excl = ix.excl;
   v.mu = ix.mu;
+  v.sig = ix.sig;
   const cudaError_t e = v.P == 2 ? sweep_table<2>(ix, v, buf, s) : sweep_table<1>(ix, v, buf, s);
   *out = v;
   return e;

@@ -649,7 +649,7 @@ int exact_path(momenti_handle* h, int d, double tau0, momenti_motif* out, int32_
   const int k = h->p.k;
   const auto te0 = std::chrono::steady_clock::now();
   // Pairs are taken in slices of their approximate dist_d (float32 Pearson
-  // form, within 1% + 0.01 of the exact value): each all-pairs sweep records
+  // form, at most 1% + 0.01 above the exact value): each all-pairs sweep records
   // the pairs with approximate distance in (lo, hi] and a histogram of them;
   // they are verified in ascending batches (float32, direct form) and added
   // to the candidates, and greedy runs after every batch.  Once every pair

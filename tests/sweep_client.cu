@@ -25,11 +25,12 @@ struct Held {
 }  // namespace
 
 // Pairs whose approximate distance lies in (lo, thr], with that distance;
-// at most cap of them are stored.  batch: through the batching form's
-// launch, beside a second copy of the series.  Returns how many there are,
-// or a negative CUDA error.
+// at most cap of them are stored.  form: 0 the plain launch, 1 the batching
+// form's, beside a second copy of the series, from 8 on the sample's with a
+// share of 1 and that many rows per block (a multiple of 8, at most 2048).
+// Returns how many there are, or a negative CUDA error.
 extern "C" long long sweep_pairs(const void* series, int dtype, long long n, int D, int w, int excl, int d, float lo,
-                                 float thr, int batch, unsigned long long* pairs, float* dist, long long cap) {
+                                 float thr, int form, unsigned long long* pairs, float* dist, long long cap) {
   Held m;
   Index ix;
   ix.n = n;
@@ -70,7 +71,10 @@ extern "C" long long sweep_pairs(const void* series, int dtype, long long n, int
   SweepView v;
   if (er == cudaSuccess) er = launch_sweep_table(ix, tab, &v, nullptr);
   if (er == cudaSuccess) {
-    if (batch) {
+    if (form >= 8) {
+      double held = 0.0;
+      er = launch_allpairs_sample(v, d, thr, rc[0], 1.0, form, &held, nullptr, nullptr);
+    } else if (form) {
       std::vector<SweepJob> jobs(2);
       for (int q = 0; q < 2; ++q) {
         jobs[size_t(q)].v = v;

@@ -31,13 +31,13 @@ def load():
     return _lib
 
 
-def sweep(T, w, d, lo, thr, excl=None, batch=False, cap=1 << 22):
+def sweep(T, w, d, lo, thr, excl=None, form=0, cap=1 << 22):
     """Recorded pairs (a << 32 | b, sorted) and their approximate distances."""
     lib = load()
     T = np.ascontiguousarray(T)
     pairs, dist = np.zeros(cap, np.uint64), np.zeros(cap, np.float32)
     n = lib.sweep_pairs(T.ctypes.data, 1 if T.dtype == np.float64 else 0, T.shape[1], T.shape[0], w,
-                        w // 2 if excl is None else excl, d, lo, thr, int(batch), pairs.ctypes.data, dist.ctypes.data,
+                        w // 2 if excl is None else excl, d, lo, thr, form, pairs.ctypes.data, dist.ctypes.data,
                         cap)
     assert 0 <= n <= cap, n
     o = np.argsort(pairs[:n], kind="stable")
