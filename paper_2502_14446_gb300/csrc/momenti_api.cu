@@ -337,6 +337,7 @@ struct momenti_handle {
   std::vector<DevBuf> bufs;
   uint64_t device_bytes = 0;
   SortScratch sort;
+  void* sweep_tab = nullptr;         // the exact path's table, in the region of sort
   CollideScratch cs;
   HashSet hs;
   PairRec* rec_dev = nullptr;
@@ -489,6 +490,7 @@ void free_all(momenti_handle* h, bool host = false) {
   h->job_cap = 0;
   h->ix = Index{};
   h->sort = SortScratch{};
+  h->sweep_tab = nullptr;
   h->cs = CollideScratch{};
   h->hs = HashSet{};
   h->ready = false;
@@ -711,11 +713,8 @@ int exact_path(momenti_handle* h, int d, double tau0, momenti_motif* out, int32_
   unsigned long long* dcnt = nullptr;
   uint32_t* dhist = nullptr;
   uint64_t* dsel = nullptr;
-  // the sweep's table of this index, for the duration of the exact path
-  PoolBuf table(h->stream);
-  CK(pool_malloc(&table.p, sweep_table_bytes(ix), h->stream));
   SweepView view;
-  CK(launch_sweep_table(ix, table.p, &view, h->stream));
+  CK(launch_sweep_table(ix, h->sweep_tab, &view, h->stream));
   auto release = [&]() {
     if (dout) cudaFreeAsync(dout, h->stream);
     if (dval) cudaFreeAsync(dval, h->stream);
@@ -1027,11 +1026,16 @@ static int hash_all_impl(momenti_handle* h, const void* series, int32_t dtype, i
     CK(cudaMemGetInfo(&free_b, &total_b));
     const uint64_t limit = p.mem_limit ? p.mem_limit : uint64_t(0.8 * double(free_b));
     const int Wp = ((w + 63) / 64) * 64;
+    const int Dp = D <= 4 ? 4 : (D <= 8 ? 8 : 16);      // padded dims of the point-major copies
+    ix.n = n;
+    ix.M = M;
+    ix.D = D;
+    ix.has_lo = dtype == MOMENTI_F64;
+    const uint64_t table_bytes = sweep_table_bytes(ix);
     const uint64_t fixed = uint64_t(D) * n * (dtype == MOMENTI_F64 ? 8 : 4)  // series hi/lo
                            + uint64_t(D) * n * elem                          // transient staging
                            + uint64_t(D) * M * (8 + 8 + 4 + 4 + 4)           // stats
-                           + (D <= 16 ? uint64_t(16) * (3 * n + 4 * M) * 4 + M : 0)  // point-major copies
-                           + (D > 16 ? uint64_t(64) * (n + M) * 4 + M : 0)   // point-major wide copy, column table
+                           + (D <= 16 ? uint64_t(Dp) * ((dtype == MOMENTI_F64 ? 3 : 2) * n + 3 * M) * 4 : 0)  // point-major copies
                            + (D <= 16 && p.d >= 2 ? job_cap_for(M, D) * sizeof(BucketJob) : 0)
                            + (uint64_t(64) << 20);                           // small scratch
     const uint64_t per_rep = uint64_t(M) * D * (8 + 4 + 1)                   // keys, order, lcp
@@ -1053,7 +1057,7 @@ static int hash_all_impl(momenti_handle* h, const void* series, int32_t dtype, i
     const uint64_t hs_cap = std::min<uint64_t>(
         uint64_t(1) << 25, std::max<uint64_t>(uint64_t(1) << 20, next_pow2(uint64_t(M) * 64)));
     auto scratch_bytes = [&](int sreps, int creps) {
-      return uint64_t(sort_scratch_bytes(M, sreps * D)) +
+      return std::max<uint64_t>(sort_scratch_bytes(M, sreps * D), table_bytes) +
              uint64_t(creps) * D * (C + 1) * (4 + 4 + 8) + new_cap * 32 + hs_cap * 8 +
              (uint64_t(1) << 22) * sizeof(Event);
     };
@@ -1083,21 +1087,17 @@ static int hash_all_impl(momenti_handle* h, const void* series, int32_t dtype, i
     h->chunk_reps = chunk;
     h->sort_reps = sort_reps;
 
-    ix.n = n;
-    ix.M = M;
-    ix.D = D;
     ix.w = w;
     ix.K = K;
     ix.L = L;
     ix.Wp = Wp;
     ix.excl = p.excl < 0 ? w / 2 : p.excl;
-    ix.has_lo = dtype == MOMENTI_F64;
     // projections per dim: K per repetition, or K/2 per half function
     const int N = (tens ? 2 * isqrt(L) : L) * kRepStride;
     CK(dalloc(h, &ix.xs_hi, size_t(D) * n));
     if (ix.has_lo) CK(dalloc(h, &ix.xs_lo, size_t(D) * n));
     if (D <= 16) {
-      ix.Dp = D <= 4 ? 4 : (D <= 8 ? 8 : 16);
+      ix.Dp = Dp;
       CK(dalloc(h, &ix.xT, size_t(ix.Dp) * n));
       CK(dalloc(h, &ix.stT, size_t(3) * ix.Dp * M));
       if (ix.has_lo) CK(dalloc(h, &ix.xlT, size_t(ix.Dp) * n));
@@ -1132,9 +1132,11 @@ static int hash_all_impl(momenti_handle* h, const void* series, int32_t dtype, i
                                               std::max<uint64_t>(uint64_t(1) << 16, uint64_t(D) * M * N / 400)));
     CK(dalloc(h, &h->flags, size_t(h->flag_cap)));
     CK(dalloc(h, &h->small, 16));
-    // index sort scratch
+    // one region: the index sort's scratch, then the exact path's table (no
+    // sort runs while it does)
     unsigned char* sort_region = nullptr;
-    CK(dalloc(h, &sort_region, sort_scratch_bytes(M, sort_reps * D)));
+    CK(dalloc(h, &sort_region, std::max<size_t>(sort_scratch_bytes(M, sort_reps * D), table_bytes)));
+    h->sweep_tab = sort_region;
     h->sort = sort_scratch_carve(sort_region, M, sort_reps * D);
     // traversal scratch
     CollideScratch& cs = h->cs;
