@@ -52,7 +52,7 @@ struct Neumaier {
   __device__ double value() const { return s + c; }
 };
 
-// A thread slides over kStatsChunk windows from a direct start.  The block's
+// A thread slides over CH windows from a direct start.  The block's
 // points are first summed in groups of 16 (each relative to its first
 // point), so a start adds w / 16 shifted group sums instead of w points.
 // FP64 runs at a sixtieth of the FP32 rate here and short series have few
@@ -62,13 +62,17 @@ struct Neumaier {
 // takes 1.9 and 0.06.
 constexpr int kStatsChunk = 16;
 constexpr int kStatsThreads = 128;
-constexpr int kStatsMaxW = 16384;        // longer windows: every start point by point (shared memory)
+// Longer windows: every start point by point (the groups would not fit the
+// shared memory), and 64 windows a thread to spread it (w = 20000, D = 8,
+// n = 1e5: 13 ms, with 16 windows 38).
+constexpr int kStatsMaxW = 16384;
+constexpr int kStatsLongChunk = 64;
 
 struct Group {
   double c, s1, s2;                      // first point; sums of x - c and its square
 };
 
-template <bool LO>
+template <bool LO, int CH>
 __global__ void __launch_bounds__(kStatsThreads)
 k_window_stats(const float* __restrict__ xh, const float* __restrict__ xl,
                int64_t n, int64_t M, int w, double* __restrict__ mu,
@@ -76,7 +80,7 @@ k_window_stats(const float* __restrict__ xh, const float* __restrict__ xl,
                float* __restrict__ ml, float* __restrict__ isg) {
   extern __shared__ Group groups[];      // the block's points from its first window, 16 each
   const int f = blockIdx.y;
-  const int64_t base = blockIdx.x * int64_t(kStatsThreads * kStatsChunk);
+  const int64_t base = blockIdx.x * int64_t(kStatsThreads * CH);
   const float* xf = xh + int64_t(f) * n;
   const float* lf = LO ? xl + int64_t(f) * n : nullptr;
   auto X = [&](int64_t t) -> double {
@@ -84,7 +88,7 @@ k_window_stats(const float* __restrict__ xh, const float* __restrict__ xl,
     if (LO) v += double(lf[t]);
     return v;
   };
-  const int full = w <= kStatsMaxW ? w / 16 : 0;       // whole groups of a window
+  const int full = CH == kStatsChunk ? w / 16 : 0;     // whole groups of a window
   if (full) {
     const int ng = kStatsThreads + full;
     for (int q = threadIdx.x; q < ng; q += kStatsThreads) {
@@ -103,9 +107,9 @@ k_window_stats(const float* __restrict__ xh, const float* __restrict__ xl,
     }
     __syncthreads();
   }
-  const int64_t a0 = base + int64_t(threadIdx.x) * kStatsChunk;
+  const int64_t a0 = base + int64_t(threadIdx.x) * CH;
   if (a0 >= M) return;
-  const int64_t a1 = min(M, a0 + kStatsChunk);
+  const int64_t a1 = min(M, a0 + CH);
   const double c = X(a0);
   Neumaier s1, s2;
   for (int q = 0; q < full; ++q) {       // sums relative to c: x - c = (x - g.c) + d
@@ -380,17 +384,22 @@ cudaError_t launch_split_series(const void* src, int dtype, int64_t n, int D, in
   return cudaGetLastError();
 }
 
-cudaError_t launch_window_stats(const Index& ix, cudaStream_t s) {
-  const int64_t span = kStatsThreads * kStatsChunk;
+template <int CH>
+static cudaError_t window_stats(const Index& ix, size_t smem, cudaStream_t s) {
+  const int64_t span = kStatsThreads * CH;
   dim3 grid(unsigned((ix.M + span - 1) / span), unsigned(ix.D));
-  const size_t smem = ix.w <= kStatsMaxW ? size_t(kStatsThreads + ix.w / 16) * sizeof(Group) : 0;
   if (ix.has_lo)
-    MOMENTI_LAUNCH("window_stats", s, k_window_stats<true><<<grid, kStatsThreads, smem, s>>>(ix.xs_hi, ix.xs_lo, ix.n, ix.M, ix.w, ix.mu, ix.sig,
+    MOMENTI_LAUNCH("window_stats", s, k_window_stats<true, CH><<<grid, kStatsThreads, smem, s>>>(ix.xs_hi, ix.xs_lo, ix.n, ix.M, ix.w, ix.mu, ix.sig,
                                               ix.mu_hi, ix.mu_lo, ix.inv_sig));
   else
-    MOMENTI_LAUNCH("window_stats", s, k_window_stats<false><<<grid, kStatsThreads, smem, s>>>(ix.xs_hi, nullptr, ix.n, ix.M, ix.w, ix.mu, ix.sig,
+    MOMENTI_LAUNCH("window_stats", s, k_window_stats<false, CH><<<grid, kStatsThreads, smem, s>>>(ix.xs_hi, nullptr, ix.n, ix.M, ix.w, ix.mu, ix.sig,
                                                ix.mu_hi, ix.mu_lo, ix.inv_sig));
   return cudaGetLastError();
+}
+
+cudaError_t launch_window_stats(const Index& ix, cudaStream_t s) {
+  if (ix.w > kStatsMaxW) return window_stats<kStatsLongChunk>(ix, 0, s);
+  return window_stats<kStatsChunk>(ix, size_t(kStatsThreads + ix.w / 16) * sizeof(Group), s);
 }
 
 cudaError_t launch_point_major(const Index& ix, cudaStream_t s) {
