@@ -404,6 +404,7 @@ k_proj_hash_tc(const __grid_constant__ CUtensorMap tmap, TcArgs g) {
         const int col0 = nc * kBN + q * 32;
         if (col0 >= NC) break;                       // columns of no repetition (warp-uniform)
         float v[32];
+        __syncwarp();                                // lanes part in the flag loops below; the load is .sync.aligned
         tmem_ld32(tmem + (uint32_t(quarter * 32) << 16) + uint32_t(buf * kBN + q * 32), v);
 #pragma unroll
         for (int rr = 0; rr < 4; ++rr) {
