@@ -445,8 +445,10 @@ struct PoolBuf {
   explicit PoolBuf(cudaStream_t st) : s(st) {}
   PoolBuf(const PoolBuf&) = delete;
   PoolBuf& operator=(const PoolBuf&) = delete;
-  ~PoolBuf() {
+  ~PoolBuf() { reset(); }
+  void reset() {
     if (p) cudaFreeAsync(p, s);
+    p = nullptr;
   }
 };
 
@@ -663,11 +665,12 @@ int exact_path(momenti_handle* h, int d, double tau0, momenti_motif* out, int32_
   const bool trace = tr && tr[0] == '1';
   auto add_batch = [&](const uint64_t* dpairs, int64_t m) -> int {
     if (m <= 0) return MOMENTI_OK;
-    double *dpd = nullptr, *ddd = nullptr;
-    uint64_t* dmask = nullptr;
-    CK(pool_malloc(&dpd, m * ix.D * 8, h->stream));
-    CK(pool_malloc(&ddd, m * 8, h->stream));
-    CK(pool_malloc(&dmask, m * 8, h->stream));
+    PoolBuf bpd(h->stream), bdd(h->stream), bmask(h->stream);
+    CK(pool_malloc(&bpd.p, m * ix.D * 8, h->stream));
+    CK(pool_malloc(&bdd.p, m * 8, h->stream));
+    CK(pool_malloc(&bmask.p, m * 8, h->stream));
+    double *dpd = static_cast<double*>(bpd.p), *ddd = static_cast<double*>(bdd.p);
+    uint64_t* dmask = static_cast<uint64_t*>(bmask.p);
     CK(launch_verify_pairs(ix, d, dpairs, m, 0, dpd, ddd, dmask, h->stream));
     std::vector<uint64_t> pk(m), mk(m);
     std::vector<double> per(m * ix.D), dd(m);
@@ -675,9 +678,6 @@ int exact_path(momenti_handle* h, int d, double tau0, momenti_motif* out, int32_
     CK(cudaMemcpyAsync(per.data(), dpd, m * ix.D * 8, cudaMemcpyDeviceToHost, h->stream));
     CK(cudaMemcpyAsync(dd.data(), ddd, m * 8, cudaMemcpyDeviceToHost, h->stream));
     CK(cudaMemcpyAsync(mk.data(), dmask, m * 8, cudaMemcpyDeviceToHost, h->stream));
-    CK(cudaFreeAsync(dpd, h->stream));
-    CK(cudaFreeAsync(ddd, h->stream));
-    CK(cudaFreeAsync(dmask, h->stream));
     CK(cudaStreamSynchronize(h->stream));
     const size_t old_n = got.size();
     for (int64_t q = 0; q < m; ++q) {
@@ -708,23 +708,14 @@ int exact_path(momenti_handle* h, int d, double tau0, momenti_motif* out, int32_
   const uint64_t cap_max = std::max<uint64_t>(uint64_t(1) << 22,
                                               std::min<uint64_t>(uint64_t(1) << 30, free_b / 4 / 12));
   uint64_t cap = std::min<uint64_t>(uint64_t(1) << 24, cap_max);
-  uint64_t* dout = nullptr;
-  float* dval = nullptr;
-  unsigned long long* dcnt = nullptr;
-  uint32_t* dhist = nullptr;
-  uint64_t* dsel = nullptr;
+  // returned to the pool on every way out
+  PoolBuf bcnt(h->stream), bhist(h->stream), bout(h->stream), bval(h->stream), bsel(h->stream);
   SweepView view;
   CK(launch_sweep_table(ix, h->sweep_tab, &view, h->stream));
-  auto release = [&]() {
-    if (dout) cudaFreeAsync(dout, h->stream);
-    if (dval) cudaFreeAsync(dval, h->stream);
-    if (dsel) cudaFreeAsync(dsel, h->stream);
-    dout = nullptr;
-    dval = nullptr;
-    dsel = nullptr;
-  };
-  CK(pool_malloc(&dcnt, 24, h->stream));           // pairs; a sample's groups, and those run twice
-  CK(pool_malloc(&dhist, kApBins * 4, h->stream));
+  CK(pool_malloc(&bcnt.p, 24, h->stream));         // pairs; a sample's groups, and those run twice
+  CK(pool_malloc(&bhist.p, kApBins * 4, h->stream));
+  unsigned long long* const dcnt = static_cast<unsigned long long*>(bcnt.p);
+  uint32_t* const dhist = static_cast<uint32_t*>(bhist.p);
   std::vector<uint32_t> hist(kApBins);
   // First edge.  A pair is worth recording if it can be among the k motifs:
   // TOP's k-th (tau0) bounds them when TOP is full, but on background pairs
@@ -825,10 +816,10 @@ int exact_path(momenti_handle* h, int d, double tau0, momenti_motif* out, int32_
                  double(tau0), std::chrono::duration<double, std::milli>(std::chrono::steady_clock::now() - te0).count());
   int rc = MOMENTI_ERR_OVERFLOW;
   for (int pass = 0; pass < 64; ++pass) {
-    if (!dout) {
-      CK(pool_malloc(&dout, cap * 8, h->stream));
-      CK(pool_malloc(&dval, cap * 4, h->stream));
-    }
+    if (!bout.p) CK(pool_malloc(&bout.p, cap * 8, h->stream));
+    if (!bval.p) CK(pool_malloc(&bval.p, cap * 4, h->stream));
+    uint64_t* const dout = static_cast<uint64_t*>(bout.p);
+    float* const dval = static_cast<float*>(bval.p);
     CK(cudaMemsetAsync(dcnt, 0, 8, h->stream));
     CK(cudaMemsetAsync(dhist, 0, kApBins * 4, h->stream));
     ApRec ar;
@@ -865,7 +856,8 @@ int exact_path(momenti_handle* h, int d, double tau0, momenti_motif* out, int32_
       if (bin > 0) {
         hi = float(double(lo) + width * bin);
       } else {
-        release();
+        bout.reset();
+        bval.reset();
         if (uint64_t(hist[0]) > cap_max)
           return fail(h, MOMENTI_ERR_MEMORY, "exact path: one distance bin exceeds memory");
         cap = std::min<uint64_t>(cap_max, (uint64_t(cnt) + (uint64_t(1) << 20)) & ~((uint64_t(1) << 20) - 1));
@@ -873,7 +865,8 @@ int exact_path(momenti_handle* h, int d, double tau0, momenti_motif* out, int32_
       continue;
     }
     // ascending batches of whole bins
-    CK(pool_malloc(&dsel, std::max<uint64_t>(cnt, 1) * 8, h->stream));
+    CK(pool_malloc(&bsel.p, std::max<uint64_t>(cnt, 1) * 8, h->stream));
+    uint64_t* const dsel = static_cast<uint64_t*>(bsel.p);
     bool done = false;
     for (int b0 = 0; b0 < kApBins && !done;) {
       int b1 = b0;
@@ -893,7 +886,9 @@ int exact_path(momenti_handle* h, int d, double tau0, momenti_motif* out, int32_
       done = exact_below((double(shi) - 1e-2) / 1.01);
       b0 = b1;
     }
-    release();
+    bout.reset();
+    bval.reset();
+    bsel.reset();
     if (done || hi >= all_edge) {
       // done, or every pair is held: fewer than k non-trivial motifs exist
       rc = finalize(h, d, got, out, n_out, 0.0, max_err);
@@ -913,8 +908,6 @@ int exact_path(momenti_handle* h, int d, double tau0, momenti_motif* out, int32_
     else if (hi_top > hi && tau0 > 0) hi = hi_top;
     else hi = std::min(2.f * hi + 1e-2f, all_edge);
   }
-  cudaFreeAsync(dcnt, h->stream);
-  cudaFreeAsync(dhist, h->stream);
   if (trace)
     std::fprintf(stderr, "momenti trace: exact done ms=%.1f\n",
                  std::chrono::duration<double, std::milli>(std::chrono::steady_clock::now() - te0).count());
