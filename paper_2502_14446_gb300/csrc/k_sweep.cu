@@ -40,7 +40,7 @@
 // of 64 windows transposed (8 x 8), so that they are consecutive.
 //
 // What bounds it (D = 8, w = 300, 5e9 pairs, edge below the background):
-// 7.6 ms, 5.2 pair-dimensions per cycle and scheduler of the 10.7 that three
+// 7.2 ms, 5.6 pair-dimensions per cycle and scheduler of the 10.7 that three
 // FMA on the FP32 lanes allow; 8 warps per SM, fixed-latency dependencies
 // first.  The form before, one diagonal per lane sliding centred products,
 // took 35.6 ms; at D = 32, w = 500, n = 2e5, 145 against 848 ms.
@@ -92,7 +92,8 @@ __host__ __device__ __forceinline__ int64_t sw_off(int64_t b) {
 // Pairs of dims per lane for a series of D dims.  Two pairs read half the
 // instructions per pair-dimension; one pair wastes at most one dimension
 // instead of three, which pays at D = 1, 2, 5, 6 (a sweep of n = 1e5, w =
-// 300 at D = 5: 5.8 ms against 6.6 with two).
+// 300: 6.8 ms at D = 5, with two pairs as at D = 8 7.2; 2.2 at D = 1, with
+// two as at D = 4 3.9).
 int sw_pairs(int D) { return D <= 2 || D == 5 || D == 6 ? 1 : 2; }
 int64_t sw_round(int64_t m) { return ((m + 63) & ~int64_t(63)) + 64 + kSwPad; }
 
@@ -761,12 +762,23 @@ __device__ __forceinline__ void sw_block(const SweepJob* jb, int64_t bx, int64_t
   float2 C[kSwR][P];
   const int cstep = 8 * G;                                       // vectors between the columns of an 8-row group
   SwVec<P> df[kSwR], dg[kSwR], sg[kSwR];
-  // C started anew for the group at row ro (df and dg of that row in rf, rg),
-  // and its columns: back by one row from the direct value, which the group's
-  // first row then takes again; into the group's checkpoint
-  auto restart = [&](int64_t ro, SwVec<P>* to, const SwVec<P>& rf, const SwVec<P>& rg) {
+  const float t1 = jb->thr / float(jb->d);
+  const float nk = -(1.f - t1 * t1 / (2.f * float(w)) - kSwSlack) * float(w);
+  const float2 nk2 = make_float2(nk, nk);
+  int qn = 0, cb = 0, redone = 0;   // queued hits, this group's checkpoint, groups run twice
+  int ro = 0;                       // the group's first row
+start:
+  // C started anew for the group at row ro, and its columns: back by one row
+  // from the direct value, which the group's first row then takes again; into
+  // the group's checkpoint.  The slow branch comes back here after a cut: a
+  // flag asked for at the head of every group, or a second copy of the start
+  // in the branch, cost the loop registers (7.6 ms against 7.2 at D = 8,
+  // n = 1e5; 24.6 against 23.4 at D = 64, n = 6e4)
+  {
     sw_start<P>(v, G, g, a0 + ro, b0 + ro, C);
     sw_cols<P>(tab, b0 + ro, G, g, df, dg, sg);
+    const SwVec<P>* ra = tab + sw_off(a0 + ro) * G + g;
+    const SwVec<P> rf = ra[0], rg = ra[64 * G];
 #pragma unroll
     for (int r = 0; r < kSwR; ++r) {
       SwVec<P> c;
@@ -776,40 +788,23 @@ __device__ __forceinline__ void sw_block(const SweepJob* jb, int64_t bx, int64_t
         C[r][p] = __ffma2_rn(make_float2(-rf.v[p].x, -rf.v[p].y), dg[r].v[p], C[r][p]);
         c.v[p] = C[r][p];
       }
-      to[r * 32 + lane] = c;
+      ck[cb + r * 32 + lane] = c;
     }
-  };
-  // One place for it, at the head of a group, costs no registers with a
-  // constant G; the runtime form spills less with a second one in the slow
-  // branch (D = 27, n = 6e4: 12.3 ms against 15.4; D = 32, n = 1e5: 33.9 against 32.2)
-  bool fresh = GT != 0;                                          // the next group begins with a direct start
-  auto restart0 = [&](int64_t ro, SwVec<P>* to) {
-    const SwVec<P>* ra = tab + sw_off(a0 + ro) * G + g;
-    restart(ro, to, ra[0], ra[64 * G]);
-  };
-  if (GT == 0) restart0(0, ck);
-  const float t1 = jb->thr / float(jb->d);
-  const float nk = -(1.f - t1 * t1 / (2.f * float(w)) - kSwSlack) * float(w);
-  const float2 nk2 = make_float2(nk, nk);
-  int qn = 0, cb = 0, redone = 0;   // queued hits, this group's checkpoint, groups run twice
-  const int nstage = (nrow + RS - 1) / RS;
-  for (int s = 0; s < nstage; ++s) {
-    asm volatile("cp.async.wait_group 0;" ::: "memory");
-    __syncthreads();                // this stage's rows are here, the other buffer is free
-    if (s + 1 < nstage) stage(s + 1);
-    const int rn = min(RS, ((nrow + 7) & ~7) - s * RS);
-    const SwVec<P>* rp = rows + (s & 1) * RS * G * 3 + g;
+  }
+  while (ro < nrow) {
+    if ((ro & (RS - 1)) == 0) {     // (RS: a power of two)
+      asm volatile("cp.async.wait_group 0;" ::: "memory");
+      __syncthreads();              // this stage's rows are here, the other buffer is free
+      if (ro + RS < nrow) stage(ro / RS + 1);
+    }
+    const int rend = min((ro | (RS - 1)) + 1, (nrow + 7) & ~7);   // of the stage
+    const SwVec<P>* rp = rows + (ro & (2 * RS - 1)) * G * 3 + g;
     SwVec<P> nf = rp[0], ng = rp[G], ns = rp[2 * G];                    // the next row's record
     // 8 rows at a time without a branch: the tests' sign bits of all their
     // pairs are combined, and a group in which one passed runs once more
     // from its start (a branch after every row, with what it kept from
     // overlapping, took 185 ms on the wide workload against 145)
-    for (int r0 = 0; r0 < rn; r0 += 8) {
-      const int64_t ro = int64_t(s) * RS + r0;
-      if (GT != 0 && fresh) {                                    // warp-uniform
-        fresh = false;
-        restart(ro, ck + cb, nf, ng);
-      }
+    for (; ro < rend; ro += 8) {
       const SwVec<P>* pc = tab + sw_off(b0 + ro + 8) * G + g;
       const SwVec<P>* r8 = rp;
       uint32_t quiet = ~0u;                                      // bit 7 - i: no dim of row i's pairs passed
@@ -819,7 +814,7 @@ __device__ __forceinline__ void sw_block(const SweepJob* jb, int64_t bx, int64_t
         float2 nt[P];
 #pragma unroll
         for (int p = 0; p < P; ++p) nt[p] = __fmul2_rn(ns.v[p], nk2);
-        if (i < 7 || r0 + 8 < rn) rp += G * 3;                   // (the last row of the stage is read again)
+        if (i < 7 || ro + 8 < rend) rp += G * 3;                 // (the last row of the stage is read again)
         nf = rp[0];
         ng = rp[G];
         ns = rp[2 * G];
@@ -841,11 +836,12 @@ __device__ __forceinline__ void sw_block(const SweepJob* jb, int64_t bx, int64_t
         ++redone;
         const uint32_t hot = __brev(__reduce_or_sync(0xffffffffu, ~quiet)) >> 24;   // bit i: row i
         qn = sw_redo<P, GT>(jb, r8, ck + (cb ^ (kSwR * 32)), queue, a0 + ro, b0 + ro, hot, qn);
-        if (qn >= kSwCut) {                                      // a cut in the group
+        if (qn >= kSwCut && ro + 8 < nrow) {                     // a cut in the group, warp-uniform
           qn &= kSwCut - 1;
-          if (GT != 0) fresh = true;
-          else if (ro + 8 < nrow) restart0(ro + 8, ck + cb);
+          ro += 8;
+          goto start;
         }
+        qn &= kSwCut - 1;
         // the state again from memory, so that none of it lives across the call
 #pragma unroll
         for (int r = 0; r < kSwR; ++r) {
