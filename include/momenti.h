@@ -451,7 +451,8 @@ uint64_t momenti_launch_count(void);
 /* Starts timing every launch of the kernel called name with CUDA events on
  * the launching stream, and clears the accumulated time; NULL stops timing.
  * A name ending in '*' selects every kernel whose name starts with the part
- * before it (for example "sort_*": all kernels of the index sort).
+ * before it (for example "sort_*": all kernels of the index sort).  The
+ * kernels of all buckets of up to 32 members run under the name "subwarp".
  * Kernel names: split_f32, split_f64, point_major, window_stats,
  * stats_pm, mean16, r_sample, draw, layout_hash, layout_boff,
  * proj_hash_fp32, proj_hash_tc, rehash, sort_init, sort_hist, sort_scan,

@@ -513,10 +513,10 @@ double predict_rep_ms(const Index& ix, uint64_t tiles, uint64_t sub_checks, uint
 }
 
 // Recording sweeps the exact path is predicted to cost: one from a full
-// TOP's k-th; without it, on a large series the slices start low and
-// double (about two), otherwise the row-minima sweep, which computes every
-// pair's distances in full (measured at about three recording sweeps at
-// D = 8), comes first.
+// TOP's k-th; without it two on a large series and four otherwise.  Four was
+// the cost with the search for a first threshold that the sampled edge has
+// replaced (some tenths of a sweep now); like the costs per pair below, the
+// numbers decide which searches end in the exact path and stay as they are.
 int exact_sweeps(const Index& ix, bool top_full) {
   if (top_full) return 1;
   const bool large = double(ix.M) * double(ix.M) * double(ix.D) > 4e11;
