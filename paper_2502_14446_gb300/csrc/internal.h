@@ -280,6 +280,11 @@ struct ApRec {
   float lo = -1.f;
   float hscale = 0.f;          // kApBins / (thr - lo)
 };
+// Bin of a recorded distance.
+__device__ __forceinline__ int ap_bin(float dd, float lo, float hscale) {
+  const float x = (dd - lo) * hscale;
+  return x < float(kApBins - 1) ? int(fmaxf(x, 0.f)) : kApBins - 1;
+}
 
 // ---- k_sweep.cu ---------------------------------------------------------
 // The sweep's view of an index: its table (k_sweep.cu: df, dg and sigma per
@@ -325,7 +330,9 @@ cudaError_t launch_allpairs_sample(const SweepView& v, int d, float thr, const A
 cudaError_t launch_allpairs_batch(std::vector<SweepJob> jobs, cudaStream_t s);
 
 // ---- k_verify.cu, continued ---------------------------------------------
-// Recorded pairs whose approximate distance lies in (lo, hi], compacted.
-cudaError_t launch_select_pairs(const uint64_t* pairs, const float* dd, uint64_t m, float lo,
-                                float hi, uint64_t* out, unsigned long long* count, cudaStream_t s);
+// Recorded pairs of the bins b0 .. b1 - 1 of rc's histogram, compacted (by the
+// bin that counted them: a distance on a bin's edge, compared with the edge
+// instead, fell into the batch below, which is skipped where it counts none).
+cudaError_t launch_select_pairs(const ApRec& rc, uint64_t m, int b0, int b1, uint64_t* out,
+                                unsigned long long* count, cudaStream_t s);
 }  // namespace momenti

@@ -275,11 +275,7 @@ __device__ __forceinline__ void sw_record(const ApRec& rc, uint32_t a, uint32_t 
     rc.out[pos] = (uint64_t(a) << 32) | uint64_t(b);
     rc.out_d[pos] = dd;
   }
-  if (rc.hist) {
-    const float x = (dd - rc.lo) * rc.hscale;
-    const int bin = x < float(kApBins - 1) ? int(fmaxf(x, 0.f)) : kApBins - 1;
-    atomicAdd(&rc.hist[bin], 1u);
-  }
+  if (rc.hist) atomicAdd(&rc.hist[ap_bin(dd, rc.lo, rc.hscale)], 1u);
 }
 
 // Sorts N registers (a power of two) descending: bitonic network.

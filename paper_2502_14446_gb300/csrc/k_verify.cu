@@ -391,12 +391,13 @@ cudaError_t launch_verify_pairs(const Index& ix, int d, const uint64_t* pairs, i
 
 // Recorded pairs whose approximate distance lies in (lo, hi], compacted.
 __global__ void k_select_pairs(const uint64_t* __restrict__ pairs, const float* __restrict__ dd,
-                               uint64_t m, float lo, float hi, uint64_t* __restrict__ out,
+                               uint64_t m, float lo, float hscale, int b0, int b1, uint64_t* __restrict__ out,
                                unsigned long long* __restrict__ count) {
   const int lane = threadIdx.x & 31;
   for (uint64_t q0 = blockIdx.x * uint64_t(blockDim.x); q0 < m; q0 += uint64_t(gridDim.x) * blockDim.x) {
     const uint64_t q = q0 + threadIdx.x;
-    const bool keep = q < m && dd[q] > lo && dd[q] <= hi;
+    const int bin = q < m ? ap_bin(dd[q], lo, hscale) : -1;
+    const bool keep = bin >= b0 && bin < b1;
     const unsigned mask = __ballot_sync(0xffffffffu, keep);
     if (!mask) continue;
     unsigned long long base = 0;
@@ -406,12 +407,12 @@ __global__ void k_select_pairs(const uint64_t* __restrict__ pairs, const float* 
   }
 }
 
-cudaError_t launch_select_pairs(const uint64_t* pairs, const float* dd, uint64_t m, float lo,
-                                float hi, uint64_t* out, unsigned long long* count, cudaStream_t s) {
+cudaError_t launch_select_pairs(const ApRec& rc, uint64_t m, int b0, int b1, uint64_t* out,
+                                unsigned long long* count, cudaStream_t s) {
   if (m == 0) return cudaSuccess;
   uint64_t g = (m + 255) / 256;
   if (g > sm_count() * 8) g = sm_count() * 8;
-  MOMENTI_LAUNCH("select_pairs", s, k_select_pairs<<<unsigned(g), 256, 0, s>>>(pairs, dd, m, lo, hi, out, count));
+  MOMENTI_LAUNCH("select_pairs", s, k_select_pairs<<<unsigned(g), 256, 0, s>>>(rc.out, rc.out_d, m, rc.lo, rc.hscale, b0, b1, out, count));
   return cudaGetLastError();
 }
 

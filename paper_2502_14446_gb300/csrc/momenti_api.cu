@@ -872,11 +872,10 @@ int exact_path(momenti_handle* h, int d, double tau0, momenti_motif* out, int32_
       int b1 = b0;
       uint64_t run = 0;
       while (b1 < kApBins && (b1 == b0 || run + hist[b1] <= uint64_t(kBatch))) run += hist[b1++];
-      const float slo = b0 == 0 ? lo : float(double(lo) + width * b0);
       const float shi = b1 == kApBins ? hi : float(double(lo) + width * b1);
       if (run > 0) {
         CK(cudaMemsetAsync(dcnt, 0, 8, h->stream));
-        CK(launch_select_pairs(dout, dval, cnt, slo, shi, dsel, dcnt, h->stream));
+        CK(launch_select_pairs(ar, cnt, b0, b1, dsel, dcnt, h->stream));
         unsigned long long ns = 0;
         CK(cudaMemcpyAsync(&ns, dcnt, 8, cudaMemcpyDeviceToHost, h->stream));
         CK(cudaStreamSynchronize(h->stream));
