@@ -458,8 +458,8 @@ uint64_t momenti_launch_count(void);
  * proj_hash_fp32, proj_hash_tc, rehash, sort_init, sort_hist, sort_scan,
  * sort_scatter, sort_local, tensor_keys, chunk_scan, scan_top,
  * scan_add, collide, bucket_jobs, subbucket, subwarp, hs_clear,
- * verify_events, verify_pairs, sweep_cuts, sweep_table, allpairs, allpairs_sample,
- * allpairs_batch, select_pairs. */
+ * verify_events, verify_pairs, sweep_cuts, sweep_table, sweep_marked, allpairs,
+ * allpairs_sample, allpairs_batch, select_pairs. */
 int momenti_time_kernel(const char* name);
 
 /* Device time in milliseconds accumulated by the timed kernel since the

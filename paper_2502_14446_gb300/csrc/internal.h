@@ -289,12 +289,13 @@ __device__ __forceinline__ int ap_bin(float dd, float lo, float hscale) {
 // ---- k_sweep.cu ---------------------------------------------------------
 // The sweep's view of an index: its table (k_sweep.cu: df, dg and sigma per
 // window, in planes of transposed 64-window blocks, then 1/sigma), the series' points in the same
-// order, the cuts, and the window means and deviations.
+// order, the marks, and the window means and deviations.
 struct SweepView {
   const void* tab = nullptr;     // [Mpad / 64][3][64][G] vectors of 2 P dims, then [Mpad][G]
   const void* xp = nullptr;      // [npad][G]
   const void* xl = nullptr;      // [npad][G] low parts, float64 input only
-  const uint8_t* cut = nullptr;  // [Mpad] nonzero: at a cut, C of the recurrence starts anew after it
+  const uint8_t* cut = nullptr;  // [Mpad] bit 0: at a cut, C of the recurrence starts anew after it; bit 1: marked
+  const uint32_t* marked = nullptr;   // [0] how many windows are marked, then those windows, in any order
   const double* mu = nullptr;    // [D][M]
   const double* sig = nullptr;   // [D][M]
   int64_t M = 0, Mpad = 0, npad = 0;
@@ -321,8 +322,9 @@ cudaError_t launch_sweep_table(const Index& ix, void* buf, SweepView* out, cudaS
 // The recording sweep over all pairs of one series.
 cudaError_t launch_allpairs(const SweepView& v, int d, float thr, const ApRec& rc, cudaStream_t s);
 // The same over a spread sample of about `fraction` of the grid's blocks
-// (of seg rows each); *pairs = the pairs it holds, groups[2] (zeroed by the
-// caller) the groups of rows run, and those that took the slow branch.
+// (of seg rows each; the pairs of marked windows only where that is all of
+// them); *pairs = the pairs it holds, groups[2] (zeroed by the caller) the
+// groups of rows run, and those that took the slow branch.
 cudaError_t launch_allpairs_sample(const SweepView& v, int d, float thr, const ApRec& rc, double fraction,
                                    int seg, double* pairs, unsigned long long* groups, cudaStream_t s);
 // The recording sweeps of several series in one persistent launch on

@@ -46,9 +46,9 @@
 // took 35.6 ms; at D = 32, w = 500, n = 2e5, 137 against 848 ms.
 //
 // Windows that C cannot resolve (flat ones, and the 7 where the series falls
-// quiet: k_sweep_cuts) have sigma = NaN in the table: their tests give NaN,
-// whose sign bit is clear, so they always reach the slow branch, which
-// computes their pairs directly and starts C again after a cut.
+// quiet: k_sweep_cuts) are marked and listed when the table is built.  The
+// sweep leaves their pairs out; a kernel of its own computes them directly
+// (k_sweep_marked).
 #include "internal.h"
 
 #include <algorithm>
@@ -63,6 +63,7 @@ constexpr int kSwWarps = kSwThreads / 32;
 constexpr int kSwR = 8;                 // diagonals per lane
 constexpr int kSwPad = 2048;            // records after the last window / point
 constexpr int kSwSegMax = 2048;         // most rows between direct starts
+constexpr int kSwAtCut = 1, kSwMarked = 2;   // bits of a window's byte
 
 // P pairs of dims: 2 P floats of one kind, loaded with one instruction.
 template <int P>
@@ -132,7 +133,9 @@ size_t sw_smem(const SweepView& v) { return v.P == 2 ? sw_smem<2>(v.G) : sw_smem
 //     after the 8-row group in which a cut falls (walks reach e = 47, even
 //     noise 8: no cuts there);
 //   - the rest of such a group still has the old C, so a cut and the 6 windows
-//     after it have sigma = NaN and their pairs are computed directly.
+//     after it are marked.  Their sigma is NaN: a test against it gives NaN,
+//     whose sign bit is clear, so a group with a cut always reaches the slow
+//     branch, which knows the cut by its byte and sends the warp to a new start.
 // One warp per dimension and 256 windows (a warp's scan is serial: 2048 took
 // 90 us); the sum starts with that of the 2048 windows before, whatever cuts
 // lie there.  kappa goes where 1/sigma will lie.  With the table 0.12 ms at
@@ -189,11 +192,13 @@ __global__ void __launch_bounds__(128) k_sweep_cuts(Index ix, SweepView v, float
 // 1/sigma}, each computed in float64 and rounded once; per point the values
 // (and their low parts for float64 input).  A block
 // builds 64 windows and points: first the marks (flat in some dim, or at a
-// cut), then the records.
+// cut), which also go to a list, then the records.  A flat window that is not
+// at a cut has a sigma no correlation reaches, as the windows past the end.
 template <int P>
-__global__ void __launch_bounds__(256) k_sweep_table(Index ix, SweepView v, SwVec<P>* tab,
-                                                     SwVec<P>* __restrict__ xp, SwVec<P>* __restrict__ xl) {
-  __shared__ int mark[64];
+__global__ void __launch_bounds__(256) k_sweep_table(Index ix, SweepView v, SwVec<P>* tab, SwVec<P>* __restrict__ xp,
+                                                     SwVec<P>* __restrict__ xl, uint8_t* cut,
+                                                     uint32_t* __restrict__ marked) {
+  __shared__ int mark[64];                       // kSwAtCut, kSwMarked
   const int64_t B = int64_t(blockIdx.x) * 64;
   const int64_t M = ix.M, n = ix.n;
   if (threadIdx.x < 64) mark[threadIdx.x] = 0;
@@ -201,9 +206,22 @@ __global__ void __launch_bounds__(256) k_sweep_table(Index ix, SweepView v, SwVe
   for (int q = threadIdx.x; q < 64 * (ix.D + 1); q += 256) {
     const int c = q & 63, f = q >> 6;
     if (B + c >= M) continue;
-    if (f == ix.D ? v.cut[B + c] != 0 : ix.inv_sig[int64_t(f) * M + B + c] == 0.f) atomicOr(&mark[c], 1);
+    if (f == ix.D) {
+      if (cut[B + c]) atomicOr(&mark[c], kSwAtCut | kSwMarked);
+    } else if (ix.inv_sig[int64_t(f) * M + B + c] == 0.f) {
+      atomicOr(&mark[c], kSwMarked);
+    }
   }
   __syncthreads();
+  if (threadIdx.x < 64 && mark[threadIdx.x]) {   // (the first 64 threads: 2 warps)
+    const uint32_t act = __activemask();
+    const int lane = threadIdx.x & 31, lead = __ffs(act) - 1;
+    uint32_t at = 0;
+    if (lane == lead) at = atomicAdd(&marked[0], uint32_t(__popc(act)));
+    at = __shfl_sync(act, at, lead) + __popc(act & ((1u << lane) - 1u));
+    marked[1 + at] = uint32_t(B) + threadIdx.x;
+    cut[B + threadIdx.x] = uint8_t(mark[threadIdx.x]);
+  }
   const int G = v.G;
   const float* kap = reinterpret_cast<const float*>(tab + 3 * v.Mpad * G);   // replaced by 1/sigma below
   for (int q = threadIdx.x; q < 64 * G; q += 256) {
@@ -229,8 +247,8 @@ __global__ void __launch_bounds__(256) k_sweep_table(Index ix, SweepView v, SwVe
           }
           const double kappa = mark[c] ? 0.0 : double(kap[(sw_pos(b) * G + g) * (2 * P) + e]);
           const double sd = ix.sig[int64_t(f) * M + b] * (1.0 - kappa);
-          vs = mark[c] ? __int_as_float(0x7fc00000) : float(sd);
-          vi = mark[c] ? vs : float(1.0 / sd);
+          if (mark[c] & kSwAtCut) vs = vi = __int_as_float(0x7fc00000);
+          else if (!mark[c]) vs = float(sd), vi = float(1.0 / sd);
         }
         if (b < n) {
           vx = h[b];
@@ -339,44 +357,9 @@ __device__ __forceinline__ SwJoint sw_joint(const SweepJob* jb) {
   return j;
 }
 
-// The correlations of pair (a, b), computed directly by the warp into e:
-// z-normalised windows point by point, as the verification does.  They err
-// to the near side by two units in the last place of 1.
-template <int P>
-__device__ __forceinline__ void sw_direct_pair(const SweepView& v, uint32_t a, uint32_t b, float* e) {
-  const int lane = threadIdx.x & 31, w = v.w, stride = v.G * 2 * P;
-  const float* px = static_cast<const float*>(v.xp);
-  const float* pl = static_cast<const float*>(v.xl);
-#pragma unroll 1
-  for (int f = 0; f < v.D; ++f) {
-    const int64_t oa = int64_t(f) * v.M + a, ob = int64_t(f) * v.M + b;
-    const double ma = v.mu[oa], sa = v.sig[oa], mb = v.mu[ob], sb = v.sig[ob];
-    const float ha = float(ma), la = float(ma - double(ha)), hb = float(mb), lb = float(mb - double(hb));
-    const float ia = sa <= kFlatRel * (1.0 + fabs(ma)) ? 0.f : float(1.0 / sa);   // flat: the zero vector
-    const float ib = sb <= kFlatRel * (1.0 + fabs(mb)) ? 0.f : float(1.0 / sb);
-    float acc = 0.f;
-#pragma unroll 1
-    for (int t = lane; t < w; t += 32) {
-      const int64_t pa = sw_pos(int64_t(a) + t) * stride + f, pb = sw_pos(int64_t(b) + t) * stride + f;
-      float ua = -la, ub = -lb;
-      if (pl) {
-        ua += pl[pa];
-        ub += pl[pb];
-      }
-      const float dd = ((px[pa] - ha) + ua) * ia - ((px[pb] - hb) + ub) * ib;
-      acc = fmaf(dd, dd, acc);
-    }
-    for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-    if (lane == 0) e[f] = 1.f - acc / (2.f * float(w)) + 1.2e-7f;
-  }
-}
-
 // The queued hits of a warp, the last 32 at a time (all of them when
-// `all`), one per lane: pairs that exist and are not trivial get their
-// distance; the correlations of pairs with a window that has sigma = NaN are
-// computed directly first (7 windows per cut, and flat ones; taken as
-// candidates at distance 0, as they were, a quiet stretch's thousands of
-// pairs per window all went through the host).  Returns the number left.
+// `all`), one per lane: pairs that exist, are not trivial and hold no marked
+// window get their distance.  Returns the number left.
 template <int P>
 __device__ __noinline__ int sw_drain(const SweepJob* jb, float* queue, int qn, bool all) {
   const SweepView& v = jb->v;
@@ -393,15 +376,8 @@ __device__ __noinline__ int sw_drain(const SweepJob* jb, float* queue, int qn, b
     if (lane < n) {
       a = __float_as_uint(e[QS - 2]);
       b = __float_as_uint(e[QS - 1]);
-      pair = int64_t(b) < v.M && int64_t(b) - int64_t(a) > int64_t(v.excl);
+      pair = int64_t(b) < v.M && int64_t(b) - int64_t(a) > int64_t(v.excl) && !((v.cut[a] | v.cut[b]) & kSwMarked);
     }
-    uint32_t direct = __ballot_sync(0xffffffffu, pair && isnan(e[0]));
-    while (direct) {
-      const int q = __ffs(int(direct)) - 1;
-      direct &= direct - 1u;
-      sw_direct_pair<P>(v, __shfl_sync(0xffffffffu, a, q), __shfl_sync(0xffffffffu, b, q), queue + (qn + q) * QS);
-    }
-    __syncwarp();
     if (pair) {
       float sm = 0.f;
       if (D <= 8) sm = sw_dist<8>(e, D, d, wf);
@@ -653,7 +629,7 @@ __device__ __noinline__ int sw_redo(const SweepJob* jb, const SwVec<P>* rows, Sw
           y[p] = __ffma2_rn(__fmul2_rn(C[r][p], ib[h + r].v[p]), ia.v[p], nyl);
           part = __fadd2_rn(part, make_float2(fmaxf(y[p].x, 0.f), fmaxf(y[p].y, 0.f)));
         }
-        sum[r] = fmaf(0.f, y[0].x, part.x + part.y);             // NaN (an unresolvable window) stays NaN
+        sum[r] = part.x + part.y;                                // (a window at a cut: 0, no hit)
       }
       if (G == 2) {                                              // over the diagonal's lanes
 #pragma unroll
@@ -711,7 +687,8 @@ __device__ __noinline__ int sw_redo(const SweepJob* jb, const SwVec<P>* rows, Sw
     load(pn + (i2 + 1) * 8 * G, 7);
   }
   const unsigned long long* cuts = reinterpret_cast<const unsigned long long*>(jb->v.cut);
-  if (__any_sync(0xffffffffu, (cuts[a >> 3] | cuts[b >> 3] | cuts[(b >> 3) + 1]) != 0ull)) qn |= kSwCut;
+  if (__any_sync(0xffffffffu, ((cuts[a >> 3] | cuts[b >> 3] | cuts[(b >> 3) + 1]) & (kSwAtCut * 0x0101010101010101ull)) != 0ull))
+    qn |= kSwCut;
   return qn;
 }
 
@@ -896,6 +873,83 @@ k_sweep_batch(const SweepJob* __restrict__ jobs, const SweepItem* __restrict__ i
   }
 }
 
+// The pairs with a marked window: a marked window against 256 others per
+// turn, a pair per thread, point by point as the verification does (a pair of
+// two marked windows from the first).  Distances err to the near side by
+// 1e-5.  Bound by the FP32 lanes: about 8 operations per point and dim.  With
+// 2% of the windows of n = 3e4, D = 8 flat, an exact search takes 36 ms; 2.9 s
+// when a warp computed such a pair in the sweep's own queue, 2.4 s when they
+// were candidates at distance 0 (with 30% flat 0.30 s, 8.4 and 42).
+template <int P>
+__global__ void __launch_bounds__(256) k_sweep_marked(const __grid_constant__ SweepJob jb) {
+  extern __shared__ __align__(16) unsigned char sw_mem[];
+  float* dist = reinterpret_cast<float*>(sw_mem) + threadIdx.x;  // [D][256]
+  const SweepView& v = jb.v;
+  const uint32_t n = v.marked[0];
+  const int64_t M = v.M, ny = (M + 255) / 256, items = int64_t(n) * ny;
+  const int G = v.G, D = v.D, w = v.w;
+  const SwVec<P>* px = static_cast<const SwVec<P>*>(v.xp);
+  const SwVec<P>* pl = static_cast<const SwVec<P>*>(v.xl);
+  for (int64_t it = blockIdx.x; it < items; it += gridDim.x) {
+    const int64_t x = v.marked[1 + it / ny], y = (it % ny) * 256 + threadIdx.x;
+    const int64_t a = min(x, y), b = max(x, y);
+    if (y >= M || b - a <= int64_t(v.excl) || (y < x && (v.cut[y] & kSwMarked))) continue;
+#pragma unroll 1
+    for (int g = 0; g < G; ++g) {
+      float2 ma[P], la[P], ia[P], mb[P], lb[P], ib[P], acc[P];
+      auto stats = [&](int64_t q, float2 (&hi)[P], float2 (&lo)[P], float2 (&is)[P]) {
+#pragma unroll
+        for (int k = 0; k < 2 * P; ++k) {
+          const int f = 2 * P * g + k;
+          const int64_t o = int64_t(f) * M + q;
+          const double m = f < D ? v.mu[o] : 0.0, sd = f < D ? v.sig[o] : 0.0;
+          const float h = float(m), l = float(m - double(h));
+          const float r = sd <= kFlatRel * (1.0 + fabs(m)) ? 0.f : float(1.0 / sd);   // flat: the zero vector
+          if (k & 1) hi[k / 2].y = -h, lo[k / 2].y = -l, is[k / 2].y = r;
+          else hi[k / 2].x = -h, lo[k / 2].x = -l, is[k / 2].x = r;
+        }
+      };
+      stats(a, ma, la, ia);
+      stats(b, mb, lb, ib);
+#pragma unroll
+      for (int p = 0; p < P; ++p) acc[p] = make_float2(0.f, 0.f);
+#pragma unroll 4
+      for (int t = 0; t < w; ++t) {
+        const int64_t pa = sw_pos(a + t) * G + g, pb = sw_pos(b + t) * G + g;
+        const SwVec<P> xa = px[pa], xb = px[pb];
+#pragma unroll
+        for (int p = 0; p < P; ++p) {
+          const float2 ua = pl ? __fadd2_rn(pl[pa].v[p], la[p]) : la[p], ub = pl ? __fadd2_rn(pl[pb].v[p], lb[p]) : lb[p];
+          const float2 za = __fmul2_rn(__fadd2_rn(__fadd2_rn(xa.v[p], ma[p]), ua), ia[p]);
+          const float2 zb = __fmul2_rn(__fadd2_rn(__fadd2_rn(xb.v[p], mb[p]), ub), ib[p]);
+          const float2 d = __fadd2_rn(za, make_float2(-zb.x, -zb.y));
+          acc[p] = __ffma2_rn(d, d, acc[p]);
+        }
+      }
+#pragma unroll
+      for (int k = 0; k < 2 * P; ++k) {
+        const int f = 2 * P * g + k;
+        if (f < D) dist[256 * f] = sqrtf((k & 1) ? acc[k / 2].y : acc[k / 2].x) * 0.99999f;
+      }
+    }
+    float sm = 0.f;                                              // the d smallest
+    for (int q = 0; q < jb.d && sm <= jb.thr; ++q) {
+      float best = INFINITY;
+      int at = 0;
+      for (int f = 0; f < D; ++f) {
+        const float c = dist[256 * f];
+        if (c < best) {
+          best = c;
+          at = f;
+        }
+      }
+      dist[256 * at] = INFINITY;
+      sm += best;
+    }
+    if (sm <= jb.thr && sm > jb.rc.lo) sw_record(jb.rc, uint32_t(a), uint32_t(b), sm);
+  }
+}
+
 int64_t sw_diags(int G) { return int64_t(kSwWarps) * (32 / G) * kSwR; }   // per block
 
 // Diagonal blocks of the whole sweep (0: no non-trivial pair).
@@ -938,7 +992,7 @@ size_t sweep_table_bytes(const Index& ix) {
   const int P = sw_pairs(ix.D);
   const size_t G = size_t((ix.D + 2 * P - 1) / (2 * P));
   return (size_t(sw_round(ix.M)) * 4 + size_t(sw_round(ix.n)) * (ix.has_lo ? 2 : 1)) * G * (8 * size_t(P)) +
-         size_t(sw_round(ix.M));
+         size_t(sw_round(ix.M)) * 5 + 16;
 }
 
 template <int P>
@@ -951,11 +1005,13 @@ static cudaError_t sweep_table(const Index& ix, SweepView& v, void* buf, cudaStr
   v.xl = xl;
   uint8_t* cut = reinterpret_cast<uint8_t*>(xp + v.npad * v.G * (ix.has_lo ? 2 : 1));
   v.cut = cut;
-  const cudaError_t e = cudaMemsetAsync(cut, 0, size_t(v.Mpad), s);
+  uint32_t* marked = reinterpret_cast<uint32_t*>(cut + v.Mpad);      // (Mpad: a multiple of 64)
+  v.marked = marked;
+  const cudaError_t e = cudaMemsetAsync(cut, 0, size_t(v.Mpad) + 4, s);
   if (e != cudaSuccess) return e;
   const dim3 gc{unsigned((ix.M + 4 * kSwCutRun - 1) / (4 * kSwCutRun)), unsigned(ix.D), 1u};
   MOMENTI_LAUNCH("sweep_cuts", s, k_sweep_cuts<P><<<gc, 128, 0, s>>>(ix, v, reinterpret_cast<float*>(tab + v.Mpad * v.G * 3), cut));
-  MOMENTI_LAUNCH("sweep_table", s, k_sweep_table<P><<<unsigned(v.npad / 64), 256, 0, s>>>(ix, v, tab, xp, xl));
+  MOMENTI_LAUNCH("sweep_table", s, k_sweep_table<P><<<unsigned(v.npad / 64), 256, 0, s>>>(ix, v, tab, xp, xl, cut, marked));
   return cudaGetLastError();
 }
 
@@ -974,6 +1030,16 @@ cudaError_t launch_sweep_table(const Index& ix, void* buf, SweepView* out, cudaS
   const cudaError_t e = v.P == 2 ? sweep_table<2>(ix, v, buf, s) : sweep_table<1>(ix, v, buf, s);
   *out = v;
   return e;
+}
+
+template <int P>
+static cudaError_t sweep_marked(const SweepJob& jb, cudaStream_t s) {
+  const size_t smem = size_t(jb.v.D) * 256 * sizeof(float);
+  const cudaError_t e = allow_smem(reinterpret_cast<const void*>(k_sweep_marked<P>), smem);
+  if (e != cudaSuccess) return e;
+  // (as many blocks as stay resident; they find the marked windows' number on the device)
+  MOMENTI_LAUNCH("sweep_marked", s, k_sweep_marked<P><<<unsigned(sm_count() * 3), 256, smem, s>>>(jb));
+  return cudaGetLastError();
 }
 
 template <int P, int GT>
@@ -1000,18 +1066,21 @@ cudaError_t launch_allpairs(const SweepView& v, int d, float thr, const ApRec& r
   // offsets of the lanes' groups as constants where D is common (n = 1e5, w =
   // 300: 6.8 ms against 8.6 at D = 5, 14.4 against 17.8 at D = 16, 29.9 against
   // 37.7 at D = 32); D = 25 to 28 and 33 to 60 take the runtime form
-  if (v.P == 1) return v.G == 1 ? sweep<1, 1>(jb, gy, s) : sweep<1, 3>(jb, gy, s);
-  switch (v.G) {
-    case 1: return sweep<2, 1>(jb, gy, s);
-    case 2: return sweep<2, 2>(jb, gy, s);
-    case 3: return sweep<2, 3>(jb, gy, s);
-    case 4: return sweep<2, 4>(jb, gy, s);
-    case 5: return sweep<2, 5>(jb, gy, s);
-    case 6: return sweep<2, 6>(jb, gy, s);
-    case 8: return sweep<2, 8>(jb, gy, s);
-    case 16: return sweep<2, 16>(jb, gy, s);
-    default: return sweep<2, 0>(jb, gy, s);
+  cudaError_t e = cudaSuccess;
+  if (v.P == 1) e = v.G == 1 ? sweep<1, 1>(jb, gy, s) : sweep<1, 3>(jb, gy, s);
+  else switch (v.G) {
+    case 1: e = sweep<2, 1>(jb, gy, s); break;
+    case 2: e = sweep<2, 2>(jb, gy, s); break;
+    case 3: e = sweep<2, 3>(jb, gy, s); break;
+    case 4: e = sweep<2, 4>(jb, gy, s); break;
+    case 5: e = sweep<2, 5>(jb, gy, s); break;
+    case 6: e = sweep<2, 6>(jb, gy, s); break;
+    case 8: e = sweep<2, 8>(jb, gy, s); break;
+    case 16: e = sweep<2, 16>(jb, gy, s); break;
+    default: e = sweep<2, 0>(jb, gy, s);
   }
+  if (e != cudaSuccess) return e;
+  return v.P == 2 ? sweep_marked<2>(jb, s) : sweep_marked<1>(jb, s);
 }
 
 template <int P>
@@ -1050,7 +1119,9 @@ cudaError_t launch_allpairs_sample(const SweepView& v, int d, float thr, const A
       *pairs += double(c) * double(std::max<int64_t>(0, std::min<int64_t>(seg, v.M - (dl + c / 2) - a0)));
     }
   }
-  return v.P == 2 ? sweep_sample<2>(jb, nbx, blocks, stride, s) : sweep_sample<1>(jb, nbx, blocks, stride, s);
+  const cudaError_t e = v.P == 2 ? sweep_sample<2>(jb, nbx, blocks, stride, s) : sweep_sample<1>(jb, nbx, blocks, stride, s);
+  if (e != cudaSuccess || stride > 1) return e;
+  return v.P == 2 ? sweep_marked<2>(jb, s) : sweep_marked<1>(jb, s);
 }
 
 template <int P>
@@ -1099,6 +1170,8 @@ cudaError_t launch_allpairs_batch(std::vector<SweepJob> jobs, cudaStream_t s) {
   if (e == cudaSuccess) e = cudaMemcpyAsync(djobs, jobs.data(), jobs.size() * sizeof(SweepJob), cudaMemcpyHostToDevice, s);
   if (e == cudaSuccess) e = sweep_batch<1>(djobs, items[0], smem[0], s);
   if (e == cudaSuccess) e = sweep_batch<2>(djobs, items[1], smem[1], s);
+  for (size_t q = 0; q < jobs.size() && e == cudaSuccess; ++q)
+    if (sw_gy(jobs[q].v) > 0) e = jobs[q].v.P == 2 ? sweep_marked<2>(jobs[q], s) : sweep_marked<1>(jobs[q], s);
   if (djobs) cudaFreeAsync(djobs, s);
   return e;
 }
