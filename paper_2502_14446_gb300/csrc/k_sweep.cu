@@ -40,7 +40,7 @@
 // of 64 windows transposed (8 x 8), so that they are consecutive.
 //
 // What bounds it (D = 8, w = 300, 5e9 pairs, edge below the background):
-// 7.2 ms, 5.6 pair-dimensions per cycle and scheduler of the 10.7 that three
+// 7.0 ms, 4.5 pair-dimensions per cycle and scheduler of the 10.7 that three
 // FMA on the FP32 lanes allow; 8 warps per SM, fixed-latency dependencies
 // first.  The form before, one diagonal per lane sliding centred products,
 // took 35.6 ms; at D = 32, w = 500, n = 2e5, 137 against 848 ms.
@@ -93,8 +93,8 @@ __host__ __device__ __forceinline__ int64_t sw_off(int64_t b) {
 // Pairs of dims per lane for a series of D dims.  Two pairs read half the
 // instructions per pair-dimension; one pair wastes at most one dimension
 // instead of three, which pays at D = 1, 2, 5, 6 (a sweep of n = 1e5, w =
-// 300: 6.8 ms at D = 5, with two pairs as at D = 8 7.2; 2.2 at D = 1, with
-// two as at D = 4 3.9).
+// 300: 6.3 ms at D = 5, with two pairs as at D = 8 7.0; 2.1 at D = 1, with
+// two as at D = 4 4.4).
 int sw_pairs(int D) { return D <= 2 || D == 5 || D == 6 ? 1 : 2; }
 int64_t sw_round(int64_t m) { return ((m + 63) & ~int64_t(63)) + 64 + kSwPad; }
 
@@ -705,12 +705,12 @@ __device__ __forceinline__ void sw_block(const SweepJob* jb, int64_t bx, int64_t
   const int LPW = 32 / G;
   const SwLane L = sw_lane(G);
   const int g = L.g;
-  const int64_t a0 = bx * jb->seg;
+  const int a0 = int(bx * jb->seg);    // rows and columns in 32 bits (fewer than 2^27 windows): 7.0 ms against 7.4 at D = 8, n = 1e5
   const int64_t dlo = ((int64_t(v.excl) + 1) & ~int64_t(7)) + by * (kSwWarps * LPW * kSwR);
   const int64_t dfirst = max(dlo, int64_t(v.excl) + 1);          // the block's first diagonal
   if (dfirst >= M || a0 >= M - dfirst) return;                   // block-uniform
   const int nrow = int(min(int64_t(jb->seg), M - dfirst - a0));
-  const int64_t b0 = a0 + dlo + int64_t(warp * LPW + L.ld) * kSwR; // this lane's first column, a multiple of 8
+  const int b0 = int(a0 + dlo) + (warp * LPW + L.ld) * kSwR;     // this lane's first column, a multiple of 8
   const int RS = sw_rows<P>(G);
   SwVec<P>* rows = reinterpret_cast<SwVec<P>*>(sw_mem);                // [2][RS][3][G]
   SwVec<P>* ck = rows + 2 * RS * G * 3 + warp * (2 * kSwR * 32); // [warps][2][8][32]: C at an 8-row group's start
