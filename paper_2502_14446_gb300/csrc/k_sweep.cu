@@ -43,7 +43,7 @@
 // 7.0 ms, 4.5 pair-dimensions per cycle and scheduler of the 10.7 that three
 // FMA on the FP32 lanes allow; 8 warps per SM, fixed-latency dependencies
 // first.  The form before, one diagonal per lane sliding centred products,
-// took 35.6 ms; at D = 32, w = 500, n = 2e5, 137 against 848 ms.
+// took 35.6 ms; at D = 32, w = 500, n = 2e5, 136 against 848 ms.
 //
 // Windows that C cannot resolve (flat ones, and the 7 where the series falls
 // quiet: k_sweep_cuts) are marked and listed when the table is built.  The
@@ -965,7 +965,7 @@ int64_t sw_gy(const SweepView& v) {
 // three blocks per SM at a time.  Long blocks where there are many of them,
 // shorter ones where waves would be partly empty.  At most 2048: the error of
 // C grows with the root of the rows (blocks of 4096 took 128 ms where this
-// takes 137, n = 2e5, D = 32, w = 500, at 1.4 times the error).
+// takes 136, n = 2e5, D = 32, w = 500, at 1.4 times the error).
 int sw_seg(const SweepView& v) {
   const int64_t slots = int64_t(sm_count()) * (v.P == 2 ? kSwBlocks<2> : kSwBlocks<1>), nd = sw_diags(v.G), gy = sw_gy(v);
   int best = kSwSegMax;
@@ -1064,8 +1064,8 @@ cudaError_t launch_allpairs(const SweepView& v, int d, float thr, const ApRec& r
   jb.d = d;
   jb.seg = sw_seg(v);
   // offsets of the lanes' groups as constants where D is common (n = 1e5, w =
-  // 300: 6.8 ms against 8.6 at D = 5, 14.4 against 17.8 at D = 16, 29.9 against
-  // 37.7 at D = 32); D = 25 to 28 and 33 to 60 take the runtime form
+  // 300: 6.3 ms against 8.3 at D = 5, 14.0 against 16.8 at D = 16, 30.3 against
+  // 36.2 at D = 32); D = 25 to 28 (36.3 at 27) and 33 to 60 take the runtime form
   cudaError_t e = cudaSuccess;
   if (v.P == 1) e = v.G == 1 ? sweep<1, 1>(jb, gy, s) : sweep<1, 3>(jb, gy, s);
   else switch (v.G) {
